@@ -170,11 +170,14 @@ typedef struct {
   int64_t n_eff;        /* non-vacant orbitals of the last realisation               */
   int32_t grid, block;  /* launch shape of the sweep kernel                           */
   double step_seconds;  /* device time of the recursion-step launches alone          */
-  int64_t step_launches;/* number of recursion-step launches timed in step_seconds   */
+  int64_t step_launches;/* number of recursion-step launches timed in step_seconds (the
+                           on-chip sweep of mid-size lattices counts its recursion steps)  */
   double step_bytes;    /* algorithmic bytes of those launches                       */
   double gemm_seconds;  /* 2D moments: device time of the tensor-core contraction    */
   double gemm_flops;    /* 2D moments: tensor flops of the contraction (4 BF16 products) */
-  int32_t ring_stages;  /* step kernel: shared-memory ring depth used (autotuned)       */
+  int32_t ring_stages;  /* step kernel: shared-memory ring depth used (autotuned; the
+                           on-chip sweep of mid-size lattices: that of the streaming launch
+                           whose moment grouping it keeps)                                 */
   int32_t ctas_per_sm;  /* step kernel: resident CTAs per SM used (autotuned)           */
   int32_t steps_per_pass; /* step kernel: recursion steps fused per pass over the iterates
                              (1, or 2 with temporal blocking; autotuned; all of them when
@@ -191,11 +194,12 @@ typedef struct kite_ctx kite_ctx;
  * moments differ only by the regrouping of FP32 partial sums, except where noted (the
  * cluster sweep reports the vanishing imaginary part as 0; KITE_GEMM_PRODUCTS=3).
  *   KITE_AUTOTUNE=0       no timing of launch shapes: 8-stage rings at full occupancy, one
- *                         recursion step per launch, no cluster sweep
+ *                         recursion step per launch, no on-chip sweep
  *   KITE_TUNE=SxK[x2|x3]  pins the 1D sweep's ring depth S, CTAs per SM K and steps per pass
  *   KITE_PASS_STEPS=1|2|3 pins the steps per pass (1D and batched sweeps; 3: 1D only)
  *   KITE_CLUSTER=0|1      forbids / forces the on-chip cluster sweep of small lattices
  *                         (KITE_CLUSTER_CTAS=2..16 pins its CTAs per cluster)
+ *   KITE_RESIDENT=0|1     forbids / forces the on-chip sweep of mid-size lattices
  *   KITE_FAM_STREAMS=1    the 2D path's two vector families in sequence on one stream
  *   KITE_FAM_CPS=K        CTAs per SM of the 2D family steps
  *   KITE_GEMM_PRODUCTS=3  drops the lo x lo product of the split-BF16 contraction
@@ -250,6 +254,12 @@ int kite_flux_nearest(const kite_system* sys, double flux, double* out);
  * measures it faster, st->cluster_ctas reports it, and the imaginary part of each
  * moment, which vanishes for a real symmetric H~, is then not formed and reads 0.
  * KITE_CLUSTER=0 / 1 in the environment forbids / forces it.
+ * A mid-size lattice (two iterates of a batch of vectors fit the GPU's shared memory: up
+ * to about a million orbitals) may run the sweep on chip as well, one region of the
+ * lattice per SM in one cooperative launch whose CTAs wait on their neighbours within a
+ * bound; it keeps the streaming launch's grouping of the FP32 moment sums.  Chosen where
+ * measured faster; KITE_RESIDENT=0 / 1 forbids / forces it.  If a wait runs out (its SMs held
+ * by another long kernel), the call runs the streaming kernels instead.
  *   mu          [M] FP64, real part of the average, host or device (required)
  *   mu_per_vec  [S*R][M] complex FP64 interleaved (re, im) per vector, or NULL
  *   st          statistics, or NULL

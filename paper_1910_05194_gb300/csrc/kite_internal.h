@@ -12,6 +12,16 @@
 
 #include "kite_gb.h"
 
+namespace kite {
+// How the resident sweep cuts a lattice over the SMs (kite_resident.cu).
+struct ResidentPlan {
+  int TX, G;          // strip width, virtual CTAs: how the moment sums are grouped
+  int regions, rows, nv, nfl, r0_rows;
+  int CR;             // 16-byte chunks per orbital and sweep (0: the lattice does not fit)
+  int T, levels, smem;
+};
+}  // namespace kite
+
 struct kite_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -41,6 +51,8 @@ struct kite_ctx {
   // Autotuner cache: key (kernel family, precision, lattice, vectors per orbital, mode,
   // size bucket) -> (ring depth, CTAs per SM) measured fastest on this context's GPU.
   std::map<uint64_t, std::pair<int, int>> tune;
+  // Plans of the resident sweep's free grouping (pure functions of the sizes), a few kept.
+  std::map<std::vector<int>, kite::ResidentPlan> resident_plans;
 };
 
 namespace kite {
@@ -142,6 +154,40 @@ size_t cluster_part_doubles(int lanes, int cs, int M, int doubling, int timing_s
 // timing_steps > 0: a timing run of that many steps, nothing stored; 0: the whole sweep,
 // then the moments into mu_vec.
 int cluster_sweep(kite_ctx* ctx, ClusterSweep* a, int timing_steps);
+
+// The 1D sweep of a mid-size lattice held on chip by the whole GPU, a region of the lattice
+// per SM (kite_resident.cu).
+ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, int realv, int field, int Lx, int Ly,
+                           int C, int M, int TX, long long G);
+ResidentPlan resident_plan_free(kite_ctx* ctx, int lattice, int doubling, int realv, int field, int Lx, int Ly, int C,
+                                int M);
+int resident_max_chunks(kite_ctx* ctx, int lattice, int Lx, int Ly, int C);
+// Bytes of the edge records the regions exchange, and (at most) of the moment partials.
+size_t resident_rec_bytes(int lattice, int Lx, int Ly, int CR);
+size_t resident_part_bytes(kite_ctx* ctx, int fp64, int realv, int C, int slots);
+struct ResidentSweep {
+  ResidentPlan plan;
+  int fp64, lattice, doubling, realv;
+  int Lx, Ly, M;
+  int C;        // chunks per orbital of the batch
+  int nvec, vec_base;
+  int open_x, open_y, stall, want_last;
+  const void* r0;
+  const void* vt;
+  const void* phase;  // Peierls phases, or null without a field
+  double tt;
+  void *bA, *bB;      // odd and even iterates: the last two when wanted
+  double* part;
+  void* rec;          // edge records, resident_rec_bytes
+  const unsigned long long* n_eff;
+  double* mu_vec;
+  // outputs
+  double seconds, bytes;
+  int grid, block;
+};
+// timing_steps > 0: a timing run of that many steps of the first chunks; 0: the whole sweep,
+// then the moments into mu_vec (with doubling, before the undoubling).
+int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps);
 
 // AdamW step coefficients of the learned reconstructor's training (kite_mlp.cu).
 struct AdamwCoeffs {

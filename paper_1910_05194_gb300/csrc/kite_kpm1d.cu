@@ -712,10 +712,54 @@ int cluster_choice(kite_ctx* ctx, const Plan& p, const ClusterSweep& c, long lon
   return pick;
 }
 
+// ---- mid-size lattices: the whole sweep on chip, a region per SM (kite_resident.cu) ------
+// KITE_RESIDENT=0 never takes it and KITE_RESIDENT=1 takes it whenever the lattice fits;
+// unset, it is a candidate of the autotuner and runs where it is measured faster per
+// recursion step than the kernels it would replace.
+inline int resident_pinned() {  // 0 unset, 1 off, 2 on
+  const char* e = getenv("KITE_RESIDENT");
+  return (e && (e[0] == '0' || e[0] == '1') && e[1] == 0) ? e[0] - '0' + 1 : 0;
+}
+// Moment partials of the resident sweep are kept for every step; beyond this the streaming
+// kernels run.
+constexpr size_t kResidentPartMax = (size_t)2 << 30;
+
+// Whether to run the batch resident.  `other_ms` times the kernels chosen otherwise, per
+// recursion step of the batch.
+template <typename OtherMs>
+bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, int per_chunk, OtherMs other_ms) {
+  if (resident_pinned() == 2) return true;
+  uint64_t key = 0x6b697465726573ull;
+  for (uint64_t f : {(uint64_t)r.fp64, (uint64_t)r.lattice, (uint64_t)r.doubling, (uint64_t)r.realv,
+                     (uint64_t)r.nvec, (uint64_t)r.C, (uint64_t)r.Lx, (uint64_t)r.Ly, (uint64_t)r.open_x,
+                     (uint64_t)r.open_y, (uint64_t)(r.phase != nullptr)})
+    key = (key ^ f) * 0x100000001b3ull;
+  key = (key | 1ull << 63) & ~(1ull << 62);
+  auto it = ctx->tune.find(key);
+  if (it != ctx->tune.end()) return it->second.first != 0;
+  // two timing runs, so that the launch and load cost drops out; the best of two each
+  auto timed = [&](int steps) {
+    double best = 1e30;
+    for (int k = 0; k < 2; ++k) {
+      ResidentSweep t = r;
+      if (resident_sweep(ctx, &t, steps) != KITE_OK) return 1e30;
+      best = std::min(best, t.seconds);
+    }
+    return best;
+  };
+  const double t8 = timed(8), t40 = timed(kClusterTimeSteps);
+  const int sweeps = ((r.nvec + per_chunk - 1) / per_chunk + r.plan.CR - 1) / r.plan.CR;
+  const float ms = (float)(1e3 * std::max(0.0, t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
+  const int pick = ms < 0.95f * other_ms() ? 1 : 0;  // it must win clearly
+  cudaGetLastError();
+  ctx->tune[key] = {pick, 0};
+  return pick != 0;
+}
+
 template <typename Real, int LAT>
 int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const Scale& sc,
               double* mu_dev, double* imag_dev, double* mu_vec_dev_ext, kite_stats* stats,
-              const double* r0_dev_all) {
+              const double* r0_dev_all, bool* resident_used, bool allow_resident) {
   constexpr int SORB = (LAT == KITE_HONEYCOMB) ? 2 : 1;
   constexpr int VPC = Chunk<Real>::kVecs;
   constexpr int kMaxC = 4;
@@ -769,8 +813,33 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       (p.field || cluster_pinned() == 1)
           ? 0
           : cluster_part_doubles(p.realv ? p.max_batch : 2 * p.max_batch, 16, p.M, p.doubling, kClusterTimeSteps);
+  // the resident sweep's moment partials and edge records, where the lattice may fit on chip
+  size_t resident_part = 0, resident_rec = 0;
+  if (allow_resident && resident_pinned() != 1 && p.M >= 4) {
+    const int cr = resident_max_chunks(ctx, LAT, p.Lx, p.Ly, Cmax);
+    if (cr >= 1) {
+      resident_part = resident_part_bytes(ctx, sizeof(Real) == 8, p.realv, cr, std::max(p.M + 1, 2 * kClusterTimeSteps + 2));
+      resident_rec = resident_rec_bytes(LAT, p.Lx, p.Ly, cr);
+    }
+    if (resident_part > kResidentPartMax) resident_part = resident_rec = 0;
+  }
+  // FP32 moment sums keep the grouping of the streaming launch (strips of TX cells, grid G);
+  // FP64 sums may be grouped freely
+  auto resident_for = [&](int C, int G) {
+    if (resident_rec == 0) return ResidentPlan{};
+    if (sizeof(Real) == 4)
+      return resident_plan(ctx, 0, LAT, p.doubling, p.realv, p.field, p.Lx, p.Ly, C, p.M, kBlock / (SORB * C), G);
+    const std::vector<int> key{LAT, p.doubling, p.realv, p.field, p.Lx, p.Ly, C, p.M >= 4};
+    auto it = ctx->resident_plans.find(key);
+    if (it != ctx->resident_plans.end()) return it->second;
+    if (ctx->resident_plans.size() >= 64) ctx->resident_plans.clear();
+    return ctx->resident_plans[key] =
+               resident_plan_free(ctx, LAT, p.doubling, p.realv, p.field, p.Lx, p.Ly, C, p.M);
+  };
+  char* res_rec = nullptr;
   auto plan_ws = [&](Carver& k, Real** vt, void** r0, void** bA, void** bB, void** bC, void** bD,
                      double** partial, unsigned long long** ne, double** mu_vec, Real** phase) {
+    res_rec = k.take<char>(resident_rec);
     *vt = k.take<Real>(p.N);
     *phase = p.field ? k.take<Real>((size_t)p.Ly * SORB * 4) : nullptr;
     *r0 = k.take<char>(vec_bytes);
@@ -778,7 +847,8 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
     *bB = k.take<char>(vec_bytes);
     *bC = two_possible ? k.take<char>(vec_bytes) : nullptr;
     *bD = two_possible ? k.take<char>(vec_bytes) : nullptr;
-    *partial = k.take<double>(std::max((size_t)(std::max(p.M, 2) + 1) * Gmax * 2 * Cmax * VPC, cluster_part));
+    *partial = k.take<double>(std::max({(size_t)(std::max(p.M, 2) + 1) * Gmax * 2 * Cmax * VPC, cluster_part,
+                                        resident_part / sizeof(double) + 1}));
     *ne = k.take<unsigned long long>(1);
     *mu_vec = k.take<double>(nvec_total * p.M * 2);
   };
@@ -808,7 +878,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
   int64_t n_eff_last = 0;
   int grid_used = 0;
   Tune tune_used{kStages, 0};
-  int cluster_used = 0, steps_used = 0;
+  int cluster_used = 0, steps_used = 0, block_used = kBlock;
   double step_s = 0.0, step_bytes = 0.0;
   int64_t step_n = 0;
   KITE_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
@@ -931,11 +1001,140 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
         return C == 1 ? one(std::integral_constant<int, 1>{})
                       : (C == 2 ? one(std::integral_constant<int, 2>{}) : one(std::integral_constant<int, 4>{}));
       };
+      FieldSweep fs{};  // magnetic field: the one-step sweep with Peierls phases (kite_field.cu)
+      const int field_occ = p.field ? field_occupancy(sizeof(Real) == 8, LAT, C, p.doubling) : 0;
+      if (p.field) {
+        fs.fp64 = sizeof(Real) == 8;
+        fs.lattice = LAT;
+        fs.C = C;
+        fs.doubling = p.doubling;
+        fs.Lx = p.Lx;
+        fs.Ly = p.Ly;
+        fs.M = p.M;
+        fs.units = u;
+        fs.G = (int)std::max(1LL, std::min({(long long)ctx->num_sms * field_occ, u, (long long)Gmax}));
+        fs.zero = p.open.zero;
+        fs.open_x = p.open.x;
+        fs.open_y = p.open.y;
+        fs.ncell = p.ncell;
+        fs.N = p.N;
+        fs.vt = vt;
+        fs.tt = (double)tt;
+        fs.r0 = r0;
+        fs.bA = bA;
+        fs.bB = bB;
+        fs.partial = partial;
+        fs.phase = phase;
+      }
+      ResidentSweep rs{};
+      rs.fp64 = sizeof(Real) == 8;
+      rs.lattice = LAT;
+      rs.doubling = p.doubling;
+      rs.realv = p.realv;
+      rs.Lx = p.Lx;
+      rs.Ly = p.Ly;
+      rs.M = p.M;
+      rs.C = C;
+      rs.nvec = nvec;
+      rs.vec_base = vec_base;
+      rs.open_x = p.open.x;
+      rs.open_y = p.open.y;
+      rs.r0 = r0;
+      rs.vt = vt;
+      rs.phase = phase;
+      rs.tt = (double)tt;
+      rs.bA = bA;
+      rs.bB = bB;
+      rs.part = partial;
+      rs.rec = res_rec;
+      rs.n_eff = ne;
+      rs.mu_vec = mu_vec;
+      // grid of the streaming launch of a tuned shape
+      auto tuned_grid = [&]() -> int {
+        auto one = [&](auto cc) -> int {
+          constexpr int CC = decltype(cc)::value;
+          auto mode = [&](auto mm) -> int {
+            constexpr int MODE = decltype(mm)::value;
+            constexpr bool DB = MODE == 3;
+            const Tune t = autotune<Real, LAT, CC, MODE>(ctx, u, p, vt, tt, r0, bA, bB, bC, bD, partial);
+            tune_used = t;
+            if (t.two == 1)
+              return t.nst == 5   ? step2_grid<Real, LAT, CC, 5, DB>(ctx, u, t.k)
+                     : t.nst == 6 ? step2_grid<Real, LAT, CC, 6, DB>(ctx, u, t.k)
+                                  : step2_grid<Real, LAT, CC, 8, DB>(ctx, u, t.k);
+            return t.nst == 4 ? grid_for<Real, LAT, CC, false, MODE, 4>(ctx, u, t.k)
+                              : grid_for<Real, LAT, CC, false, MODE, 8>(ctx, u, t.k);
+          };
+          return p.doubling ? mode(std::integral_constant<int, 3>{}) : mode(std::integral_constant<int, 0>{});
+        };
+        return C == 1 ? one(std::integral_constant<int, 1>{})
+                      : (C == 2 ? one(std::integral_constant<int, 2>{}) : one(std::integral_constant<int, 4>{}));
+      };
+      // the kernels that run otherwise, per recursion step: the cluster sweep, the field
+      // sweep, or the streaming kernel of the tuned shape
+      auto other_ms = [&]() -> float {
+        if (cl.cs > 0) return cluster_step_ms(ctx, cl);
+        if (p.field) {
+          FieldSweep f = fs;
+          f.M = std::min(p.M, 33);
+          if (field_sweep(ctx, &f) != KITE_OK || field_sweep(ctx, &f) != KITE_OK || f.launches < 1) return 1e30f;
+          return (float)(1e3 * f.seconds / (double)f.launches);
+        }
+        auto one = [&](auto cc) -> float {
+          constexpr int CC = decltype(cc)::value;
+          auto mode = [&](auto mm) -> float {
+            constexpr int MODE = decltype(mm)::value;
+            constexpr bool DB = MODE == 3;
+            const Tune t = autotune<Real, LAT, CC, MODE>(ctx, u, p, vt, tt, r0, bA, bB, bC, bD, partial);
+            tune_used = t;
+            if (t.two == 1)
+              return t.nst == 5 ? time_candidate2<Real, LAT, CC, 5, DB>(ctx, t.k, u, p, vt, tt, r0, bA, bB, bC, bD, partial)
+                     : t.nst == 6
+                         ? time_candidate2<Real, LAT, CC, 6, DB>(ctx, t.k, u, p, vt, tt, r0, bA, bB, bC, bD, partial)
+                         : time_candidate2<Real, LAT, CC, 8, DB>(ctx, t.k, u, p, vt, tt, r0, bA, bB, bC, bD, partial);
+            return t.nst == 4 ? time_candidate<Real, LAT, CC, MODE, 4>(ctx, t.k, u, p, vt, tt, r0, bA, bB, partial)
+                              : time_candidate<Real, LAT, CC, MODE, 8>(ctx, t.k, u, p, vt, tt, r0, bA, bB, partial);
+          };
+          return p.doubling ? mode(std::integral_constant<int, 3>{}) : mode(std::integral_constant<int, 0>{});
+        };
+        return C == 1 ? one(std::integral_constant<int, 1>{})
+                      : (C == 2 ? one(std::integral_constant<int, 2>{}) : one(std::integral_constant<int, 4>{}));
+      };
       const bool want_last = kpm->r_last && !p.doubling;
+      rs.want_last = want_last;
       cl.last_prev = want_last ? bA : nullptr;
       cl.last_cur = want_last ? bB : nullptr;
       cl.cs = cluster_choice(ctx, p, cl, u, stream_ms);
-      if (cl.cs > 0) {
+      // (an FP32 batch that runs on chip in clusters stays there: its moment sums are grouped
+      // by the clusters' threads)
+      const bool pinned_res = resident_pinned() == 2;
+      const bool may_reside = resident_rec != 0 && (pinned_res || (!ctx->debug_stall && autotune_enabled() &&
+                                                                   !pass_steps_pinned() && !getenv("KITE_TUNE") &&
+                                                                   cluster_pinned() != 2));
+      if (may_reside && (sizeof(Real) == 8 || cl.cs == 0 || pinned_res))
+        rs.plan = resident_for(C, sizeof(Real) == 8 ? 0 : (p.field ? fs.G : tuned_grid()));
+      if (rs.plan.CR && resident_choice(ctx, rs, per_chunk, other_ms)) {
+        // mid-size lattice: the whole sweep on chip, a region per SM (kite_resident.cu)
+        rs.stall = ctx->debug_stall;
+        ctx->debug_stall = 0;
+        *resident_used = true;
+        rc = resident_sweep(ctx, &rs, 0);
+        if (rc != KITE_OK) return rc;
+        if (p.doubling) {
+          k_undouble<<<(nvec * p.M + 255) / 256, 256, 0, st>>>(mu_vec, p.M, nvec, vec_base);
+          KITE_CUDA_TRY(ctx, cudaGetLastError());
+        }
+        step_s += rs.seconds;
+        step_n += steps_for(p);  // recursion steps: each sweep is one launch of all of them
+        step_bytes += rs.bytes;
+        grid_used = rs.grid;
+        block_used = rs.block;
+        // (FP32: the streaming shape whose moment grouping was kept)
+        if (sizeof(Real) == 8 || p.field) tune_used = Tune{kStages, 1, 0};
+        tune_used.two = 0;
+        lc = ((p.M - 1) & 1) ? bA : bB;
+        lp = ((p.M - 1) & 1) ? bB : bA;
+      } else if (cl.cs > 0) {
         // small lattice: the whole sweep on chip (kite_cluster.cu)
         rc = cluster_sweep(ctx, &cl, 0);
         if (rc != KITE_OK) return rc;
@@ -949,31 +1148,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
         lp = bA;
         lc = bB;
       } else if (p.field) {
-        // magnetic field: the one-step sweep with Peierls phases (kite_field.cu)
-        const int occ = field_occupancy(sizeof(Real) == 8, LAT, C, p.doubling);
-        FieldSweep fs{};
-        fs.fp64 = sizeof(Real) == 8;
-        fs.lattice = LAT;
-        fs.C = C;
-        fs.doubling = p.doubling;
-        fs.Lx = p.Lx;
-        fs.Ly = p.Ly;
-        fs.M = p.M;
-        fs.units = u;
-        fs.G = (int)std::max(1LL, std::min({(long long)ctx->num_sms * occ, u, (long long)Gmax}));
         fs.stall = ctx->debug_stall;
-        fs.zero = p.open.zero;
-        fs.open_x = p.open.x;
-        fs.open_y = p.open.y;
-        fs.ncell = p.ncell;
-        fs.N = p.N;
-        fs.vt = vt;
-        fs.tt = (double)tt;
-        fs.r0 = r0;
-        fs.bA = bA;
-        fs.bB = bB;
-        fs.partial = partial;
-        fs.phase = phase;
         ctx->debug_stall = 0;
         rc = field_sweep(ctx, &fs);
         if (rc != KITE_OK) return rc;
@@ -988,7 +1163,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
         step_n += fs.launches;
         step_bytes += fs.bytes;
         grid_used = fs.G;
-        tune_used = Tune{8, occ, 0};
+        tune_used = Tune{8, field_occ, 0};
       } else if (C == 1) KITE_SWEEP(1);
       else if (C == 2) KITE_SWEEP(2);
       else KITE_SWEEP(4);
@@ -1060,7 +1235,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
     stats->gbps = stats->seconds > 0 ? stats->bytes_moved / stats->seconds * 1e-9 : 0.0;
     stats->n_eff = n_eff_last;
     stats->grid = grid_used;
-    stats->block = kBlock;
+    stats->block = block_used;
     stats->ring_stages = tune_used.nst;
     stats->steps_per_pass = cluster_used ? steps_used : tune_used.two + 1;
     stats->cluster_ctas = cluster_used;
@@ -1078,11 +1253,24 @@ int moments_1d_impl(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
                     double* mu_dev, double* imag_dev, double* mu_vec_dev, kite_stats* st,
                     const double* r0_dev_all) {
   const bool fp64 = kpm->precision == KITE_FP64;
-  if (sys->lattice == KITE_HONEYCOMB)
-    return fp64 ? run_typed<double, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all)
-                : run_typed<float, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all);
-  return fp64 ? run_typed<double, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all)
-              : run_typed<float, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all);
+  bool resident = false;
+  const bool stalled = ctx->debug_stall != 0;
+  auto run = [&](bool allow_resident) {
+    if (sys->lattice == KITE_HONEYCOMB)
+      return fp64 ? run_typed<double, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
+                                                      &resident, allow_resident)
+                  : run_typed<float, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
+                                                     &resident, allow_resident);
+    return fp64 ? run_typed<double, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
+                                                 &resident, allow_resident)
+                : run_typed<float, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
+                                                &resident, allow_resident);
+  };
+  int rc = run(true);
+  // A neighbour that never came up within the bounded wait (another long kernel holding its
+  // SM): the streaming kernels, whose CTAs do not wait on one another, take the call.
+  if (rc == KITE_ERR_TIMEOUT && resident && !stalled) rc = run(false);
+  return rc;
 }
 
 }  // namespace kite

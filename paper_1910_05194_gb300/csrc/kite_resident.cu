@@ -1,0 +1,828 @@
+// kite_resident.cu -- the 1D moment sweep of a mid-size lattice held on chip by the whole
+// GPU: one cooperative launch runs every recursion step of a batch (Eqs. e6-e8).
+//
+// The lattice is cut as the streaming kernels cut it: strips of TX cells, row segments as
+// work units in strip order, and a range of units per (virtual) CTA of the streaming grid.
+// One SM owns the units of a few consecutive virtual CTAs, its region: a block of rows of
+// one strip, or the end of one strip and the beginning of the next.  It keeps r_n and
+// r_{n-1} of the region in shared memory, each with a frame of one halo cell, and the
+// on-site terms beside them; r_0 as far as it fits, the rest of it is read from L2.  r_{n+1}
+// overwrites r_{n-1} in place.
+//
+// Per step the compute threads (one per column of a virtual CTA, sublattice and 16-byte
+// chunk) march down their rows with the next row's operands in flight, while 256 exchange
+// threads (1) compute the region's edge sites once more, with their r_{n-1} in registers, and
+// send them at once, (2) add up the moment partials of the step before, (3) receive the
+// neighbours' edge sites into the frame.  The exchange's latency thus lies beside the march.  No grid-wide barrier and no fence: a
+// 16-byte chunk travels as four 8-byte words of 32 data bits and the 32-bit step number, so a
+// word that carries the step's number carries its data (8-byte accesses are single copies).
+// The records are double-buffered by step parity: a region sends r_{n+1} only after it has
+// received all of its neighbours' r_n, which they sent after they had received r_{n-1}, so
+// the record that r_{n+1} overwrites has been read.  (A flag per region behind a release
+// fence, with the halo read after an acquire, took 9.5 us per step whatever the size.)
+//
+// Results: the site update is the streaming kernels' rounding sequence, so the iterates are
+// the same bits; and each FP32 moment sum runs over the same sites in the same order as in
+// the streaming launch it stands in for (a virtual CTA's rows of one column, promoted to
+// FP64 every kRFlush rows), so the moments agree with that launch's to the rounding of FP64
+// sums.  As there, the FP32 sweeps form the imaginary part too and the FP64 sweeps do not.
+//
+// What bounds it: the march, by shared-memory wavefronts and issue slots (five 16-byte loads
+// and a store per chunk), with the exchange (1.4-1.7 us: edge sites, one flight through L2, a
+// poll) beside it.  Per recursion step of the batch, against the streaming kernels' launch,
+// ring fill and CTA reduction per step: honeycomb 257 x 510, R = 8 FP32 14.6 -> 5.0 us (two
+// sweeps of four vectors), 512 x 601 in a field, R = 4 17.4 -> 5.9 us, 300 x 300, R = 8
+// 11.4 -> 3.8 us; 64 x 64, R = 4 FP64 1.6-1.9 us against the cluster sweep's 2.2 us.  Which
+// runs is measured (resident_choice in kite_kpm1d.cu).
+#include <math.h>
+
+#include <algorithm>
+#include <mutex>
+#include <set>
+#include <utility>
+
+#include "kite_device.cuh"
+#include "kite_internal.h"
+
+namespace kite {
+namespace {
+
+constexpr int kRMax = 256;     // most compute threads of a CTA (512 threads: 128 registers each)
+constexpr int kRComm = 256;    // exchange threads
+constexpr int kRSites = 2;     // most edge sites, and most halo chunks, of one exchange thread
+constexpr int kRMaxV = 64;     // most virtual CTAs of a region
+constexpr int kRFlush = 32;    // rows of one FP32 moment sum (the streaming kernels' kFlushRows)
+constexpr int kResSmem = 227 * 1024 - 512;  // (the rest: static shared memory)
+
+// One record: 16 bytes of data as four 8-byte words of (data, step number), moved by one
+// 32-byte access.
+struct alignas(32) Rec {
+  unsigned long long w[4];
+};
+__device__ __forceinline__ void send_rec(Rec* p, const uint4& d, uint32_t step) {
+  const unsigned long long h = (unsigned long long)step << 32;
+  asm volatile("st.relaxed.gpu.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(h | d.x), "l"(h | d.y),
+               "l"(h | d.z), "l"(h | d.w)
+               : "memory");
+}
+__device__ __forceinline__ Rec load_rec(const Rec* p) {
+  Rec r;
+  asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(r.w[0]), "=l"(r.w[1]), "=l"(r.w[2]), "=l"(r.w[3])
+               : "l"(p)
+               : "memory");
+  return r;
+}
+__device__ __forceinline__ bool rec_ready(const Rec& r, uint32_t step) {
+  return (uint32_t)(r.w[0] >> 32) == step && (uint32_t)(r.w[1] >> 32) == step && (uint32_t)(r.w[2] >> 32) == step &&
+         (uint32_t)(r.w[3] >> 32) == step;
+}
+
+template <typename Real>
+struct ResArgs {
+  const void* r0;     // batch layout [cell][sublattice][C chunks]
+  const Real* vt;     // 2 V~ per orbital, NaN on vacancies
+  const Real* phase;  // [Ly][sublattice][2][2] (cos, sin), field only
+  void* last[2];      // r_last: the last two iterates in the batch layout, r_n in last[n & 1]
+  double* part;       // moment partials [slot n][CTA][exchange warps][32 >> levels]
+  Rec* rec;           // edge records [parity][cell][sublattice][CR chunks]
+  int* err;
+  Real tt;
+  int Lx, Ly, TX, G;  // strip width, virtual CTAs
+  int rows_max, nv_max, nfl, r0_rows, levels;
+  int C, c0, CR;      // chunks per orbital of the batch, first chunk and chunks of this sweep
+  int steps, open_x, open_y, stall;
+  int write_last;
+};
+
+// Shared-memory carve, the same on host and device: offsets in bytes.
+struct ResSmem {
+  int x0, x1, r0, vt, phase, sums, total;
+};
+__host__ __device__ inline ResSmem res_smem(int sorb, int CR, int TX, int rows, int nv, int nfl, int real_bytes,
+                                            int nsums, int dbl, int r0_rows, int field) {
+  ResSmem s;
+  const int cellb = sorb * CR * 16, frame = (rows + 4) * (TX + 2);
+  int off = 0;
+  auto take = [&](int bytes) {
+    const int at = off;
+    off += (bytes + 127) & ~127;
+    return at;
+  };
+  s.x0 = take(frame * cellb);
+  s.x1 = take(frame * cellb);
+  s.vt = take(rows * TX * sorb * real_bytes);
+  s.phase = take(field ? rows * sorb * 4 * real_bytes : 0);
+  s.sums = take((dbl ? 4 : 2) * nv * nfl * TX * sorb * CR * nsums * real_bytes);  // of two steps
+  s.r0 = take(r0_rows * TX * cellb);
+  s.total = off;
+  return s;
+}
+
+// VAR 0: complex vectors, 1: complex vectors in a magnetic field, 2: real vectors.
+template <typename Real, int LAT, bool DBL, int VAR>
+__global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Real> a) {
+  using Ch = Chunk<Real>;
+  constexpr int SORB = LAT == KITE_HONEYCOMB ? 2 : 1;
+  constexpr int NR = Ch::kReals, VPC = Ch::kVecs;
+  constexpr bool IM = sizeof(Real) == 4 && VAR != 2;          // real and imaginary parts
+  constexpr int NV = VAR == 2 ? NR : (IM ? 2 * VPC : VPC);    // moment sums per chunk
+  constexpr int SETS = DBL ? 2 : 1;        // <.|r_{n+1}>, and <r_n|r_n> with doubling
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int s_abort, s_vrow[kRMaxV + 1];  // first local row of each virtual CTA
+  const int T = (int)blockDim.x - kRComm;  // compute threads
+  const int tid = threadIdx.x, cta = blockIdx.x;
+  const int CR = a.CR, TPC = SORB * CR, TX = a.TX, colT = TX * TPC;
+  const ResSmem sm = res_smem(SORB, CR, TX, a.rows_max, a.nv_max, a.nfl, (int)sizeof(Real), NV, DBL, a.r0_rows,
+                              VAR == 1);
+  // r_n and r_{n-1} are kept by sublattice, [sublattice][framed cell][chunk]: a warp's lanes
+  // hold one sublattice of a row (where a row of TX * CR chunks fills whole warps)
+  const int P = TX + 2, CB = CR * 16, PB = P * CB;   // framed row; bytes of a cell, of a framed row
+  const int PS = (a.rows_max + 4) * PB;              // bytes of a sublattice
+  // the region: virtual CTAs v0 .. v1-1, units U0 .. U0+nrows-1, in one or two segments
+  const long long units = (long long)((a.Lx + TX - 1) / TX) * a.Ly;
+  const int v0 = (int)((long long)a.G * cta / gridDim.x), v1 = (int)((long long)a.G * (cta + 1) / gridDim.x);
+  const long long U0 = units * v0 / a.G;
+  const int nrows = (int)(units * v1 / a.G - U0);
+  const int sx = (int)(U0 / a.Ly), yb = (int)(U0 - (long long)sx * a.Ly);
+  const int nr0 = min(nrows, a.Ly - yb), nr1 = nrows - nr0;
+  // segment g: strip sx + g, first row (g ? 0 : yb), owned rows local 0 .. and frame row base
+  auto seg_tx = [&](int g) { return min(TX, a.Lx - (sx + g) * TX); };
+  auto row_y = [&](int r) { return r < nr0 ? yb + r : r - nr0; };
+  auto frame_row = [&](int r) { return r < nr0 ? r + 1 : r + 3; };
+  Real* vts = reinterpret_cast<Real*>(smem + sm.vt);
+  Real* phs = reinterpret_cast<Real*>(smem + sm.phase);
+  Real* sums = reinterpret_cast<Real*>(smem + sm.sums);  // [parity][set][(j, flush, column)][NV]
+  const int nsum = a.nv_max * a.nfl * colT * NV;          // of one set
+
+  auto wrap = [](int v, int L) { return v < 0 ? v + L : (v >= L ? v - L : v); };
+  // lattice cell of segment g's local (lx, ly), -1 across an open boundary
+  auto lattice_cell = [&](int g, int lx, int ly) -> int {
+    const int x = (sx + g) * TX + lx, y = (g ? 0 : yb) + ly;
+    if ((a.open_x && (x < 0 || x >= a.Lx)) || (a.open_y && (y < 0 || y >= a.Ly))) return -1;
+    return wrap(y, a.Ly) * a.Lx + wrap(x, a.Lx);
+  };
+  auto frame_cell = [&](int g, int lx, int ly) { return ((g ? nr0 + 2 : 0) + ly + 1) * P + lx + 1; };
+
+  for (int i = tid; i < nrows * TX * SORB; i += blockDim.x) {
+    const int r = i / (TX * SORB), k = i - r * TX * SORB, lx = k / SORB, s = k - lx * SORB;
+    const int g = r < nr0 ? 0 : 1;
+    if (lx < seg_tx(g))
+      vts[(s * a.rows_max + r) * TX + lx] = a.vt[((size_t)row_y(r) * a.Lx + (sx + g) * TX + lx) * SORB + s];
+  }
+  if (VAR == 1)
+    for (int i = tid; i < nrows * SORB * 4; i += blockDim.x) {
+      const int r = i / (SORB * 4);
+      phs[i] = a.phase[(size_t)row_y(r) * SORB * 4 + (i - r * SORB * 4)];
+    }
+  for (int i = tid; i < SETS * 2 * nsum; i += blockDim.x) sums[i] = Real(0);
+  if (tid == 0) s_abort = 0;
+  if (tid <= v1 - v0) s_vrow[tid] = (int)(units * (v0 + tid) / a.G - U0);
+  // r_0 with its frame; the other buffer starts at zero (open boundaries keep it so)
+  for (int g = 0; g < (nr1 ? 2 : 1); ++g) {
+    const int w = seg_tx(g) + 2, h = (g ? nr1 : nr0) + 2;
+    for (int i = tid; i < w * h * TPC; i += blockDim.x) {
+      const int f = i / TPC, k = i - f * TPC;
+      const int ly = f / w - 1, lx = f - (ly + 1) * w - 1;
+      const int s = k / CR, c = k - s * CR;
+      const int at = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+      const int q = lattice_cell(g, lx, ly);
+      Ch z, r;
+#pragma unroll
+      for (int e = 0; e < NR; ++e) z.v[e] = r.v[e] = Real(0);
+      if (q >= 0) r = Ch::ldg(a.r0, ((size_t)q * SORB + s) * a.C + a.c0 + c);
+      *reinterpret_cast<Ch*>(smem + sm.x0 + at) = r;
+      *reinterpret_cast<Ch*>(smem + sm.x1 + at) = z;
+      if (!DBL && lx >= 0 && lx < w - 2 && ly >= 0 && ly < h - 2) {
+        const int row = (g ? nr0 : 0) + ly;
+        if (row < a.r0_rows) reinterpret_cast<Ch*>(smem + sm.r0)[((s * a.r0_rows + row) * TX + lx) * CR + c] = r;
+      }
+    }
+  }
+  unsigned char* const xb = smem + sm.x0;
+  const int xd = sm.x1 - sm.x0;
+  const Real tt = a.tt, tt2 = a.tt + a.tt;
+
+  // byte offsets of the neighbours of a site of sublattice s from its own chunk
+  struct Nb {
+    int o1, o2, o3, o4;
+  };
+  auto offsets = [&](int s) {
+    Nb b;
+    if (LAT == KITE_HONEYCOMB) {
+      b.o1 = s == 0 ? PS : -PS;
+      b.o3 = b.o1 + (s == 0 ? -PB : PB);
+      b.o2 = b.o3 + (s == 0 ? CB : -CB);
+      b.o4 = 0;
+    } else {
+      b.o1 = -CB;
+      b.o2 = CB;
+      b.o3 = -PB;
+      b.o4 = PB;
+    }
+    return b;
+  };
+  auto ld = [](const unsigned char* p) { return *reinterpret_cast<const Ch*>(p); };
+  // the streaming kernels' site update; ph: the site's two bond rotations (field)
+  auto update = [&](auto first_tag, Ch n1, Ch n2, Ch n3, const Ch& n4, const Ch& me, const Ch& pv, Real v,
+                    const Real* ph) -> Ch {
+    constexpr bool FIRST = decltype(first_tag)::value;
+    if constexpr (VAR == 1) {
+      auto rot = [&](Ch& x, Real cph, Real sph) {
+#pragma unroll
+        for (int q = 0; q < VPC; ++q) {
+          const Real re = x.v[2 * q], im = x.v[2 * q + 1];
+          x.v[2 * q] = rfma(cph, re, -rmul(sph, im));
+          x.v[2 * q + 1] = rfma(sph, re, rmul(cph, im));
+        }
+      };
+      if (LAT == KITE_HONEYCOMB) {
+        rot(n2, ph[0], ph[1]);
+        rot(n3, ph[2], ph[3]);
+      } else {
+        rot(n1, ph[0], ph[1]);
+        rot(n2, ph[2], ph[3]);
+      }
+    }
+    const bool vacant = is_vacancy(v);
+    Ch out;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      Real sum = radd(n1.v[q], n2.v[q]);
+      sum = radd(sum, n3.v[q]);
+      if (LAT == KITE_SQUARE) sum = radd(sum, n4.v[q]);
+      const Real o = FIRST ? rfma(tt, sum, rmul(Real(0.5) * v, me.v[q])) : rfma(tt2, sum, rfma(v, me.v[q], -pv.v[q]));
+      out.v[q] = vacant ? Real(0) : o;
+    }
+    return out;
+  };
+  __syncthreads();
+
+  if (tid >= T) {  // ---- exchange threads
+    const int ct = tid - T, lane = ct & 31, warp = ct >> 5;
+    const size_t half = (size_t)a.Lx * a.Ly * TPC;  // records per parity
+    // edge sites (sent) and halo chunks (received) of this thread: smem offset, record
+    int e_off[kRSites], h_off[kRSites], e_row[kRSites];
+    unsigned e_rec[kRSites], h_rec[kRSites];
+    Real e_v[kRSites];
+    Ch e_prev[kRSites];
+    unsigned e_on = 0, h_on = 0, e_s = 0;
+    {
+      int off = 0, hoff = 0;  // list positions of the segment's first entry
+      for (int g = 0; g < (nr1 ? 2 : 1); ++g) {
+        const int w = seg_tx(g), h = g ? nr1 : nr0, base = g ? nr0 : 0;
+        // honeycomb: A along the first row and the last column, B along the last row and the
+        // first column; square: the four sides
+        const int len = LAT == KITE_HONEYCOMB ? 2 * (w + h - 1) : 2 * (w + h);
+#pragma unroll
+        for (int u = 0; u < kRSites; ++u) {
+          const int j = ct + u * kRComm, e = j / CR - off, c = j - (j / CR) * CR;
+          if (e < 0 || e >= len) continue;
+          int lx, ly, s = 0;
+          if (LAT == KITE_HONEYCOMB) {
+            const int hl = w + h - 1, k = e < hl ? e : e - hl;
+            s = e < hl ? 0 : 1;
+            if (s == 0) lx = k < w ? k : w - 1, ly = k < w ? 0 : k - w + 1;
+            else lx = k < w ? k : 0, ly = k < w ? h - 1 : k - w;
+          } else {
+            if (e < 2 * w) lx = e >> 1, ly = (e & 1) ? h - 1 : 0;
+            else lx = (e & 1) ? w - 1 : 0, ly = (e - 2 * w) >> 1;
+          }
+          e_on |= 1u << u;
+          e_s |= (unsigned)s << u;
+          e_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+          e_row[u] = base + ly;
+          e_v[u] = vts[(s * a.rows_max + base + ly) * TX + lx];
+          e_rec[u] = (unsigned)((lattice_cell(g, lx, ly) * SORB + s) * CR + c);
+        }
+        off += len;
+        const int hlen = 2 * (w + h);
+#pragma unroll
+        for (int u = 0; u < kRSites; ++u) {
+          const int j = ct + u * kRComm, e = j / CR - hoff, c = j - (j / CR) * CR;
+          if (e < 0 || e >= hlen) continue;
+          int lx, ly, s = 0;
+          if (LAT == KITE_HONEYCOMB) {
+            const int k = e < w + h ? e : e - (w + h);
+            if (e < w + h) {  // B above (and above right), then B right
+              s = 1;
+              lx = k <= w ? k : w;
+              ly = k <= w ? -1 : k - w - 1;
+            } else {  // A below (and below left), then A left
+              lx = k <= w ? k - 1 : -1;
+              ly = k <= w ? h : k - w;
+            }
+          } else {
+            if (e < 2 * w) lx = e >> 1, ly = (e & 1) ? h : -1;
+            else lx = (e & 1) ? w : -1, ly = (e - 2 * w) >> 1;
+          }
+          const int q = lattice_cell(g, lx, ly);
+          if (q < 0) continue;
+          h_on |= 1u << u;
+          h_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+          h_rec[u] = (unsigned)((q * SORB + s) * CR + c);
+        }
+        hoff += hlen;
+      }
+    }
+    const Nb nb0 = offsets(0), nb1 = offsets(1);
+    const bool mute = a.stall && cta == 0;
+    auto send_edges = [&](int n, auto first_tag) {
+      const unsigned char* cur = xb + (n & 1) * xd;
+      Rec* dst = a.rec + ((n + 1) & 1) * half;
+#pragma unroll
+      for (int u = 0; u < kRSites; ++u) {
+        if (!(e_on >> u & 1)) continue;
+        const Nb nb = (e_s >> u & 1) ? nb1 : nb0;
+        const unsigned char* p = cur + e_off[u];
+        const Ch me = ld(p);
+        Ch n4 = me;
+        if (LAT == KITE_SQUARE) n4 = ld(p + nb.o4);
+        const Ch out = update(first_tag, ld(p + nb.o1), ld(p + nb.o2), ld(p + nb.o3), n4, me, e_prev[u], e_v[u],
+                              phs + (e_row[u] * SORB + (int)(e_s >> u & 1)) * 4);
+        e_prev[u] = me;
+        if (!mute) send_rec(dst + e_rec[u], *reinterpret_cast<const uint4*>(&out), (uint32_t)(n + 1));
+      }
+    };
+    // FP64 sums of step n's partials: each thread every kRComm-th entry (its own (chunk, sum)
+    // class), then `levels` folds inside the warp
+    const int keep = 32 >> a.levels;
+    const size_t pstep = (size_t)gridDim.x * (kRComm / 32) * keep;
+    double* pp = a.part + ((size_t)cta * (kRComm / 32) + warp) * keep + lane;
+    auto add_sums = [&](int n) {  // (plain: n = -1 is <r_0|r_0>)
+      const Real* src = sums + (size_t)(n & 1) * SETS * nsum;
+#pragma unroll
+      for (int set = 0; set < SETS; ++set) {
+        double d = 0.0;
+        for (int e = ct; e < nsum; e += kRComm) d += (double)src[set * nsum + e];
+        for (int l = 0, o = 16; l < a.levels; ++l, o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane < keep) pp[(size_t)(DBL ? 2 * n + 1 - set : n + 1) * pstep] = d;
+      }
+    };
+    __syncthreads();  // <r_0|r_0> is in the sums of step -1
+    for (int n = 0; n < a.steps; ++n) {
+      bool ok = true;
+      if (n + 1 < a.steps) {
+        if (n == 0) send_edges(n, std::true_type{});
+        else send_edges(n, std::false_type{});
+      }
+      if (n > 0 || !DBL) add_sums(n - 1);
+      if (n + 1 < a.steps) {
+        const uint32_t step = (uint32_t)(n + 1);
+        unsigned char* nxt = xb + ((n + 1) & 1) * xd;
+        const Rec* src = a.rec + ((n + 1) & 1) * half;
+        unsigned want = h_on;
+        const long long t0 = clock64();
+        while (want) {
+          Rec d[kRSites];
+#pragma unroll
+          for (int u = 0; u < kRSites; ++u)
+            if (want >> u & 1) d[u] = load_rec(src + h_rec[u]);
+#pragma unroll
+          for (int u = 0; u < kRSites; ++u)
+            if ((want >> u & 1) && rec_ready(d[u], step)) {
+              *reinterpret_cast<uint4*>(nxt + h_off[u]) =
+                  make_uint4((uint32_t)d[u].w[0], (uint32_t)d[u].w[1], (uint32_t)d[u].w[2], (uint32_t)d[u].w[3]);
+              want &= ~(1u << u);
+            }
+          if (want && clock64() - t0 > kWaitCycles) {
+            ok = false;
+            break;
+          }
+        }
+      }
+      if (!ok) s_abort = 1;
+      __syncthreads();  // r_{n+1} complete in the region and its frame
+      if (s_abort) {
+        if (ct == 0) atomicExch(a.err, 1);
+        return;
+      }
+    }
+    add_sums(a.steps - 1);
+    return;
+  }
+
+  // ---- compute threads
+  const int col = tid % colT, s = col / (TX * CR), xc = col - s * TX * CR, xl = xc / CR, c = xc - xl * CR;
+  const int jstep = T / colT, jfirst = tid < jstep * colT ? tid / colT : v1 - v0;
+  const Nb nb = offsets(s);
+  const bool tx_on0 = xl < seg_tx(0), tx_on1 = nr1 && xl < seg_tx(1);
+  const size_t gstep = (size_t)a.Lx * SORB * a.C;
+
+  if constexpr (!DBL) {  // <r_0|r_0>, grouped as the other moments (real part)
+    Real* out_sums = sums + nsum;
+    for (int j = jfirst; j < v1 - v0; j += jstep) {
+      const int re = s_vrow[j + 1];
+      Real f[NV];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) f[q] = Real(0);
+      int rows = 0, fl = 0;
+      auto flush = [&]() {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+          out_sums[((size_t)(j * a.nfl + fl) * colT + col) * NV + q] = f[q];
+          f[q] = Real(0);
+        }
+        rows = 0;
+        ++fl;
+      };
+      for (int r = s_vrow[j]; r < re; ++r) {
+        if (!(r < nr0 ? tx_on0 : tx_on1)) continue;
+        const Ch me = ld(xb + s * PS + (frame_row(r) * P + xl + 1) * CB + c * 16);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+          const int v = IM ? q >> 1 : q;
+          if (VAR == 2) f[q] = rfma(me.v[q], me.v[q], f[q]);
+          else if (!IM || !(q & 1)) f[q] = rfma(me.v[2 * v + 1], me.v[2 * v + 1], rfma(me.v[2 * v], me.v[2 * v], f[q]));
+        }
+        if (++rows == kRFlush) flush();
+      }
+      if (rows) flush();
+    }
+  }
+  __syncthreads();
+
+  // rows [r, rend) of segment g in one column, S the sublattice (a template argument: the
+  // carried neighbour is the first or the third of the sum)
+  Real f0[NV], f1[NV];       // FP32 (FP64) sums since the last flush, over `rows` rows
+  int rows = 0;
+  Real* sum_at = nullptr;    // where the next flush goes
+  auto flush = [&]() {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      sum_at[q] = f0[q];
+      if (DBL) sum_at[(SETS - 1) * nsum + q] = f1[q];
+      f0[q] = f1[q] = Real(0);
+    }
+    rows = 0;
+    sum_at += colT * NV;
+  };
+  auto march = [&](auto first_tag, auto s_tag, const unsigned char* cur, unsigned char* nxt, int g, int r, int rend) {
+    constexpr bool FIRST = decltype(first_tag)::value;
+    constexpr int S = decltype(s_tag)::value;
+    int at = s * PS + (frame_row(r) * P + xl + 1) * CB + c * 16;
+    const Real* pv_v = vts + (s * a.rows_max + r) * TX + xl;
+    const Ch* pr = reinterpret_cast<const Ch*>(smem + sm.r0) + ((s * a.r0_rows + r) * TX + xl) * CR + c;
+    size_t gq = (((size_t)row_y(r) * a.Lx + (sx + g) * TX + xl) * SORB + s) * a.C + a.c0 + c;
+    const Real* ph = phs + (r * SORB + s) * 4;
+    // honeycomb: B(x,y-1) for A, A(x,y) for B; square: the upper and the own value
+    Ch up, mid;
+    if (LAT == KITE_HONEYCOMB) up = ld(cur + at + (S == 0 ? nb.o3 : nb.o1));
+    else up = ld(cur + at + nb.o3), mid = ld(cur + at);
+    auto row = [&](Ch na, Ch nbv, Ch nc, const Ch& pv, Ch z0, Real v, int at_, const Real* ph_) {
+      Ch n1, n2, n3, n4, me;
+      if (LAT == KITE_HONEYCOMB) {  // na: B(x,y) for A, A(x,y+1) for B
+        n1 = S == 0 ? na : up;
+        n3 = S == 0 ? up : na;
+        up = na;
+        n2 = nbv;
+        me = n4 = nc;
+      } else {  // left, right, below
+        n1 = na;
+        n2 = nbv;
+        n3 = up;
+        me = mid;
+        n4 = nc;
+        up = mid;
+        mid = nc;
+      }
+      const Ch out = update(first_tag, n1, n2, n3, n4, me, pv, v, ph_);
+      *reinterpret_cast<Ch*>(nxt + at_) = out;
+      const Ch& l = (DBL || FIRST) ? me : z0;  // the bra: <r_n| with doubling, else <r_0|
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        if (VAR == 2) {
+          f0[q] = rfma(l.v[q], out.v[q], f0[q]);
+          if (DBL) f1[q] = rfma(l.v[q], l.v[q], f1[q]);
+        } else {
+          const int w = IM ? q >> 1 : q;  // conj(bra) ket, as in the streaming kernels' cacc
+          const Real br = l.v[2 * w], bi = l.v[2 * w + 1], kr = out.v[2 * w], ki = out.v[2 * w + 1];
+          if (!IM || !(q & 1)) {
+            f0[q] = rfma(bi, ki, rfma(br, kr, f0[q]));
+            if (DBL) f1[q] = rfma(bi, bi, rfma(br, br, f1[q]));
+          } else {
+            f0[q] = rfma(-bi, kr, rfma(br, ki, f0[q]));
+          }
+        }
+      }
+      if (++rows == kRFlush) flush();
+    };
+    auto oa = (LAT == KITE_HONEYCOMB && S == 1) ? nb.o3 : nb.o1;
+    auto oc = LAT == KITE_HONEYCOMB ? 0 : nb.o4;
+    // two rows' operands in flight; the rows whose r_0 is off chip apart (their loads take an
+    // L2 round trip)
+    auto run = [&](const int end, const bool on_chip) {
+      for (; r + 1 < end; r += 2) {
+        const unsigned char *p = cur + at, *p1 = p + PB;
+        const Ch a0 = ld(p + oa), b0 = ld(p + nb.o2), c0_ = ld(p + oc), a1 = ld(p1 + oa), b1 = ld(p1 + nb.o2),
+                 c1 = ld(p1 + oc);
+        Ch q0, q1;
+        if (!FIRST) q0 = ld(nxt + at), q1 = ld(nxt + at + PB);
+        Ch z0, z1;
+        if (!FIRST && !DBL) {
+          z0 = on_chip ? pr[0] : Ch::ldg(a.r0, gq);
+          z1 = on_chip ? pr[TX * CR] : Ch::ldg(a.r0, gq + gstep);
+        }
+        const Real va = pv_v[0], vb = pv_v[TX];
+        row(a0, b0, c0_, q0, z0, va, at, ph);
+        row(a1, b1, c1, q1, z1, vb, at + PB, ph + SORB * 4);
+        at += 2 * PB;
+        pv_v += 2 * TX;
+        pr += 2 * TX * CR;
+        gq += 2 * gstep;
+        ph += 2 * SORB * 4;
+      }
+      if (r < end) {
+        const unsigned char* p = cur + at;
+        Ch q0, z0;
+        if (!FIRST) q0 = ld(nxt + at);
+        if (!FIRST && !DBL) z0 = on_chip ? pr[0] : Ch::ldg(a.r0, gq);
+        row(ld(p + oa), ld(p + nb.o2), ld(p + oc), q0, z0, *pv_v, at, ph);
+        ++r;
+        at += PB;
+        pv_v += TX;
+        pr += TX * CR;
+        gq += gstep;
+        ph += SORB * 4;
+      }
+    };
+    if (FIRST || DBL) {
+      run(rend, true);
+    } else {
+      if (r < a.r0_rows) run(min(rend, a.r0_rows), true);
+      if (r < rend) run(rend, false);
+    }
+  };
+  auto run_step = [&](int n, auto first_tag) {
+    const unsigned char* cur = xb + (n & 1) * xd;
+    unsigned char* nxt = xb + ((n + 1) & 1) * xd;
+    Real* out_sums = sums + (size_t)(n & 1) * SETS * nsum;
+    for (int j = jfirst; j < v1 - v0; j += jstep) {
+      const int r = s_vrow[j], re = s_vrow[j + 1];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) f0[q] = f1[q] = Real(0);
+      rows = 0;
+      sum_at = out_sums + ((size_t)j * a.nfl * colT + col) * NV;
+      // the virtual CTA's rows of segment 0, then of segment 1
+      for (int g = 0; g < 2; ++g) {
+        const int ra = g ? max(r, nr0) : r, rb = g ? re : min(re, nr0);
+        if (ra >= rb || !(g ? tx_on1 : tx_on0)) continue;
+        if (SORB == 1 || s == 0)
+          march(first_tag, std::integral_constant<int, 0>{}, cur, nxt, g, ra, rb);
+        else
+          march(first_tag, std::integral_constant<int, 1>{}, cur, nxt, g, ra, rb);
+      }
+      if (rows) flush();
+    }
+  };
+  run_step(0, std::true_type{});
+  __syncthreads();
+  for (int n = 1; n < a.steps; ++n) {
+    if (s_abort) return;
+    run_step(n, std::false_type{});
+    __syncthreads();
+  }
+  if (a.write_last && !s_abort) {  // r_{steps-1} and r_steps
+    for (int i = tid; i < nrows * colT; i += T) {
+      const int r = i / colT, kk = i - r * colT, ss = kk / (TX * CR), lx = (kk - ss * TX * CR) / CR, q = kk % CR;
+      const int g = r < nr0 ? 0 : 1;
+      if (lx >= seg_tx(g)) continue;
+      const int at = ss * PS + (frame_row(r) * P + lx + 1) * CB + q * 16;
+      const size_t o = (((size_t)row_y(r) * a.Lx + (sx + g) * TX + lx) * SORB + ss) * a.C + a.c0 + q;
+      for (int b = 0; b < 2; ++b) ld(xb + b * xd + at).st(a.last[b], o);
+    }
+  }
+}
+
+// mu_vec[vec_base + vector][n]: the sum of slot n's partials in a fixed order (a class of
+// entries per thread, then a tree), over N_eff.  One block per moment; entry e belongs to the
+// lane e % lanes of the sweep: a vector, or its real and imaginary part (im).
+__global__ void __launch_bounds__(256) k_resident_reduce(const double* __restrict__ part, int M, int count, int lanes,
+                                                         int im, int nvec, int vec_base,
+                                                         const unsigned long long* __restrict__ n_eff,
+                                                         double* __restrict__ mu_vec) {
+  const int n = blockIdx.x;
+  const double* p = part + (size_t)n * count;
+  double s = 0.0;
+  for (int e = threadIdx.x; e < count; e += 256) s += p[e];  // 256 is a multiple of lanes
+  __shared__ double red[256];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int st = 128; st >= lanes; st >>= 1) {
+    if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+    __syncthreads();
+  }
+  const int l = (int)threadIdx.x, v = im ? l >> 1 : l;
+  if (l < lanes && v < nvec) {
+    const double ne = (double)*n_eff;
+    double* out = mu_vec + ((size_t)(vec_base + v) * M + n) * 2;
+    out[im ? l & 1 : 0] = ne > 0.0 ? red[l] / ne : 0.0;
+    if (!im) out[1] = 0.0;
+  }
+}
+
+template <typename Real, int LAT, bool DBL>
+const void* res_kernel_var(int var) {
+  return var == 0   ? reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 0>)
+         : var == 1 ? reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 1>)
+                    : reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 2>);
+}
+template <typename Real>
+const void* res_kernel(int lattice, int dbl, int var) {
+  if (lattice == KITE_HONEYCOMB)
+    return dbl ? res_kernel_var<Real, KITE_HONEYCOMB, true>(var) : res_kernel_var<Real, KITE_HONEYCOMB, false>(var);
+  return dbl ? res_kernel_var<Real, KITE_SQUARE, true>(var) : res_kernel_var<Real, KITE_SQUARE, false>(var);
+}
+
+int per_chunk_of(int fp64, int realv) { return fp64 ? (realv ? 2 : 1) : (realv ? 4 : 2); }  // vectors
+int sums_of(int fp64, int realv) { return fp64 ? (realv ? 2 : 1) : 4; }                      // moment sums
+
+}  // namespace
+
+// The regions for strips of TX cells and G virtual CTAs, and the chunks per sweep: as many as
+// fit on chip (fewer sweeps), with as many rows of r_0 as fit beside them.  CR = 0: no fit.
+ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, int realv, int field, int Lx, int Ly,
+                           int C, int M, int TX, long long G) {
+  ResidentPlan p{};
+  const int sorb = lattice == KITE_HONEYCOMB ? 2 : 1, real = fp64 ? 8 : 4;
+  const int nstrips = (Lx + TX - 1) / TX;
+  const long long units = (long long)nstrips * Ly;
+  // (records are indexed in 32 bits)
+  if (Lx < 3 || Ly < 3 || M < 4 || G < 1 || G > units || (double)Lx * Ly * sorb * C > 4e8) return p;
+  const int regions = (int)std::min<long long>(ctx->num_sms, G);
+  int rows = 0, nv = 0, edge = 0;
+  const int vrows = (int)((units + G - 1) / G);
+  for (int i = 0; i < regions; ++i) {
+    const long long v0 = G * i / regions, v1 = G * (i + 1) / regions, u0 = units * v0 / G, u1 = units * v1 / G;
+    if (u1 - u0 > Ly) return p;  // more than two segments
+    rows = std::max(rows, (int)(u1 - u0));
+    nv = std::max(nv, (int)(v1 - v0));
+    const bool two = u0 / Ly != (u1 - 1) / Ly;
+    edge = std::max(edge, 2 * ((int)(u1 - u0) + (two ? 2 : 1) * TX));
+  }
+  if (nv > kRMaxV) return ResidentPlan{};
+  p.nfl = (vrows + kRFlush - 1) / kRFlush;
+  for (int cr = C; cr >= 1; cr >>= 1) {
+    const int colT = TX * sorb * cr;
+    if (colT > kRMax || edge * cr > kRSites * kRComm) continue;
+    const int per = sums_of(fp64, realv);
+    auto need = [&](int r0_rows) {
+      return res_smem(sorb, cr, TX, rows, nv, p.nfl, real, per, doubling, r0_rows, field).total;
+    };
+    if (need(0) > kResSmem) continue;
+    int r0_rows = doubling ? 0 : rows;
+    while (r0_rows > 0 && need(r0_rows) > kResSmem) --r0_rows;
+    p.regions = regions;
+    p.TX = TX;
+    p.G = (int)G;
+    p.rows = rows;
+    p.nv = nv;
+    p.r0_rows = r0_rows;
+    p.CR = cr;
+    p.T = std::min(nv, kRMax / colT) * colT;
+    p.T = (p.T + 31) / 32 * 32;
+    p.smem = need(r0_rows);
+    int lv = 0;
+    while ((32 >> (lv + 1)) >= cr * per && (!fp64 || lv < 2)) ++lv;
+    p.levels = lv;
+    return p;
+  }
+  return p;
+}
+
+// Whether any sweep of the lattice could fit, and the most chunks of one (for the work space).
+int resident_max_chunks(kite_ctx* ctx, int lattice, int Lx, int Ly, int C) {
+  const double orb = (double)Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1);
+  int cr = C;
+  while (cr >= 1 && orb * cr * 32.0 > (double)ctx->num_sms * kResSmem) cr >>= 1;
+  return cr;
+}
+
+// FP64 sums may be grouped freely: strips and virtual CTAs that give every SM a compact
+// region and its threads one column of few rows each.
+ResidentPlan resident_plan_free(kite_ctx* ctx, int lattice, int doubling, int realv, int field, int Lx, int Ly, int C,
+                                int M) {
+  ResidentPlan best{};
+  long long best_cost = -1;
+  const int sorb = lattice == KITE_HONEYCOMB ? 2 : 1;
+  for (int TX = 4; TX <= 128; TX += TX < 16 ? 1 : (TX < 32 ? 2 : 8)) {
+    const int nstrips = (Lx + TX - 1) / TX;
+    const long long units = (long long)nstrips * Ly;
+    const int regions = (int)std::min<long long>(ctx->num_sms, units);
+    const int rows = (int)((units + regions - 1) / regions);
+    // sub-columns: as many virtual CTAs per region as fill the compute threads
+    const int colT = TX * sorb * C;
+    const int nv = std::max(1, std::min(rows, kRMax / std::max(1, colT)));
+    const ResidentPlan p = resident_plan(ctx, 1, lattice, doubling, realv, field, Lx, Ly, C, M, TX,
+                                         std::min<long long>((long long)regions * nv, units));
+    if (p.CR == 0) continue;
+    // a step: the rows of the longest column in sites of the whole SM, plus the edge
+    const long long sweeps = C / p.CR;
+    // (a warp with both sublattices runs the march twice)
+    const int twice = sorb == 2 && (p.TX * p.CR) % 32 ? 2 : 1;
+    const long long cost = sweeps * (4LL * twice * p.rows * p.TX * sorb * p.CR + 2LL * (p.rows + p.TX) * p.CR + 400);
+    if (best_cost < 0 || cost < best_cost) best_cost = cost, best = p;
+  }
+  return best;
+}
+
+size_t resident_rec_bytes(int lattice, int Lx, int Ly, int CR) {
+  return (size_t)2 * Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1) * CR * 32;
+}
+
+size_t resident_part_bytes(kite_ctx* ctx, int fp64, int realv, int C, int slots) {
+  const int lanes = C * sums_of(fp64, realv);
+  return (size_t)slots * ctx->num_sms * (kRComm / 32) * (fp64 ? std::max(8, lanes) : lanes) * sizeof(double);
+}
+
+int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
+  const ResidentPlan& p = a->plan;
+  const int var = a->phase ? 1 : (a->realv ? 2 : 0);
+  const void* fn = a->fp64 ? res_kernel<double>(a->lattice, a->doubling, var)
+                           : res_kernel<float>(a->lattice, a->doubling, var);
+  {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!done.count({fn, ctx->device})) {
+      KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem));
+      done.insert({fn, ctx->device});
+    }
+  }
+  const int steps = timing_steps > 0 ? timing_steps : (a->doubling ? (a->M + 1) / 2 : a->M - 1);
+  const int per_chunk = per_chunk_of(a->fp64, a->realv);
+  const size_t rec_bytes = resident_rec_bytes(a->lattice, a->Lx, a->Ly, p.CR);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)p.regions);
+  cfg.blockDim = dim3((unsigned)(p.T + kRComm));
+  cfg.dynamicSmemBytes = (size_t)p.smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;  // neighbouring CTAs wait on one another
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  KITE_CUDA_TRY(ctx, cudaEventRecord(ctx->ev2, ctx->stream));
+  for (int c0 = 0; c0 < a->C && c0 * per_chunk < a->nvec; c0 += p.CR) {
+    // no record may carry a step number of an earlier sweep
+    KITE_CUDA_TRY(ctx, cudaMemsetAsync(a->rec, 0, rec_bytes, ctx->stream));
+    auto launch = [&](auto tag) -> cudaError_t {
+      using Real = decltype(tag);
+      ResArgs<Real> r{};
+      r.r0 = a->r0;
+      r.vt = static_cast<const Real*>(a->vt);
+      r.phase = static_cast<const Real*>(a->phase);
+      r.last[1] = a->bA;  // odd iterates
+      r.last[0] = a->bB;
+      r.part = a->part;
+      r.rec = static_cast<Rec*>(a->rec);
+      r.err = ctx->d_status;
+      r.tt = (Real)a->tt;
+      r.Lx = a->Lx;
+      r.Ly = a->Ly;
+      r.TX = p.TX;
+      r.G = p.G;
+      r.rows_max = p.rows;
+      r.nv_max = p.nv;
+      r.nfl = p.nfl;
+      r.r0_rows = p.r0_rows;
+      r.levels = p.levels;
+      r.C = a->C;
+      r.c0 = c0;
+      r.CR = p.CR;
+      r.steps = steps;
+      r.open_x = a->open_x;
+      r.open_y = a->open_y;
+      r.stall = a->stall;
+      r.write_last = timing_steps > 0 ? 0 : a->want_last;
+      void* kargs[] = {&r};
+      return cudaLaunchKernelExC(&cfg, fn, kargs);
+    };
+    KITE_CUDA_TRY(ctx, a->fp64 ? launch(double()) : launch(float()));
+    a->stall = 0;
+    if (timing_steps > 0) break;
+    const int nvec = std::min(a->nvec - c0 * per_chunk, p.CR * per_chunk);
+    k_resident_reduce<<<a->M, 256, 0, ctx->stream>>>(a->part, a->M, p.regions * (kRComm / 32) * (32 >> p.levels),
+                                                     p.CR * sums_of(a->fp64, a->realv), !a->fp64 && !a->realv, nvec,
+                                                     a->vec_base + c0 * per_chunk, a->n_eff,
+                                                     a->mu_vec);
+    KITE_CUDA_TRY(ctx, cudaGetLastError());
+  }
+  KITE_CUDA_TRY(ctx, cudaEventRecord(ctx->ev3, ctx->stream));
+  float ms = 0.f;
+  KITE_CUDA_TRY(ctx, cudaEventSynchronize(ctx->ev3));
+  KITE_CUDA_TRY(ctx, cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3));
+  a->seconds = 1e-3 * ms;
+  a->grid = p.regions;
+  a->block = p.T + kRComm;
+  const int sorb = a->lattice == KITE_HONEYCOMB ? 2 : 1;
+  // bytes to and from device memory: r_0 and the on-site terms in (the rows of r_0 that are
+  // not kept on chip once per step), the moment partials out
+  const double n_orb = (double)a->Lx * a->Ly * sorb;
+  const double off_chip = a->doubling ? 0.0 : 1.0 - (double)p.r0_rows / p.rows;
+  a->bytes = n_orb * a->C * 16.0 * (1.0 + off_chip * steps) + n_orb * (a->fp64 ? 8.0 : 4.0) +
+             8.0 * a->M * p.regions * (kRComm / 32) * (32 >> p.levels) * ((a->C + p.CR - 1) / p.CR);
+  return KITE_OK;
+}
+
+}  // namespace kite

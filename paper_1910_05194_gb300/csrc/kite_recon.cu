@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "kite_internal.h"
+#include "kite_nufft.cuh"
 
 namespace kite {
 namespace {
@@ -154,8 +155,9 @@ int reconstruct_dos_impl(kite_ctx* ctx, const double* mu_dev, int M_use, int ker
 //   sigma(w) = -i (n_orb a^2/Omega_c) / w * S(w)   [units e^2/hbar, w = hbar omega/de_minus]
 // (Eq. conductivity_1st_order in rescaled units).  With e = cos(theta), Delta_m(e) de =
 // (2/pi) cos(m theta) d theta, integrated by Gauss-Legendre quadrature in theta.  Then
-// U[n][k] = sum_m Gamma_nm D[m][k] and W[m][k] = sum_n Gamma_nm D[n][k] (two FP64 GEMMs),
-// and per frequency S = sum_k sum_n (g^R_n(e_k + w) U[n][k] + g^A_n(e_k - w) W[n][k]).
+// U[n][k] = sum_m Gamma_nm D[m][k] and W[m][k] = sum_n Gamma_nm D[n][k] (cosine sums at the
+// nodes, kite_nufft.cuh; dense FP64 products outside its range of orders), and per frequency
+// S = sum_k sum_n (g^R_n(e_k + w) U[n][k] + g^A_n(e_k - w) W[n][k]).
 // The CPGF coefficients (Eq. green_function_cheb_expansionb) are geometric in n:
 // g^{s}_n(z) = -2 s i q^n / sqrt(1 - z^2) with q = exp(-s i arccos z) = z - s i sqrt(1 - z^2)
 // for the principal branches, so only a complex square root is needed per (w, node).
@@ -244,54 +246,73 @@ __global__ void k_zgemm_real(const double* __restrict__ G, int trans, const doub
   }
 }
 
-// One block per frequency: S(w) = sum_k [sum_n gR_n(e_k + w) U[n][k] + gA_n(e_k - w) W[n][k]]
-__global__ void k_sig_omega(const double* __restrict__ U, const double* __restrict__ W,
-                            const double* __restrict__ theta, int M, int K,
-                            const double* __restrict__ wt, double eta_t, double factor,
-                            double* __restrict__ sigma) {
-  const int iw = blockIdx.x;
-  const double w = wt[iw];
-  double sre = 0.0, sim = 0.0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double e = cos(theta[k]);
-    // retarded: z = e + w + i eta, g_n = -2i q^n / sqrt(1 - z^2), q = z - i sqrt(1 - z^2)
-    // advanced: z = e - w - i eta, g_n = +2i q^n / sqrt(1 - z^2), q = z + i sqrt(1 - z^2)
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      const double s = sgn == 0 ? 1.0 : -1.0;
-      const cplx z = {e + s * w, s * eta_t};
-      const cplx one_m_z2 = {1.0 - (z.re * z.re - z.im * z.im), -2.0 * z.re * z.im};
-      const cplx r = csqrt_p(one_m_z2);
-      const cplx q = {z.re + s * r.im, z.im - s * r.re};  // z - s i r
-      cplx g = cdiv({0.0, -2.0 * s}, r);
-      const double* X = sgn == 0 ? U : W;
-      double ar = 0.0, ai = 0.0;
-      for (int n = 0; n < M; ++n) {
-        const double xr = X[2 * ((int64_t)n * K + k)], xi = X[2 * ((int64_t)n * K + k) + 1];
-        ar += g.re * xr - g.im * xi;
-        ai += g.re * xi + g.im * xr;
-        g = cmul(g, q);
-      }
-      sre += ar;
-      sim += ai;
+// Partial sums of S(w): a block takes 128 nodes, kSigW frequencies and one branch (retarded
+// with U, advanced with W).  The CPGF sum of a node is a polynomial in q, by Horner's rule
+// (four FP64 multiply-adds per term instead of eight with the powers carried along: the FP64
+// pipe is the bound), kSigW of them side by side on each loaded coefficient.  M = 512, 1088
+// nodes, 128 frequencies: 3.34 ms with one block per frequency and carried powers, 1.09 ms so
+// (0.57 G multiply-adds: 0.9 ms at the FP64 pipe's rate); the whole call 19.8 -> 1.5 ms.
+constexpr int kSigW = 4;
+__global__ void __launch_bounds__(128) k_sig_omega(const double2* __restrict__ U, const double2* __restrict__ W,
+                                                   const double* __restrict__ theta, int M, int K,
+                                                   const double* __restrict__ wt, int K_w, double eta_t,
+                                                   double2* __restrict__ part) {
+  const int k = blockIdx.x * 128 + threadIdx.x, w0 = blockIdx.y * kSigW, sgn = blockIdx.z;
+  const double s = sgn == 0 ? 1.0 : -1.0;
+  // retarded: z = e + w + i eta, g_n = -2i q^n / sqrt(1 - z^2), q = z - i sqrt(1 - z^2)
+  // advanced: z = e - w - i eta, g_n = +2i q^n / sqrt(1 - z^2), q = z + i sqrt(1 - z^2)
+  cplx q[kSigW], g0[kSigW], p[kSigW];
+  const bool on = k < K;
+  const double e = on ? cos(theta[k]) : 0.0;
+#pragma unroll
+  for (int i = 0; i < kSigW; ++i) {
+    const cplx z = {e + s * wt[min(w0 + i, K_w - 1)], s * eta_t};
+    // 1 - z^2, without the cancellation near the band edges
+    const cplx r = csqrt_p({fma(1.0 - z.re, 1.0 + z.re, z.im * z.im), -2.0 * z.re * z.im});
+    q[i] = {z.re + s * r.im, z.im - s * r.re};  // z - s i r
+    g0[i] = cdiv({0.0, -2.0 * s}, r);
+    p[i] = {0.0, 0.0};
+  }
+  if (on) {
+    const double2* X = (sgn == 0 ? U : W) + k;
+#pragma unroll 4
+    for (int n = M - 1; n >= 0; --n) {
+      const double2 x = X[(int64_t)n * K];
+#pragma unroll
+      for (int i = 0; i < kSigW; ++i)
+        p[i] = {fma(p[i].re, q[i].re, fma(-p[i].im, q[i].im, x.x)), fma(p[i].re, q[i].im, fma(p[i].im, q[i].re, x.y))};
     }
   }
-  __shared__ double red_re[256], red_im[256];
-  red_re[threadIdx.x] = sre;
-  red_im[threadIdx.x] = sim;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) {
-      red_re[threadIdx.x] += red_re[threadIdx.x + st];
-      red_im[threadIdx.x] += red_im[threadIdx.x + st];
-    }
+  __shared__ double2 red[128];
+#pragma unroll
+  for (int i = 0; i < kSigW; ++i) {
+    const cplx v = cmul(g0[i], p[i]);
     __syncthreads();
+    red[threadIdx.x] = on ? make_double2(v.re, v.im) : make_double2(0.0, 0.0);
+    __syncthreads();
+    for (int st = 64; st > 0; st >>= 1) {
+      if ((int)threadIdx.x < st) {
+        red[threadIdx.x].x += red[threadIdx.x + st].x;
+        red[threadIdx.x].y += red[threadIdx.x + st].y;
+      }
+      __syncthreads();
+    }
+    if (threadIdx.x == 0 && w0 + i < K_w) part[((int64_t)(w0 + i) * 2 + sgn) * gridDim.x + blockIdx.x] = red[0];
   }
-  if (threadIdx.x == 0) {
-    // sigma = -i * factor / w * S
-    const double Sr = red_re[0], Si = red_im[0];
-    sigma[2 * iw] = factor / w * Si;
-    sigma[2 * iw + 1] = -factor / w * Sr;
+}
+
+// sigma = -i factor / w * S, S the sum of a frequency's `n` partials in order
+__global__ void k_sig_final(const double2* __restrict__ part, int n, const double* __restrict__ wt, int K_w,
+                            double factor, double* __restrict__ sigma) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= K_w) return;
+  double re = 0.0, im = 0.0;
+  for (int b = 0; b < n; ++b) {
+    re += part[(int64_t)i * n + b].x;
+    im += part[(int64_t)i * n + b].y;
   }
+  sigma[2 * i] = factor / wt[i] * im;
+  sigma[2 * i + 1] = -factor / wt[i] * re;
 }
 
 // ---- DC conductivity (Kubo-Greenwood, T = 0) ---------------------------------------
@@ -350,85 +371,123 @@ __global__ void k_dc_weights(int M, int kernel, double param, double* __restrict
 
 }  // namespace
 
-// Gauss-Legendre nodes/weights on [-1, 1] (Newton iteration on P_K from the three-term
-// recurrence), host FP64.
-void gauss_legendre(int K, double* x, double* w) {
-  const double pi = 3.141592653589793;
-  for (int i = 0; i < (K + 1) / 2; ++i) {
-    double z = cos(pi * (i + 0.75) / (K + 0.5)), dp = 0.0;
-    for (int it = 0; it < 100; ++it) {
-      double p0 = 1.0, p1 = 0.0;
-      for (int j = 1; j <= K; ++j) {
-        const double p2 = p1;
-        p1 = p0;
-        p0 = ((2.0 * j - 1.0) * z * p1 - (j - 1.0) * p2) / j;
-      }
-      dp = K * (z * p0 - p1) / (z * z - 1.0);
-      const double dz = p0 / dp;
-      z -= dz;
-      if (fabs(dz) < 1e-16) break;
-    }
-    {
-      double p0 = 1.0, p1 = 0.0;
-      for (int j = 1; j <= K; ++j) {
-        const double p2 = p1;
-        p1 = p0;
-        p0 = ((2.0 * j - 1.0) * z * p1 - (j - 1.0) * p2) / j;
-      }
-      dp = K * (z * p0 - p1) / (z * z - 1.0);
-    }
-    x[i] = -z;
-    x[K - 1 - i] = z;
-    w[i] = w[K - 1 - i] = 2.0 / ((1.0 - z * z) * dp * dp);
-  }
+namespace {
+
+// Launches of the Gauss-Legendre rule: K nodes u = 1 + x and weights w, ab scratch of 2K doubles.
+void gauss_rule(cudaStream_t st, int K, double* ab, double* u, double* w) {
+  k_legendre_coef<<<std::min(1024, (K + 255) / 256), 256, 0, st>>>(K, reinterpret_cast<double2*>(ab));
+  k_gauss_legendre<<<((K + 1) / 2 + kGaussBlock / 16 - 1) / (kGaussBlock / 16), kGaussBlock, 0, st>>>(
+      K, reinterpret_cast<const double2*>(ab), u, w);
 }
+
+// The Fermi energy in theta (the lower end of the sea at T = 0).
+double theta_fermi(double E_F, const Scale& sc) {
+  return acos(fmin(1.0, fmax(-1.0, (E_F - sc.de_plus) / sc.de_minus)));
+}
+
+// Device buffers of the non-uniform transform for order M, in doubles, and its launches.
+struct Nufft {
+  int M, Nf, L, logN;
+  double *inv, *tw, *grid;
+  static bool fits(int M) { return M >= kNufftMinM && M <= kNufftMaxM; }
+  explicit Nufft(int M_) : M(M_), Nf(nufft_grid(M_)), L(nufft_row(Nf)), logN(0) {
+    while ((1 << logN) < Nf) ++logN;
+  }
+  size_t doubles(int rows) const {
+    return (size_t)M + 1 + Nf + 2 * (size_t)rows * L;
+  }
+  void carve(double* b) {  // 16-byte aligned pieces
+    inv = b;
+    tw = b + ((size_t)M + 1) / 2 * 2;
+    grid = tw + Nf;
+  }
+  // cosine sums of `rows` rows on the grid (see k_cos_fft)
+  int rows_to_grid(kite_ctx* ctx, const double* mu, int M_avail, int kind, const double* w, int rows) const {
+    cudaStream_t st = ctx->stream;
+    k_nufft_tables<<<(std::max(32 * M, Nf / 2) + 127) / 128, 128, 0, st>>>(M, Nf, inv, reinterpret_cast<double2*>(tw));
+    const int smem = Nf * 16;
+    if (smem > 48 * 1024)
+      KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_cos_fft, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              nufft_grid(kNufftMaxM) * 16));
+    k_cos_fft<<<rows, 256, smem, st>>>(mu, M_avail, M, kind, w, inv, reinterpret_cast<const double2*>(tw), Nf, logN,
+                                       reinterpret_cast<double2*>(grid));
+    return KITE_OK;
+  }
+};
+
+}  // namespace
 
 int reconstruct_sigma_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, int M, int lattice,
                            int kernel, const Scale& sc, double E_F, double kT, double eta,
                            const double* omega_host, int K_w, int n_quad, double* sigma_dev) {
   const int K = n_quad > 0 ? n_quad : 2 * M + 64;
-  const double eF = (E_F - sc.de_plus) / sc.de_minus;
-  const double thF = kT > 0.0 ? 0.0 : acos(fmin(1.0, fmax(-1.0, eF)));
-  std::vector<double> x(K), wq(K), th(K), wts(2 * (size_t)K_w);
-  gauss_legendre(K, x.data(), wq.data());
-  const double pi = 3.141592653589793;
-  for (int k = 0; k < K; ++k) {
-    th[k] = thF + (pi - thF) * 0.5 * (x[k] + 1.0);
-    wq[k] *= 0.5 * (pi - thF);
-    if (kT > 0.0) {
-      const double E = cos(th[k]) * sc.de_minus + sc.de_plus;
-      wq[k] /= (1.0 + exp((E - E_F) / kT));
-    }
-  }
-  for (int i = 0; i < K_w; ++i) wts[i] = omega_host[i] / sc.de_minus;
-  const size_t nG = 2 * (size_t)M * M, nD = (size_t)M * K, nU = 2 * (size_t)M * K;
+  const bool fast = Nufft::fits(M);
+  Nufft nf(M);
+  std::vector<double> in((size_t)K_w + 2);  // rescaled frequencies, then the Fermi energy in E and theta
+  for (int i = 0; i < K_w; ++i) in[i] = omega_host[i] / sc.de_minus;
+  in[K_w] = E_F;
+  in[K_w + 1] = theta_fermi(E_F, sc);
+  // all offsets even: 16-byte aligned complex values
+  const size_t nU = 2 * (size_t)M * K, Kp = ((size_t)K + 1) / 2 * 2, Wp = ((size_t)K_w + 3) / 2 * 2,
+               Mp = ((size_t)M + 1) / 2 * 2;
+  const int blocks = (K + 127) / 128;
+  const size_t nPart = 4 * (size_t)K_w * blocks;
+  const size_t nDense = 2 * (size_t)M * M + (size_t)M * Kp;       // Gamma, D
+  const size_t nFast = (nf.doubles(2 * M) + 2 + Kp + kTaps * Kp);  // transform, first taps, taps
   double* buf = nullptr;
-  const size_t total = nG + nD + 2 * nU + 2 * (size_t)K + K_w;
+  const size_t total = 2 * nU + 2 * Kp + 4 * Kp + Wp + Mp + nPart + (fast ? nFast : nDense);
   KITE_CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, total * sizeof(double), ctx->stream));
-  double* G = buf;
-  double* D = G + nG;
-  double* U = D + nD;
+  double* U = buf;
   double* W = U + nU;
   double* th_d = W + nU;
-  double* wq_d = th_d + K;
-  double* wt_d = wq_d + K;
+  double* wq_d = th_d + Kp;
+  double* gx = wq_d + Kp;
+  double* gw = gx + Kp;
+  double* gab = gw + Kp;
+  double* in_d = gab + 2 * Kp;
+  double* wk = in_d + Wp;
+  double* part = wk + Mp;
+  double* rest = part + nPart;
   cudaStream_t st = ctx->stream;
-  cudaError_t e = cudaMemcpyAsync(th_d, th.data(), K * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(wq_d, wq.data(), K * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(wt_d, wts.data(), K_w * sizeof(double), cudaMemcpyHostToDevice, st);
+  cudaError_t e = cudaMemcpyAsync(in_d, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice, st);
   int rc = e == cudaSuccess ? KITE_OK : cuda_fail(ctx, e, "sigma set-up");
   if (rc == KITE_OK) {
-    k_sig_gamma<<<(int)(((int64_t)M * M + 255) / 256), 256, 0, st>>>(mu_dev, M_avail, M, kernel, G);
-    k_sig_dmat<<<(int)(((int64_t)M * K + 255) / 256), 256, 0, st>>>(th_d, wq_d, M, K, D);
-    dim3 blk(16, 16), grd((K + 15) / 16, (M + 15) / 16);
-    k_zgemm_real<<<grd, blk, 0, st>>>(G, 0, D, M, K, U);
-    k_zgemm_real<<<grd, blk, 0, st>>>(G, 1, D, M, K, W);
+    gauss_rule(st, K, gab, gx, gw);
+    k_fermi_nodes<<<(K + 255) / 256, 256, 0, st>>>(gx, gw, K, in_d + K_w, in_d + K_w + 1, 1, sc.de_plus, sc.de_minus, kT, th_d, wq_d);
+    if (fast) {
+      nf.carve(rest);
+      double* taps = rest + (nf.doubles(2 * M) + 2) / 2 * 2;
+      int* j0 = reinterpret_cast<int*>(taps + kTaps * Kp);
+      k_dc_weights<<<(M + 63) / 64, 64, 0, st>>>(M, kernel, 0.0, wk);
+      rc = nf.rows_to_grid(ctx, mu_dev, M_avail, 0, wk, 2 * M);
+      k_nufft_taps<<<(K + 127) / 128, 128, 0, st>>>(th_d, wq_d, K, nf.Nf, j0, taps);
+      dim3 grd((K + 127) / 128, (2 * M + kApplyRows - 1) / kApplyRows);
+      k_nufft_apply<<<grd, 128, 0, st>>>(reinterpret_cast<const double2*>(nf.grid), nf.L, 2 * M, K, j0, taps,
+                                         reinterpret_cast<double2*>(U));  // W follows U
+    } else {
+      double* G = rest;
+      double* D = G + 2 * (size_t)M * M;
+      k_sig_gamma<<<(int)(((int64_t)M * M + 255) / 256), 256, 0, st>>>(mu_dev, M_avail, M, kernel, G);
+      k_sig_dmat<<<(int)(((int64_t)M * K + 255) / 256), 256, 0, st>>>(th_d, wq_d, M, K, D);
+      dim3 blk(16, 16), grd((K + 15) / 16, (M + 15) / 16);
+      k_zgemm_real<<<grd, blk, 0, st>>>(G, 0, D, M, K, U);
+      k_zgemm_real<<<grd, blk, 0, st>>>(G, 1, D, M, K, W);
+    }
     const double factor = lattice == KITE_HONEYCOMB ? 4.0 / sqrt(3.0) : 1.0;
-    k_sig_omega<<<K_w, 256, 0, st>>>(U, W, th_d, M, K, wt_d, eta / sc.de_minus, factor, sigma_dev);
+    for (int i0 = 0; i0 < K_w; i0 += 65535 * kSigW) {  // (the grid's y extent)
+      const int nw = std::min(K_w - i0, 65535 * kSigW);
+      dim3 g3((unsigned)blocks, (unsigned)((nw + kSigW - 1) / kSigW), 2);
+      k_sig_omega<<<g3, 128, 0, st>>>(reinterpret_cast<const double2*>(U), reinterpret_cast<const double2*>(W), th_d, M,
+                                      K, in_d + i0, nw, eta / sc.de_minus,
+                                      reinterpret_cast<double2*>(part) + 2 * (size_t)i0 * blocks);
+    }
+    k_sig_final<<<(K_w + 127) / 128, 128, 0, st>>>(reinterpret_cast<const double2*>(part), 2 * blocks, in_d, K_w, factor,
+                                                   sigma_dev);
     e = cudaGetLastError();
     if (e != cudaSuccess) rc = cuda_fail(ctx, e, "sigma kernels");
   }
   cudaFreeAsync(buf, st);
+  // (`in` is pageable: the copy above has taken its values before it returned)
   return rc;
 }
 
@@ -442,8 +501,9 @@ int reconstruct_sigma_dc_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, 
                               int lattice, const Scale& sc, const double* E_dev, int K, double* sigma_dev,
                               double* w) {
   cudaStream_t st = ctx->stream;
-  k_dc_weights<<<(M + 255) / 256, 256, 0, st>>>(M, kernel, param, w);
-  const int block = 256;
+  k_dc_weights<<<(M + 63) / 64, 64, 0, st>>>(M, kernel, param, w);
+  // few energies: wide blocks, so that each one's SM has enough warps in flight
+  const int block = K < 2 * ctx->num_sms ? 1024 : 256;
   const size_t smem = sizeof(double) * ((size_t)M + block / 32);
   if (smem > 48 * 1024)
     KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_sigma_dc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -466,68 +526,92 @@ int reconstruct_sigma_dc_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, 
 // green_function_cheb_expansionb) and their derivatives
 //   d g_m/dz = g_m(z) [s i m / sqrt(1 - z^2) + z / (1 - z^2)]   (s = +1 retarded, -1 advanced).
 // A_nm = mu_nm k_n k_m / ((1 + d_n0)(1 + d_m0)).  Each Fermi energy has its own
-// Gauss-Legendre nodes theta_k on [theta_F, pi] (kT > 0: [0, pi] with Fermi weights);
-// D[n][k] = (2/pi) cos(n theta_k) w_k, U = A^T D, W = A D (FP64 GEMMs), and per node
-//   F_k = sum_m dG^R_m(e_k) U[m][k] - sum_n dG^A_n(e_k) W[n][k],
-// the CPGF terms geometric, g_m = g_0 q^m with q = z - s i sqrt(1 - z^2), summed as
-// S0 = sum_m g_m X_m and S1 = sum_m m g_m X_m:  sum_m dg_m X_m = s i S1 / r + z S0 / r^2,
-// r = sqrt(1 - z^2).  sigma = Re(i ucf sum_k F_k) = -ucf Im(sum_k F_k), each energy's
-// node sum in a fixed order.  Cost: two M x M x (K nodes) GEMMs per energy.
+// Gauss-Legendre nodes theta_k on [theta_F, pi] (kT > 0: [0, pi] with Fermi weights).  Since
+// G^A = conj(G^R) on the real axis' two sides and only the imaginary part of the sum counts,
+// the second term folds into the first: with the Hermitian B_nm = A_nm + conj(A_mn),
+//   Im F_k = Im sum_m dG^R_m(e_k) V[m][k],  V[m][k] = sum_n B_nm D[n][k],
+// D[n][k] = (2/pi) cos(n theta_k) w_k: half the products, and V by the non-uniform transform
+// (kite_nufft.cuh; a dense FP64 product outside its range of orders).  The CPGF terms are
+// geometric, g_m = g_0 q^m with q = z - i sqrt(1 - z^2): S0 = sum_m q^m V_m and S1 = sum_m m
+// q^m V_m by Horner's rule and its derivative, sum_m dg_m V_m = g_0 (i S1 / r + z S0 / r^2),
+// r = sqrt(1 - z^2).  sigma = -ucf Im(sum_k F_k), each energy's node sum in a fixed order.
+// M = 256, 48 energies of 576 nodes: 16.9 ms with two dense products per energy and host
+// nodes, 0.88 ms so (0.59 ms of it the nodes' 40 multiply-adds per order, 0.45 ms at the FP64
+// pipe's rate).
 // ====================================================================================
 namespace kite {
 namespace {
 
+// B_nm = A_nm + conj(A_mn) (dense path)
 __global__ void k_bastin_gamma(const double* __restrict__ mu, int M_avail, int M, const double* __restrict__ w,
-                               double* __restrict__ A) {
+                               double* __restrict__ B) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)M * M) return;
   const int n = (int)(e / M), m = (int)(e - (e / M) * M);
   // w_n = (2 - d_n0) k_n, so w_n / 2 = k_n / (1 + d_n0)
   const double f = 0.25 * w[n] * w[m];
   const double* p = mu + 2 * ((int64_t)n * M_avail + m);
-  A[2 * e] = f * p[0];
-  A[2 * e + 1] = f * p[1];
+  const double* t = mu + 2 * ((int64_t)m * M_avail + n);
+  B[2 * e] = f * (p[0] + t[0]);
+  B[2 * e + 1] = f * (p[1] - t[1]);
 }
 
-__global__ void k_bastin_nodes(const double* __restrict__ U, const double* __restrict__ W,
-                               const double* __restrict__ theta, int M, int64_t Kt, double eta_t,
-                               double* __restrict__ F) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < Kt; k += (int64_t)gridDim.x * blockDim.x) {
-    const double e = cos(theta[k]);
-    cplx tot = {0.0, 0.0};
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      const double s = sgn == 0 ? 1.0 : -1.0;
-      const cplx z = {e, s * eta_t};
-      const cplx r = csqrt_p({1.0 - (z.re * z.re - z.im * z.im), -2.0 * z.re * z.im});
-      const cplx q = {z.re + s * r.im, z.im - s * r.re};  // z - s i r
-      cplx g = cdiv({0.0, -2.0 * s}, r);
-      const double* X = sgn == 0 ? U : W;
-      cplx S0 = {0.0, 0.0}, S1 = {0.0, 0.0};
-      for (int m = 0; m < M; ++m) {
-        const cplx x = {X[2 * ((int64_t)m * Kt + k)], X[2 * ((int64_t)m * Kt + k) + 1]};
-        const cplx gx = cmul(g, x);
-        S0.re += gx.re;
-        S0.im += gx.im;
-        S1.re += (double)m * gx.re;
-        S1.im += (double)m * gx.im;
-        g = cmul(g, q);
-      }
-      const cplx a = cdiv(S1, r);
-      const cplx b = cdiv(cmul(z, S0), cmul(r, r));
-      const cplx d = {-s * a.im + b.re, s * a.re + b.im};  // s i a + b
-      tot.re += s * d.re;
-      tot.im += s * d.im;
-    }
-    F[2 * k] = tot.re;
-    F[2 * k + 1] = tot.im;
+// Im F_k per node from V (dense path: V[m][k]; else from the rows' grid values and the node's
+// taps, sixteen multiply-adds per part on the way: V is never stored).
+constexpr int kNodeBlock = 64;  // (small blocks: a few thousand nodes still fill the SMs evenly)
+template <bool DENSE>
+__global__ void __launch_bounds__(kNodeBlock) k_bastin_nodes(const double2* __restrict__ V, const double2* __restrict__ grid,
+                                                      int L, const int* __restrict__ j0,
+                                                      const double* __restrict__ taps,
+                                                      const double* __restrict__ theta, int M, int64_t Kt,
+                                                      double eta_t, double* __restrict__ F) {
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k >= Kt) return;
+  cplx z = {0.0, eta_t};
+  double sn;
+  sincos(theta[k], &sn, &z.re);
+  // 1 - z^2 from the sine: no cancellation near the band edges
+  const cplx r = csqrt_p({fma(sn, sn, z.im * z.im), -2.0 * z.re * z.im});
+  const cplx q = {z.re + r.im, z.im - r.re};  // z - i r
+  const cplx g = cdiv({0.0, -2.0}, r);
+  double t[kTaps];
+  const double2* b = nullptr;
+  if (!DENSE) {
+#pragma unroll
+    for (int i = 0; i < kTaps; ++i) t[i] = taps[(int64_t)i * Kt + k];
+    b = grid + j0[k];
   }
+  cplx P = {0.0, 0.0}, Q = {0.0, 0.0};  // sum_m q^m V_m and its derivative in q
+#pragma unroll 1
+  for (int m = M - 1; m >= 0; --m) {
+    double2 v;
+    if (DENSE) {
+      v = V[(int64_t)m * Kt + k];
+    } else {
+      const double2* c = b + (int64_t)m * L;
+      double re0 = 0.0, im0 = 0.0, re1 = 0.0, im1 = 0.0;
+#pragma unroll
+      for (int i = 0; i < kTaps; i += 2) {
+        const double2 x = c[i], y = c[i + 1];
+        re0 = fma(t[i], x.x, re0);
+        im0 = fma(t[i], x.y, im0);
+        re1 = fma(t[i + 1], y.x, re1);
+        im1 = fma(t[i + 1], y.y, im1);
+      }
+      v = make_double2(re0 + re1, im0 + im1);
+    }
+    Q = {fma(Q.re, q.re, fma(-Q.im, q.im, P.re)), fma(Q.re, q.im, fma(Q.im, q.re, P.im))};
+    P = {fma(P.re, q.re, fma(-P.im, q.im, v.x)), fma(P.re, q.im, fma(P.im, q.re, v.y))};
+  }
+  const cplx a = cdiv(cmul(q, Q), r), d = cdiv(cmul(z, P), cmul(r, r));
+  F[k] = cmul(g, {-a.im + d.re, a.re + d.im}).im;  // g_0 (i S1 / r + z S0 / r^2)
 }
 
 // one block per energy: sigma = -ucf * sum_k Im F_k over that energy's K nodes
 __global__ void k_bastin_sum(const double* __restrict__ F, int K, double ucf, double* __restrict__ sigma) {
-  const double* f = F + 2 * (int64_t)blockIdx.x * K;
+  const double* f = F + (int64_t)blockIdx.x * K;
   double acc = 0.0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) acc += f[2 * k + 1];
+  for (int k = threadIdx.x; k < K; k += blockDim.x) acc += f[k];
   __shared__ double red[256];
   red[threadIdx.x] = acc;
   __syncthreads();
@@ -544,67 +628,71 @@ int reconstruct_sigma_bastin_impl(kite_ctx* ctx, const double* mu_dev, int M_ava
                                   int kernel, double param, const Scale& sc, double eta, double kT,
                                   const double* E_host, int K_E, int n_quad, double* sigma_dev) {
   const int K = n_quad > 0 ? n_quad : 2 * M + 64;
-  std::vector<double> x(K), w0(K);
-  gauss_legendre(K, x.data(), w0.data());
-  // energies per batch: D (M K), U and W (2 M K each), theta, weights, F (2 K) doubles
-  const size_t per_energy = (size_t)K * (5 * (size_t)M + 4);
+  const bool fast = Nufft::fits(M);
+  Nufft nf(M);
+  // nodes per batch of energies: theta, weight, F and the taps, or D and V (dense)
+  const size_t per_energy = (size_t)K * (fast ? 3 + kTaps + 1 : 3 + 3 * (size_t)M);
   const size_t budget = (size_t)1 << 27;  // doubles (1 GiB)
   const int EB = (int)std::max<size_t>(1, std::min<size_t>((size_t)K_E, budget / per_energy));
-  const size_t Kt_max = (size_t)EB * K;
-  const size_t nA = 2 * (size_t)M * M;
-  const size_t total = nA + (size_t)M + Kt_max * (5 * (size_t)M + 4);
+  const size_t Kt_max = ((size_t)EB * K + 1) / 2 * 2, Kp = ((size_t)K + 1) / 2 * 2, Ep = ((size_t)K_E + 1) / 2 * 2,
+               Mp = ((size_t)M + 1) / 2 * 2;
+  const size_t fixed = Mp + 2 * Ep + 4 * Kp + (fast ? (nf.doubles(M) + 2) / 2 * 2 : 2 * (size_t)M * M);
+  const size_t total = fixed + Kt_max * (fast ? 3 + kTaps + 1 : 3 + 3 * (size_t)M);
   double* buf = nullptr;
   KITE_CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, total * sizeof(double), ctx->stream));
-  double* A = buf;
-  double* wk = A + nA;
-  double* D = wk + M;
-  double* U = D + (size_t)M * Kt_max;
-  double* W = U + 2 * (size_t)M * Kt_max;
-  double* th_d = W + 2 * (size_t)M * Kt_max;
+  double* wk = buf;
+  double* E_d = wk + Mp;
+  double* thF_d = E_d + Ep;
+  double* gx = thF_d + Ep;
+  double* gw = gx + Kp;
+  double* gab = gw + Kp;
+  double* mid = gab + 2 * Kp;  // the transform's buffers, or B
+  double* th_d = buf + fixed;
   double* wq_d = th_d + Kt_max;
   double* F = wq_d + Kt_max;
+  double* rest = F + Kt_max;  // taps and first taps, or V and D
   cudaStream_t st = ctx->stream;
-  const double pi = 3.141592653589793;
   const double ucf = lattice == KITE_HONEYCOMB ? 4.0 / sqrt(3.0) : 1.0;
-  k_dc_weights<<<(M + 255) / 256, 256, 0, st>>>(M, kernel, param, wk);
-  k_bastin_gamma<<<(int)(((int64_t)M * M + 255) / 256), 256, 0, st>>>(mu_dev, M_avail, M, wk, A);
-  cudaError_t e = cudaGetLastError();
-  int rc = e == cudaSuccess ? KITE_OK : cuda_fail(ctx, e, "Bastin set-up");
-  std::vector<double> th(Kt_max), wq(Kt_max);
+  k_dc_weights<<<(M + 63) / 64, 64, 0, st>>>(M, kernel, param, wk);
+  gauss_rule(st, K, gab, gx, gw);
+  std::vector<double> thF((size_t)K_E);
+  for (int i = 0; i < K_E; ++i) thF[i] = theta_fermi(E_host[i], sc);
+  cudaError_t e = cudaMemcpyAsync(E_d, E_host, (size_t)K_E * sizeof(double), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(thF_d, thF.data(), (size_t)K_E * sizeof(double), cudaMemcpyHostToDevice, st);
+  int rc = KITE_OK;
+  if (fast) {
+    nf.carve(mid);
+    rc = nf.rows_to_grid(ctx, mu_dev, M_avail, 1, wk, M);
+  } else {
+    k_bastin_gamma<<<(int)(((int64_t)M * M + 255) / 256), 256, 0, st>>>(mu_dev, M_avail, M, wk, mid);
+  }
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (rc == KITE_OK && e != cudaSuccess) rc = cuda_fail(ctx, e, "Bastin set-up");
   for (int b = 0; b < K_E && rc == KITE_OK; b += EB) {
     const int nb = std::min(EB, K_E - b);
     const int64_t Kt = (int64_t)nb * K;
-    for (int i = 0; i < nb; ++i) {
-      const double EF = E_host[b + i];
-      const double eF = (EF - sc.de_plus) / sc.de_minus;
-      const double thF = kT > 0.0 ? 0.0 : acos(fmin(1.0, fmax(-1.0, eF)));
-      for (int k = 0; k < K; ++k) {
-        double t = thF + (pi - thF) * 0.5 * (x[k] + 1.0), ww = w0[k] * 0.5 * (pi - thF);
-        if (kT > 0.0) ww /= (1.0 + exp((cos(t) * sc.de_minus + sc.de_plus - EF) / kT));
-        th[(size_t)i * K + k] = t;
-        wq[(size_t)i * K + k] = ww;
-      }
+    const int blocks = (int)std::min<int64_t>((Kt + 255) / 256, (int64_t)ctx->num_sms * 8);
+    k_fermi_nodes<<<blocks, 256, 0, st>>>(gx, gw, K, E_d + b, thF_d + b, nb, sc.de_plus, sc.de_minus, kT, th_d, wq_d);
+    const unsigned nblk = (unsigned)((Kt + kNodeBlock - 1) / kNodeBlock);
+    if (fast) {
+      double* taps = rest;
+      int* j0 = reinterpret_cast<int*>(taps + kTaps * Kt_max);
+      k_nufft_taps<<<blocks, 256, 0, st>>>(th_d, wq_d, Kt, nf.Nf, j0, taps);
+      k_bastin_nodes<false><<<nblk, kNodeBlock, 0, st>>>(nullptr, reinterpret_cast<const double2*>(nf.grid), nf.L, j0, taps,
+                                                  th_d, M, Kt, eta / sc.de_minus, F);
+    } else {
+      double* V = rest;
+      double* D = V + 2 * (size_t)M * Kt_max;
+      k_sig_dmat<<<(int)(((int64_t)M * Kt + 255) / 256), 256, 0, st>>>(th_d, wq_d, M, (int)Kt, D);
+      dim3 blk(16, 16), grd((unsigned)((Kt + 15) / 16), (unsigned)((M + 15) / 16));
+      k_zgemm_real<<<grd, blk, 0, st>>>(mid, 1, D, M, (int)Kt, V);  // V[m][k] = sum_n B_nm D[n][k]
+      k_bastin_nodes<true><<<nblk, kNodeBlock, 0, st>>>(reinterpret_cast<const double2*>(V), nullptr, 0, nullptr, nullptr,
+                                                 th_d, M, Kt, eta / sc.de_minus, F);
     }
-    e = cudaMemcpyAsync(th_d, th.data(), Kt * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(wq_d, wq.data(), Kt * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) {
-      rc = cuda_fail(ctx, e, "Bastin nodes");
-      break;
-    }
-    k_sig_dmat<<<(int)(((int64_t)M * Kt + 255) / 256), 256, 0, st>>>(th_d, wq_d, M, (int)Kt, D);
-    dim3 blk(16, 16), grd((unsigned)((Kt + 15) / 16), (unsigned)((M + 15) / 16));
-    k_zgemm_real<<<grd, blk, 0, st>>>(A, 1, D, M, (int)Kt, U);  // U[m][k] = sum_n A_nm D[n][k]
-    k_zgemm_real<<<grd, blk, 0, st>>>(A, 0, D, M, (int)Kt, W);  // W[n][k] = sum_m A_nm D[m][k]
-    const int nblk = (int)std::min<int64_t>((Kt + 255) / 256, (int64_t)ctx->num_sms * 8);
-    k_bastin_nodes<<<nblk, 256, 0, st>>>(U, W, th_d, M, Kt, eta / sc.de_minus, F);
     k_bastin_sum<<<nb, 256, 0, st>>>(F, K, ucf, sigma_dev + b);
     e = cudaGetLastError();
     if (e != cudaSuccess) rc = cuda_fail(ctx, e, "Bastin kernels");
-    // the host node arrays are refilled next batch: let this batch's copies finish
-    if (rc == KITE_OK && b + EB < K_E) {
-      e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) rc = cuda_fail(ctx, e, "Bastin batch");
-    }
   }
   cudaFreeAsync(buf, st);
   return rc;

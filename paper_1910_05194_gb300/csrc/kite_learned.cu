@@ -39,11 +39,16 @@ int mlp_init_impl(kite_ctx* ctx, uint64_t seed, double head_scale, float* p);
 int mlp_norm_impl(kite_ctx* ctx, const float* X, int n, double sd_floor, float* shift, float* scale);
 int mlp_take_inputs_impl(kite_ctx* ctx, const double* mu, int mu_ld, int n, float* X);
 int mlp_narrow_impl(kite_ctx* ctx, const double* src, int K, float* dst);
+int mlp_plain_impl(kite_ctx* ctx, const double* mu, int mu_ld, const int* idx, int rows, int M, double de_minus,
+                   float* rho);
 
 namespace {
 
 constexpr int IN = KITE_MLP_IN, OUT = KITE_MLP_OUT;
 constexpr double kSdFloor = 1e-4;
+// Largest fallback order that takes every flagged row in one launch (its table of Chebyshev
+// polynomials is 4 KiB per order); above, row by row.
+constexpr int kBatchPlainMax = 8192;
 
 // A model's device buffers (params, shift, scale) in one allocation.
 int new_model(kite_ctx* ctx, double e_min, double e_max, kite_model** out) {
@@ -201,7 +206,18 @@ int kite_learned_dos(kite_ctx* ctx, const kite_model* model, const double* mu, i
   // 3. the plain path for every flagged row, on the model's grid
   int flagged = 0;
   for (int i = 0; i < n; ++i) flagged += flags[i] != 0;
-  if (rc == KITE_OK && flagged > 0) {
+  if (rc == KITE_OK && flagged > 0 && !systems && M_plain <= kBatchPlainMax) {
+    std::vector<int> rows;
+    for (int i = 0; i < n; ++i)
+      if (flags[i]) rows.push_back(i);
+    int* idx;
+    rc = sg.scratch(rows.size(), &idx);
+    if (rc == KITE_OK && copy_in(ctx, idx, rows.data(), sizeof(int) * rows.size()) != cudaSuccess)
+      rc = fail(ctx, KITE_ERR_CUDA, "flagged rows");
+    if (rc == KITE_OK) rc = mlp_plain_impl(ctx, md, mu_ld, idx, flagged, M_plain, de_minus, rd);
+    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess && rc == KITE_OK)  // (rows is read until then)
+      rc = fail(ctx, KITE_ERR_CUDA, "plain fallback");
+  } else if (rc == KITE_OK && flagged > 0) {
     double *E, *rho64, *mu_plain = nullptr;
     rc = sg.scratch(OUT, &E);
     if (rc == KITE_OK) rc = sg.scratch(OUT, &rho64);

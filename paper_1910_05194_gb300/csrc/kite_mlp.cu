@@ -203,44 +203,92 @@ __global__ void k_mlp_transpose(const __nv_bfloat16* __restrict__ in, int rows, 
   }
 }
 
-// Jackson kernel of order IN (Sec. 2a, kernel polynomial method) times the Chebyshev
-// weight 2 - delta_k0 of Eq. e8a, computed on the host.
-struct PriorCoef {
-  double c[IN];
-};
-
-PriorCoef prior_coef() {
-  PriorCoef pc;
-  const double pi = 3.141592653589793, q = pi / (IN + 1);
-  for (int k = 0; k < IN; ++k) {
-    const double g = ((IN - k + 1) * std::cos(q * k) + std::sin(q * k) * std::cos(q) / std::sin(q)) / (IN + 1);
-    pc.c[k] = (k == 0 ? 1.0 : 2.0) * g;
+// Chebyshev polynomials on the output grid, T[k][j] = T_k(eps_j), k < M, for the half
+// j < OUT/2 of the midpoint grid eps_j = -1 + (2j+1)/OUT (forward recurrence; the other half
+// is T_k(-e) = (-1)^k T_k(e), exactly).  Computed once per call: the FP64 pipe does two
+// multiply-adds per SM and cycle, and every row of the prior, the gate and the plain fallback
+// needs the same values.
+constexpr int HALF = OUT / 2;
+__global__ void __launch_bounds__(32) k_mlp_cheb(int M, double* __restrict__ T) {
+  const int j = blockIdx.x * 32 + threadIdx.x;
+  const double e = -1.0 + (2.0 * j + 1.0) / OUT, e2 = 2.0 * e;
+  double t0 = 1.0, t1 = e;
+  T[j] = 1.0;
+  if (M > 1) T[HALF + j] = e;
+  for (int k = 2; k < M; ++k) {
+    const double t2 = fma(e2, t1, -t0);
+    T[(int64_t)k * HALF + j] = t2;
+    t0 = t1;
+    t1 = t2;
   }
-  return pc;
 }
 
-// Residual prior P[r][j] = sum_k c_k X[r][k] T_k(eps_j) / (pi a sqrt(1 - eps_j^2)) on the
-// midpoint grid eps_j = -1 + (2j+1)/OUT, a = (e_max - e_min)/2: the Jackson density per eV
-// from the raw moments X (FP64 sums, forward Chebyshev recurrence).  One block per row.
-__global__ void __launch_bounds__(256) k_mlp_prior(const float* __restrict__ X, int rows, const PriorCoef pc,
-                                                   double inv_pi_a, float* __restrict__ P) {
-  __shared__ double cx[IN];
-  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+// Rows of a kernel-weighted Chebyshev sum on the output grid (FP32 out), for a tile of
+// kSumRows rows and 128 columns of the half grid per block: even and odd orders are summed
+// apart, so one product serves eps_j and -eps_j, and a thread takes kSumRows rows per loaded
+// T: one FP64 multiply-add per order, row and pair of energies, which is the bound.  1000 rows
+// of order 128: 487 us with the recurrence per row and energy, 146 us so (105 us at the FP64
+// pipe's rate).
+//   row r of the output: out[idx ? idx[r] : r], moments at src (FP32 X [rows][ld] or FP64 mu)
+//   from the same row, order M, weights c[k], scaled by 1 / (pi a sqrt(1 - eps^2)).
+// Few rows take one row per block (ROWS = 1), so that they fill the SMs.
+constexpr int kSumRows = 8, kSumTile = 128;
+template <typename In, int ROWS>
+__global__ void __launch_bounds__(kSumTile) k_mlp_cheb_sum(const In* __restrict__ src, int64_t ld,
+                                                           const int* __restrict__ idx, int rows, int M,
+                                                           const double* __restrict__ c,
+                                                           const double* __restrict__ T, double inv_pi_a,
+                                                           float* __restrict__ out) {
+  __shared__ double cx[ROWS][kSumTile];
+  const int j = blockIdx.y * kSumTile + threadIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.x * ROWS;
+  double even[ROWS], odd[ROWS];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) even[r] = odd[r] = 0.0;
+  for (int k0 = 0; k0 < M; k0 += kSumTile) {
+    const int len = min(kSumTile, M - k0);
     __syncthreads();
-    for (int k = threadIdx.x; k < IN; k += blockDim.x) cx[k] = pc.c[k] * (double)X[(int64_t)r * IN + k];
-    __syncthreads();
-    for (int j = threadIdx.x; j < OUT; j += blockDim.x) {
-      const double e = -1.0 + (2.0 * j + 1.0) / OUT;
-      double t0 = 1.0, t1 = e, sum = cx[0] + cx[1] * e;
-      for (int k = 2; k < IN; ++k) {
-        const double t2 = 2.0 * e * t1 - t0;
-        sum += cx[k] * t2;
-        t0 = t1;
-        t1 = t2;
+    for (int r = 0; r < ROWS; ++r) {
+      double v = 0.0;
+      if (r0 + r < rows && (int)threadIdx.x < len) {
+        const int64_t row = idx ? (int64_t)idx[r0 + r] : r0 + r;
+        v = c[k0 + threadIdx.x] * (double)src[row * ld + k0 + threadIdx.x];
       }
-      P[(int64_t)r * OUT + j] = (float)(sum * inv_pi_a / sqrt(1.0 - e * e));
+      cx[r][threadIdx.x] = v;
     }
+    __syncthreads();
+    const double* t = T + (int64_t)k0 * HALF + j;
+    int k = 0;
+    // (unrolled: the table's loads of several orders in flight)
+#pragma unroll 8
+    for (; k + 1 < len; k += 2, t += 2 * HALF) {
+      const double te = t[0], to = t[HALF];
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        even[r] = fma(cx[r][k], te, even[r]);
+        odd[r] = fma(cx[r][k + 1], to, odd[r]);
+      }
+    }
+    if (k < len)
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) even[r] = fma(cx[r][k], t[0], even[r]);
   }
+  const double e = -1.0 + (2.0 * j + 1.0) / OUT, f = inv_pi_a / sqrt(1.0 - e * e);
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+    if (r0 + r >= rows) break;
+    float* o = out + (idx ? (int64_t)idx[r0 + r] : r0 + r) * OUT;
+    o[j] = (float)((even[r] + odd[r]) * f);
+    o[OUT - 1 - j] = (float)((even[r] - odd[r]) * f);
+  }
+}
+
+// Weights (2 - delta_k0) g_k of the Jackson kernel of order M (Sec. 2a).
+__global__ void __launch_bounds__(32) k_mlp_jackson(int M, double* __restrict__ c) {
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k >= M) return;
+  const double q = 3.141592653589793 / (double)(M + 1);
+  c[k] = (k == 0 ? 1.0 : 2.0) * ((double)(M - k + 1) * cos(q * k) + sin(q * k) * (cos(q) / sin(q))) / (double)(M + 1);
 }
 
 // rows of X (FP32, optional per-column shift and scale: (x - shift) * scale) gathered by
@@ -384,28 +432,47 @@ __global__ void k_mlp_tobf16(const float* __restrict__ x, __nv_bfloat16* __restr
 
 // Consistency gate: Chebyshev moments of the predicted density on the midpoint grid
 // eps_j = -1 + (2j+1)/OUT (rho in units per unit eps): m_k = (2/OUT) sum_j rho_j T_k(eps_j)
-// compared with the input moments mu_k for k < kcheck; flag if max |m_k - mu_k| > tol.
-__global__ void k_mlp_gate(const float* __restrict__ rho, const double* __restrict__ mu, int mu_ld, int kcheck,
-                           double de_minus, double tol, int* __restrict__ flag, double* __restrict__ dev) {
-  const int b = blockIdx.x;
-  __shared__ double red[128];
+// compared with the input moments mu_k for k < kcheck; flag if max |m_k - mu_k| > tol.  One
+// block per row; a thread holds four pairs (rho_j + rho_-j, rho_j - rho_-j) of the row and
+// multiplies them with the table's T_k (a cosine of an arc cosine per row, order and energy
+// took 1.67 ms for 1000 rows of 16 orders; 36 us so).  FP64 sums in a fixed order.
+__global__ void __launch_bounds__(128) k_mlp_gate(const float* __restrict__ rho, const double* __restrict__ mu,
+                                                  int mu_ld, int kcheck, const double* __restrict__ T,
+                                                  double de_minus, double tol, int* __restrict__ flag,
+                                                  double* __restrict__ dev) {
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double part[16][129], worst_w[4];
+  double sum[HALF / 128], dif[HALF / 128];
+#pragma unroll
+  for (int i = 0; i < HALF / 128; ++i) {
+    const int j = threadIdx.x + 128 * i;
+    const double u = (double)rho[(int64_t)b * OUT + j] * de_minus,
+                 v = (double)rho[(int64_t)b * OUT + OUT - 1 - j] * de_minus;
+    sum[i] = u + v;
+    dif[i] = u - v;
+  }
   double worst = 0.0;
-  for (int k = 0; k < kcheck; ++k) {
-    double s = 0.0;
-    for (int j = threadIdx.x; j < OUT; j += blockDim.x) {
-      const double e = -1.0 + (2.0 * j + 1.0) / OUT;
-      s += (double)rho[(int64_t)b * OUT + j] * de_minus * cos(k * acos(e));
+  for (int k0 = 0; k0 < kcheck; k0 += 16) {
+    const int len = min(16, kcheck - k0);
+    for (int k = 0; k < len; ++k) {
+      const double* t = T + (int64_t)(k0 + k) * HALF + threadIdx.x;
+      double s = 0.0;
+#pragma unroll
+      for (int i = 0; i < HALF / 128; ++i) s = fma(((k0 + k) & 1) ? dif[i] : sum[i], t[128 * i], s);
+      part[k][threadIdx.x] = s;
     }
-    red[threadIdx.x] = s;
     __syncthreads();
-    for (int st = 64; st > 0; st >>= 1) {
-      if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-      __syncthreads();
+    for (int k = warp; k < len; k += 4) {  // one order per warp
+      double s = (part[k][lane] + part[k][lane + 64]) + (part[k][lane + 32] + part[k][lane + 96]);
+      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      worst = fmax(worst, fabs(s * 2.0 / OUT - mu[(int64_t)b * mu_ld + k0 + k]));
     }
-    if (threadIdx.x == 0) worst = fmax(worst, fabs(red[0] * 2.0 / OUT - mu[(int64_t)b * mu_ld + k]));
     __syncthreads();
   }
+  if (lane == 0) worst_w[warp] = worst;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    worst = fmax(fmax(worst_w[0], worst_w[1]), fmax(worst_w[2], worst_w[3]));
     flag[b] = worst > tol ? 1 : 0;
     if (dev) dev[b] = worst;
   }
@@ -520,11 +587,33 @@ int forward(kite_ctx* ctx, cudaStream_t st, const Net& net, const float* p32, in
 
 bool use_prior(const kite_mlp_prior* prior) { return prior && prior->kind == KITE_PRIOR_JACKSON; }
 
-void launch_prior(cudaStream_t st, int num_sms, const float* X, int rows, const kite_mlp_prior* prior, float* P) {
-  const double a = 0.5 * (prior->e_max - prior->e_min);
-  const int blocks = std::max(1, std::min(rows, num_sms * 8));
-  k_mlp_prior<<<blocks, 256, 0, st>>>(X, rows, prior_coef(), 1.0 / (3.141592653589793 * a), P);
+template <typename In>
+void launch_cheb_sum(cudaStream_t st, const In* src, int64_t ld, const int* idx, int rows, int M, const double* c,
+                     const double* T, double inv_pi_a, float* out) {
+  // 512 rows fill the SMs once with eight rows per block (4 column tiles of 64 row tiles)
+  if (rows >= 512) {
+    dim3 grid((rows + kSumRows - 1) / kSumRows, HALF / kSumTile);
+    k_mlp_cheb_sum<In, kSumRows><<<grid, kSumTile, 0, st>>>(src, ld, idx, rows, M, c, T, inv_pi_a, out);
+  } else {
+    dim3 grid(rows, HALF / kSumTile);
+    k_mlp_cheb_sum<In, 1><<<grid, kSumTile, 0, st>>>(src, ld, idx, rows, M, c, T, inv_pi_a, out);
+  }
 }
+
+// The residual prior of `rows` rows of X: c and T are the Jackson weights and the table of
+// order IN (prior_tables).
+void launch_prior(cudaStream_t st, const float* X, int rows, const kite_mlp_prior* prior, const double* c,
+                  const double* T, float* P) {
+  const double a = 0.5 * (prior->e_max - prior->e_min);
+  launch_cheb_sum(st, X, IN, nullptr, rows, IN, c, T, 1.0 / (3.141592653589793 * a), P);
+}
+
+// Jackson weights of order M (c [M]) and the table of order MT (T [MT][OUT/2]).
+void launch_tables(cudaStream_t st, int M, double* c, int MT, double* T) {
+  k_mlp_jackson<<<(M + 31) / 32, 32, 0, st>>>(M, c);
+  k_mlp_cheb<<<HALF / 32, 32, 0, st>>>(MT, T);
+}
+constexpr size_t kPriorFloats = 2 * ((size_t)IN + (size_t)IN * HALF);  // c and T of the prior
 
 // backward of the mean L1 loss over rows x OUT; gradient into net.grad.  Each product with
 // a transposed operand takes the transposes of activations, deltas or weights, so that
@@ -667,18 +756,21 @@ int mlp_forward_impl(kite_ctx* ctx, const float* params, const float* X, int n, 
   Net net;
   float* ex;
   const bool pri = use_prior(prior);
-  int rc = carve_net(ctx, std::min(n, chunk), &net, &ex, kParams + (pri ? (size_t)std::min(n, chunk) * OUT : 0));
+  int rc = carve_net(ctx, std::min(n, chunk), &net, &ex, kParams + (pri ? (size_t)std::min(n, chunk) * OUT + kPriorFloats : 0));
   if (rc != KITE_OK) return rc;
   cudaStream_t st = ctx->stream;
   if ((rc = clear_status(ctx)) != KITE_OK) return rc;
   KITE_CUDA_TRY(ctx, cudaMemcpyAsync(ex, params, sizeof(float) * kParams, cudaMemcpyDefault, st));
   k_mlp_tobf16<<<1024, 256, 0, st>>>(ex, net.pb, kParams);
+  static_assert(kParams % 2 == 0, "the tables that follow the parameters are FP64");
+  double* pc = reinterpret_cast<double*>(ex + kParams);
+  if (pri) launch_tables(st, IN, pc, IN, pc + IN);
   for (int r0 = 0; r0 < n; r0 += chunk) {
     const int rows = std::min(chunk, n - r0);
     k_mlp_gather<<<1024, 256, 0, st>>>(X + (int64_t)r0 * IN, nullptr, rows, IN, shift, scale, net.X, nullptr,
                                        nullptr, 0);
-    float* P = pri ? ex + kParams : nullptr;
-    if (pri) launch_prior(st, ctx->num_sms, X + (int64_t)r0 * IN, rows, prior, P);
+    float* P = pri ? ex + kParams + kPriorFloats : nullptr;
+    if (pri) launch_prior(st, X + (int64_t)r0 * IN, rows, prior, pc, pc + IN, P);
     rc = forward(ctx, st, net, ex, rows, P);
     if (rc != KITE_OK) return rc;
     KITE_CUDA_TRY(ctx, cudaMemcpyAsync(Y + (int64_t)r0 * OUT, net.Y, sizeof(float) * rows * OUT, cudaMemcpyDefault, st));
@@ -696,7 +788,7 @@ int mlp_train_impl(kite_ctx* ctx, const float* X, const float* T, int n, const f
   const bool pri = use_prior(prior);
   const size_t lsum_floats = 2 * (size_t)128 * ((n + bs - 1) / bs);  // FP64 partial sums of every step
   const size_t idx_floats = ((size_t)n + 63) / 64 * 64;
-  int rc = carve_net(ctx, bs, &net, &ex, 3 * kParams + lsum_floats + idx_floats + (pri ? (size_t)n * OUT : 0));
+  int rc = carve_net(ctx, bs, &net, &ex, 3 * kParams + lsum_floats + idx_floats + (pri ? (size_t)n * OUT + kPriorFloats : 0));
   if (rc != KITE_OK) return rc;
   cudaStream_t st = ctx->stream;
   float* p32 = ex;
@@ -705,9 +797,13 @@ int mlp_train_impl(kite_ctx* ctx, const float* X, const float* T, int n, const f
   double* lsum = reinterpret_cast<double*>(ex + 3 * kParams);
   int* d_idx = reinterpret_cast<int*>(ex + 3 * kParams + lsum_floats);
   // the prior of every training row, once; the batches gather T - prior as targets
-  float* P = pri ? ex + 3 * kParams + lsum_floats + idx_floats : nullptr;
+  double* pc = reinterpret_cast<double*>(ex + 3 * kParams + lsum_floats + idx_floats);
+  float* P = pri ? ex + 3 * kParams + lsum_floats + idx_floats + kPriorFloats : nullptr;
   if ((rc = clear_status(ctx)) != KITE_OK) return rc;
-  if (pri) launch_prior(st, ctx->num_sms, X, n, prior, P);
+  if (pri) {
+    launch_tables(st, IN, pc, IN, pc + IN);
+    launch_prior(st, X, n, prior, pc, pc + IN, P);
+  }
   KITE_CUDA_TRY(ctx, cudaMemcpyAsync(p32, params, sizeof(float) * kParams, cudaMemcpyDefault, st));
   KITE_CUDA_TRY(ctx, cudaMemsetAsync(m, 0, sizeof(float) * 2 * kParams, st));
   k_mlp_tobf16<<<1024, 256, 0, st>>>(p32, net.pb, kParams);
@@ -774,8 +870,30 @@ int mlp_narrow_impl(kite_ctx* ctx, const double* src, int K, float* dst) {
 
 int mlp_gate_impl(kite_ctx* ctx, const float* rho, const double* mu, int mu_ld, int n, int kcheck,
                   double de_minus, double tol, int* flags, double* dev) {
-  k_mlp_gate<<<n, 128, 0, ctx->stream>>>(rho, mu, mu_ld, kcheck, de_minus, tol, flags, dev);
-  KITE_CUDA_TRY(ctx, cudaGetLastError());
+  double* T = nullptr;
+  KITE_CUDA_TRY(ctx, cudaMallocAsync((void**)&T, sizeof(double) * (size_t)kcheck * HALF, ctx->stream));
+  k_mlp_cheb<<<HALF / 32, 32, 0, ctx->stream>>>(kcheck, T);
+  k_mlp_gate<<<n, 128, 0, ctx->stream>>>(rho, mu, mu_ld, kcheck, T, de_minus, tol, flags, dev);
+  const cudaError_t e = cudaGetLastError();
+  cudaFreeAsync(T, ctx->stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "consistency gate");
+  return KITE_OK;
+}
+
+// Jackson densities of order M on the output grid from the first M moments of `rows` rows of
+// mu [.][mu_ld] (row numbers idx, device), into the same rows of rho: the plain fallback of
+// every flagged row at once.
+int mlp_plain_impl(kite_ctx* ctx, const double* mu, int mu_ld, const int* idx, int rows, int M, double de_minus,
+                   float* rho) {
+  double* buf = nullptr;
+  KITE_CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, sizeof(double) * (size_t)M * (HALF + 1), ctx->stream));
+  double* T = buf;
+  double* c = buf + (size_t)M * HALF;
+  launch_tables(ctx->stream, M, c, M, T);
+  launch_cheb_sum(ctx->stream, mu, mu_ld, idx, rows, M, c, T, 1.0 / (3.141592653589793 * de_minus), rho);
+  const cudaError_t e = cudaGetLastError();
+  cudaFreeAsync(buf, ctx->stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "plain fallback");
   return KITE_OK;
 }
 

@@ -9,6 +9,7 @@
 // iterate; the accumulator becomes the next step's psi.  Bessel functions by Miller's
 // backward recurrence normalised with J_0 + 2 sum_k J_2k = 1.
 #include <math.h>
+#include <stdlib.h>
 
 #include <algorithm>
 #include <vector>
@@ -17,6 +18,7 @@
 #include "kite_internal.h"
 
 #include "kite_step.cuh"
+#include "kite_step2.cuh"
 
 namespace kite {
 
@@ -139,6 +141,46 @@ __global__ void k_extract64(int64_t ncell, const void* __restrict__ buf, int nve
   }
 }
 
+// Two recursion steps per pass (kite_step2.cuh) with the series: TERMS of r_{n-1} .. r_{n+2}
+// into the accumulator.  FP32 only (bound by the iterates' traffic; the FP64 steps are bound by
+// the FP64 pipe, which the pass's halo would load further), periodic, no field.  Honeycomb
+// 1024 x 1024, four packets, 81 terms, four time steps: 22.1 ms with a term per one-step
+// launch (five vector streams a step at 4.9 TB/s), 13.6 ms so (2.5 streams a step).
+constexpr int kSeriesStages = 6;
+template <typename Real, int LAT, int C, int TERMS>
+__global__ void __launch_bounds__(kBlock2, 3)
+    k_series2(const void* r_prev, const void* __restrict__ r_cur, void* out1, void* out2, const Real* __restrict__ vt,
+              Real tt, int Lx, int Ly, long long units, int* __restrict__ err, const Series2 ser) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int s_abort;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < kSeriesStages; ++k) mbar_init(&bars[k], 1);
+    mbar_fence_init();
+    s_abort = 0;
+  }
+  Ring ring{bars, smem + kBarBytes, &s_abort, 0};
+  griddep_wait();  // the previous launch's iterates and accumulator are complete
+  griddep_launch_dependents();
+  step2_body<Real, LAT, C, kSeriesStages, false, false, TERMS>(ring, blockIdx.x, gridDim.x, r_prev, r_cur, out1, out2,
+                                                                nullptr, vt, tt, Lx, Ly, units, nullptr, nullptr, err,
+                                                                0, nullptr, nullptr, &ser);
+}
+
+template <typename Real, int LAT, int C, int TERMS>
+int series2_occupancy() {
+  static int occ = -1;  // per template instance
+  if (occ < 0) {
+    int o = 0;
+    constexpr int SM = Step2Shape<LAT, C, kSeriesStages, false, false, TERMS>::SMEM;
+    cudaFuncSetAttribute(k_series2<Real, LAT, C, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_series2<Real, LAT, C, TERMS>, kBlock2, SM) != cudaSuccess)
+      o = 1;
+    occ = std::max(1, o);
+  }
+  return occ;
+}
+
 template <typename Real, int LAT, int C, bool FIELD>
 int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const Scale& sc, double dt,
                     int nsteps, double* psi, double* norms, kite_stats* stats) {
@@ -153,9 +195,16 @@ int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
   const long long units = (long long)((sys->Lx + Sh::TX - 1) / Sh::TX) * sys->Ly;
   const int G = grid_for<Real, LAT, C, false, 4, kStages, FIELD>(ctx, units);
   const int nb = (int)std::min<int64_t>((nchunk + 255) / 256, (int64_t)ctx->num_sms * 8);
+  // two steps per pass (its outputs never alias its inputs: two more buffers)
+  constexpr bool kPass = sizeof(Real) == 4 && !FIELD;
+  const char* pin = getenv("KITE_PASS_STEPS");
+  const bool pass = kPass && !sys->open_x && !sys->open_y && M >= 4 && !(pin && pin[0] == '1' && pin[1] == 0);
+  void *bC = nullptr, *bD = nullptr;
   Carver probe(nullptr);
   auto lay = [&](Carver& k, Real** vt, void** r0, void** bA, void** bB, void** acc, double** part,
                  unsigned long long** ne, Real** ph) {
+    bC = pass ? k.take<char>(vb) : nullptr;
+    bD = pass ? k.take<char>(vb) : nullptr;
     *vt = k.take<Real>(N);
     *ph = FIELD ? k.take<Real>((size_t)sys->Ly * SORB * 4) : nullptr;
     *r0 = k.take<char>(vb);
@@ -211,17 +260,49 @@ int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
     void* cur = r0;  // psi(t) in the batch layout
     void* nxt = acc;
     for (int k = 0; k < nsteps; ++k) {
-      auto where = [&](int n) -> void* { return n == 0 ? cur : ((n & 1) ? bA : bB); };
+      // iterate n >= 1 lives in bufs[n mod 4] (two buffers without the pass: r_{n+1} over r_{n-1})
+      void* bufs[4] = {pass ? bC : bB, bA, bB, pass ? bD : bA};
+      auto where = [&](int n) -> void* { return n == 0 ? cur : bufs[n & 3]; };
+      auto one_step = [&](int n) {  // r_{n+1} and its term
+        const SeriesOut so{nxt, coef[2 * (n + 1)], coef[2 * (n + 1) + 1]};
+        if (n == 0)
+          launch_pdl(k_step<Real, LAT, C, true, 4, kStages, FIELD>, G, kBlock, SM, st, nullptr, cur, where(1), nullptr,
+                     vt, tt, sys->Lx, sys->Ly, units, nullptr, nullptr, ctx->d_status, 0, FamOut{}, 0, so, ph, open);
+        else
+          launch_pdl(k_step<Real, LAT, C, false, 4, kStages, FIELD>, G, kBlock, SM, st, where(n - 1), where(n),
+                     where(n + 1), nullptr, vt, tt, sys->Lx, sys->Ly, units, nullptr, nullptr, ctx->d_status, 0,
+                     FamOut{}, 0, so, ph, open);
+        ++launches;
+      };
       k_series_init<Real><<<nb, 256, 0, st>>>(nchunk, cur, nxt, coef[0], coef[1]);
-      if (M >= 2)
-        k_step<Real, LAT, C, true, 4, kStages, FIELD><<<G, kBlock, SM, st>>>(
-            nullptr, cur, bA, nullptr, vt, tt, sys->Lx, sys->Ly, units, nullptr, nullptr, ctx->d_status, 0, FamOut{},
-            0, SeriesOut{nxt, coef[2], coef[3]}, ph, open);
-      for (int n = 1; n + 1 < M; ++n)
-        k_step<Real, LAT, C, false, 4, kStages, FIELD><<<G, kBlock, SM, st>>>(
-            where(n - 1), where(n), where(n + 1), nullptr, vt, tt, sys->Lx, sys->Ly, units, nullptr, nullptr,
-            ctx->d_status, 0, FamOut{}, 0, SeriesOut{nxt, coef[2 * (n + 1)], coef[2 * (n + 1) + 1]}, ph, open);
-      launches += std::max(0, M - 1);
+      if (M >= 2) one_step(0);
+      int n = 1;  // r_n is the newest iterate
+      if constexpr (kPass) {
+        // Every second pass adds the four terms it holds (its own two and, from its inputs, the
+        // pass's before), so the accumulator is read and written once per four steps: ten
+        // vector streams per four steps instead of twenty with a term per step.
+        auto two_steps = [&](auto terms) {
+          constexpr int TERMS = decltype(terms)::value;
+          Series2 se{nxt, {}};
+          for (int t = 0; t < 8; ++t) se.c[t] = coef[2 * (n - 1) + t];
+          const int G2 = (int)std::max(1LL, std::min((long long)ctx->num_sms * series2_occupancy<Real, LAT, C, TERMS>(),
+                                                     units));
+          launch_pdl(k_series2<Real, LAT, C, TERMS>, G2, kBlock2,
+                     Step2Shape<LAT, C, kSeriesStages, false, false, TERMS>::SMEM, st, where(n - 1), where(n),
+                     where(n + 1), where(n + 2), vt, tt, sys->Lx, sys->Ly, units, ctx->d_status, se);
+          n += 2;
+          ++launches;
+        };
+        while (pass && n + 2 <= M - 1) {
+          if (n + 4 <= M - 1) {
+            two_steps(std::integral_constant<int, 0>{});
+            two_steps(std::integral_constant<int, 4>{});
+          } else {
+            two_steps(std::integral_constant<int, 2>{});
+          }
+        }
+      }
+      for (; n + 1 < M; ++n) one_step(n);
       KITE_CUDA_TRY(ctx, cudaGetLastError());
       std::swap(cur, nxt);
       if (norms) {

@@ -521,8 +521,22 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
 #pragma unroll
           for (int q = 0; q < VPC; ++q) {
             const Real br = out.v[2 * q], bi = out.v[2 * q + 1];
-            a.v[2 * q] += cr * br - ci * bi;
-            a.v[2 * q + 1] += cr * bi + ci * br;
+            if constexpr (sizeof(Real) == 8) {
+              // the FP64 pipe bounds the step: multiply-adds only, and only those of nonzero parts
+              // (a symmetric window's coefficients are real or imaginary: two instead of six
+              // FP64 operations beside the stencil's eight)
+              if (cr != Real(0)) {
+                a.v[2 * q] = rfma(cr, br, a.v[2 * q]);
+                a.v[2 * q + 1] = rfma(cr, bi, a.v[2 * q + 1]);
+              }
+              if (ci != Real(0)) {
+                a.v[2 * q] = rfma(-ci, bi, a.v[2 * q]);
+                a.v[2 * q + 1] = rfma(ci, br, a.v[2 * q + 1]);
+              }
+            } else {
+              a.v[2 * q] += cr * br - ci * bi;
+              a.v[2 * q + 1] += cr * bi + ci * br;
+            }
           }
           a.st(ser.acc, qi);
         } else if constexpr (MODE == 3) {

@@ -27,13 +27,15 @@ namespace {
 // DBL: the moment-doubling pass (no r_0 staged; four moment slots per pass, their FP64
 // partials kept in shared memory: kBlock threads x 4 slots x 4 doubles at most).  SMACC:
 // the plain pass with its two FP64 partials in shared memory as well (fewer registers, for
-// the persistent batched kernel).
-template <int LAT, int C, int NST, bool DBL = false, bool SMACC = false>
+// the persistent batched kernel).  SER >= 0: the Chebyshev-series pass (time evolution): no
+// moments and no r_0; SER of the terms r_{n-1} .. r_{n+2}, the last ones, are added to an
+// accumulator.
+template <int LAT, int C, int NST, bool DBL = false, bool SMACC = false, int SER = -1>
 struct Step2Shape {
   using S1 = StepShape<LAT, C, NST>;
   static constexpr int SORB = S1::SORB, TPC = S1::TPC, TX = S1::TX, CELLB = S1::CELLB;
   static constexpr int RNB = (TX + 4) * CELLB;  // r_n row, two halo cells each side
-  static constexpr int R0B = DBL ? 0 : TX * CELLB;  // r_0 row
+  static constexpr int R0B = (DBL || SER >= 0) ? 0 : TX * CELLB;  // r_0 row
   static constexpr int STAGEB = RNB + R0B;      // (r_{n-1} is read once per site: registers)
   static constexpr int TILEB = (TX + 2) * CELLB;  // one r_{n+1} row of the tile ring
   static constexpr int DACCB = (DBL ? 4 : (SMACC ? 2 : 0)) * kBlock * 4 * 8;
@@ -46,20 +48,28 @@ struct Step2Shape {
 // compute warps carry equal work between the barriers.
 constexpr int kBlock2 = kBlock + 32;
 
+// Accumulator of the series pass, in the batch layout, and the coefficients (re, im) of its
+// four terms r_{n-1}, r_n, r_{n+1}, r_{n+2}.
+struct Series2 {
+  void* acc;
+  double c[8];
+};
+
 // Plain moments: partial1 <- <r_0|r_{n+1}>, partial2 <- <r_0|r_{n+2}>.  DBL (moment doubling,
 // the slots of k_undouble): partial1 <- <r_n|r_n>, partial2 <- <r_n|r_{n+1}>, partial3 <-
 // <r_{n+1}|r_{n+1}>, partial4 <- <r_{n+1}|r_{n+2}> (slots 2n .. 2n+3); r0 is not read.
-template <typename Real, int LAT, int C, int NST, bool DBL = false, bool SMACC = false>
+template <typename Real, int LAT, int C, int NST, bool DBL = false, bool SMACC = false, int SER = -1>
 __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const void* __restrict__ r_prev,
                                            const void* __restrict__ r_cur, void* __restrict__ out1,
                                            void* __restrict__ out2, const void* __restrict__ r0,
                                            const Real* __restrict__ vt, Real tt, int Lx, int Ly, long long units,
                                            double* __restrict__ partial1, double* __restrict__ partial2,
                                            int* __restrict__ err, int realv, double* __restrict__ partial3 = nullptr,
-                                           double* __restrict__ partial4 = nullptr) {
+                                           double* __restrict__ partial4 = nullptr, const Series2* ser = nullptr) {
+  static_assert(SER < 0 || (!DBL && !SMACC && (SER == 0 || SER == 2 || SER == 4)), "series pass: 0, 2 or 4 terms");
   using Ch = Chunk<Real>;
   using Acc = typename AccT<Real>::T;
-  using Sh = Step2Shape<LAT, C, NST, DBL, SMACC>;
+  using Sh = Step2Shape<LAT, C, NST, DBL, SMACC, SER>;
   constexpr bool SMEMSUMS = DBL || SMACC;  // FP64 partials in shared memory
   const Real tt2 = tt + tt;  // exact; the on-site terms vt hold 2 V~
   constexpr int VPC = Ch::kVecs, NR = Ch::kReals;
@@ -146,7 +156,7 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
       int row = yb - 2 + jj;
       while (row < 0) row += Ly;
       while (row >= Ly) row -= Ly;
-      const bool need_r0 = !DBL && jj >= 2 && jj <= nr + 1;  // owned rows
+      const bool need_r0 = !DBL && SER < 0 && jj >= 2 && jj <= nr + 1;  // owned rows
       const uint32_t bytes = (uint32_t)(txv + 4) * CELLB + (need_r0 ? (uint32_t)txv * CELLB : 0u);
       mbar_arrive_expect_tx(&bars[st], bytes);
       const size_t roff = (size_t)row * Lx * CELLB;
@@ -320,6 +330,13 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
     const unsigned char* pp = static_cast<const unsigned char*>(r_prev) + pcol * 16 + (size_t)yb * orowb;
     const Real* pvt = vcol + (size_t)yb * vrow;
     const long long ly_orowb = (long long)Ly * orowb, ly_vrow = (long long)Ly * vrow;
+    // series pass: the accumulator's row yb-3+i, loaded one row ahead, and r_{n-1} of the rows of
+    // iterations i-1, i-2
+    unsigned char* pa = nullptr;
+    if constexpr (SER > 0)
+      pa = static_cast<unsigned char*>(ser->acc) + (long long)(ocol * 16) + (long long)(yb - 3) * orowb;
+    Ch anext{}, pvm1{}, pvm2{};
+    (void)pa, (void)anext, (void)pvm1, (void)pvm2;
     // One barrier per row: iteration i computes r_{n+1} row yb-1+i (slots i, i+1, i+2 hold
     // r_n rows yb-2+i .. yb+i) into tile row i mod 4, and r_{n+2} row yb-3+i from the three
     // tile rows written by the previous iterations, with r_n and r_0 of that row from slot
@@ -360,7 +377,9 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
         *reinterpret_cast<Ch*>(t3 + (xl + 1) * CELLB + choff) = o;
         if (i >= 1 && i <= nr) {
           o.st(po1, 0);
-          if constexpr (DBL) {
+          if constexpr (SER >= 0) {
+            // (no moments)
+          } else if constexpr (DBL) {
             const Ch me = *reinterpret_cast<const Ch*>(mid + (xl + 2) * CELLB + choff);  // r_n
             accumulate_dbl(facc1, gacc1, rows1, 0, 1, me, o);
           } else {
@@ -379,7 +398,28 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
         const unsigned char* prev = stages + stm * Sh::STAGEB;
         const Ch o = site2(tile + o0, tile + o1, tile + o2, prev, vm2);
         o.st(po2, 0);
-        if constexpr (DBL) {
+        if constexpr (SER >= 0) {
+          if constexpr (SER > 0) {
+            // term by term, as one step at a time adds them (the same bits)
+            Ch a = anext;
+            auto add = [&](const Ch& r, int t) {
+              const Real cr = (Real)ser->c[2 * t], ci = (Real)ser->c[2 * t + 1];
+#pragma unroll
+              for (int q = 0; q < VPC; ++q) {
+                const Real br = r.v[2 * q], bi = r.v[2 * q + 1];
+                a.v[2 * q] += cr * br - ci * bi;
+                a.v[2 * q + 1] += cr * bi + ci * br;
+              }
+            };
+            if constexpr (SER == 4) {
+              add(pvm2, 0);
+              add(*reinterpret_cast<const Ch*>(prev + (xl + 2) * CELLB + choff), 1);
+            }
+            add(*reinterpret_cast<const Ch*>(tile + o1 + (xl + 1) * CELLB + choff), 2);
+            add(o, 3);
+            a.st(pa, 0);
+          }
+        } else if constexpr (DBL) {
           const Ch me = *reinterpret_cast<const Ch*>(tile + o1 + (xl + 1) * CELLB + choff);  // r_{n+1}
           accumulate_dbl(facc2, gacc2, rows2, 2, 3, me, o);
         } else {
@@ -387,6 +427,14 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
           if constexpr (SMACC) accumulate_sm(facc2, rows2, 1, z0, o);
           else accumulate(facc2, dacc2, rows2, z0, o);
         }
+      }
+      if constexpr (SER > 0) {
+        if (active && i >= 2 && i + 1 < nr + 3) anext = Ch::ld(pa + orowb, 0);  // row yb-3+(i+1)
+        pa += orowb;
+      }
+      if constexpr (SER == 4) {
+        pvm2 = pvm1;
+        pvm1 = pv1;
       }
       vm2 = vm1;
       vm1 = v1;
@@ -437,6 +485,7 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
     u += nr;
   }
   ring.gslot = gslot;
+  if constexpr (SER >= 0) return true;
   // partial1 <- <r_0|r_{n+1}>, partial2 <- <r_0|r_{n+2}>: fixed-order sums over the compute
   // threads holding each chunk, as in the one-step kernel (the ring is drained; its
   // memory is reused)

@@ -256,7 +256,7 @@ int kite_flux_nearest(const kite_system* sys, double flux, double* out);
  * moment, which vanishes for a real symmetric H~, is then not formed and reads 0.
  * KITE_CLUSTER=0 / 1 in the environment forbids / forces it.
  * A mid-size lattice (two iterates of a batch of vectors fit the GPU's shared memory: up
- * to about a million orbitals) may run the sweep on chip as well, one region of the
+ * to about 1.5 million orbitals in FP32) may run the sweep on chip as well, one region of the
  * lattice per SM in one cooperative launch whose CTAs wait on their neighbours within a
  * bound; it keeps the streaming launch's grouping of the FP32 moment sums.  Chosen where
  * measured faster; KITE_RESIDENT=0 / 1 forbids / forces it.  If a wait runs out (its SMs held

@@ -17,7 +17,8 @@ namespace kite {
 struct ResidentPlan {
   int TX, G;          // strip width, virtual CTAs: how the moment sums are grouped
   int regions, rows, nv, nfl, r0_rows;
-  int CR;             // 16-byte chunks per orbital and sweep (0: the lattice does not fit)
+  int cby, vecs;      // the sweep's unit: bytes (16-byte chunk or half of one) and vectors
+  int CR;             // units per orbital and sweep (0: the lattice does not fit)
   int T, levels, smem;
 };
 }  // namespace kite
@@ -158,13 +159,13 @@ int cluster_sweep(kite_ctx* ctx, ClusterSweep* a, int timing_steps);
 // The 1D sweep of a mid-size lattice held on chip by the whole GPU, a region of the lattice
 // per SM (kite_resident.cu).
 ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, int realv, int field, int Lx, int Ly,
-                           int C, int M, int TX, long long G);
+                           int C, int M, int TX, long long G, int cby = 16);
 ResidentPlan resident_plan_free(kite_ctx* ctx, int lattice, int doubling, int realv, int field, int Lx, int Ly, int C,
                                 int M);
-int resident_max_chunks(kite_ctx* ctx, int lattice, int Lx, int Ly, int C);
-// Bytes of the edge records the regions exchange, and (at most) of the moment partials.
-size_t resident_rec_bytes(int lattice, int Lx, int Ly, int CR);
-size_t resident_part_bytes(kite_ctx* ctx, int fp64, int realv, int C, int slots);
+// Most bytes any plan of the lattice needs for the edge records and, for `slots` moments, the
+// moment partials (0: none fits).
+void resident_space(kite_ctx* ctx, int fp64, int lattice, int realv, int Lx, int Ly, int C, int slots, size_t* rec,
+                    size_t* part);
 struct ResidentSweep {
   ResidentPlan plan;
   int fp64, lattice, doubling, realv;
@@ -178,7 +179,7 @@ struct ResidentSweep {
   double tt;
   void *bA, *bB;      // odd and even iterates: the last two when wanted
   double* part;
-  void* rec;          // edge records, resident_rec_bytes
+  void* rec;          // edge records, resident_space
   const unsigned long long* n_eff;
   double* mu_vec;
   // outputs

@@ -727,7 +727,7 @@ constexpr size_t kResidentPartMax = (size_t)2 << 30;
 // Whether to run the batch resident.  `other_ms` times the kernels chosen otherwise, per
 // recursion step of the batch.
 template <typename OtherMs>
-bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, int per_chunk, OtherMs other_ms) {
+bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
   if (resident_pinned() == 2) return true;
   uint64_t key = 0x6b697465726573ull;
   for (uint64_t f : {(uint64_t)r.fp64, (uint64_t)r.lattice, (uint64_t)r.doubling, (uint64_t)r.realv,
@@ -748,7 +748,7 @@ bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, int per_chunk, Other
     return best;
   };
   const double t8 = timed(8), t40 = timed(kClusterTimeSteps);
-  const int sweeps = ((r.nvec + per_chunk - 1) / per_chunk + r.plan.CR - 1) / r.plan.CR;
+  const int per_sweep = r.plan.CR * r.plan.vecs, sweeps = (r.nvec + per_sweep - 1) / per_sweep;
   const float ms = (float)(1e3 * std::max(0.0, t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
   const int pick = ms < 0.95f * other_ms() ? 1 : 0;  // it must win clearly
   cudaGetLastError();
@@ -815,14 +815,10 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
           : cluster_part_doubles(p.realv ? p.max_batch : 2 * p.max_batch, 16, p.M, p.doubling, kClusterTimeSteps);
   // the resident sweep's moment partials and edge records, where the lattice may fit on chip
   size_t resident_part = 0, resident_rec = 0;
-  if (allow_resident && resident_pinned() != 1 && p.M >= 4) {
-    const int cr = resident_max_chunks(ctx, LAT, p.Lx, p.Ly, Cmax);
-    if (cr >= 1) {
-      resident_part = resident_part_bytes(ctx, sizeof(Real) == 8, p.realv, cr, std::max(p.M + 1, 2 * kClusterTimeSteps + 2));
-      resident_rec = resident_rec_bytes(LAT, p.Lx, p.Ly, cr);
-    }
-    if (resident_part > kResidentPartMax) resident_part = resident_rec = 0;
-  }
+  if (allow_resident && resident_pinned() != 1 && p.M >= 4)
+    resident_space(ctx, sizeof(Real) == 8, LAT, p.realv, p.Lx, p.Ly, Cmax, std::max(p.M + 1, 2 * kClusterTimeSteps + 2),
+                   &resident_rec, &resident_part);
+  if (resident_part > kResidentPartMax) resident_part = resident_rec = 0;
   // FP32 moment sums keep the grouping of the streaming launch (strips of TX cells, grid G);
   // FP64 sums may be grouped freely
   auto resident_for = [&](int C, int G) {
@@ -1113,7 +1109,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
                                                                    cluster_pinned() != 2));
       if (may_reside && (sizeof(Real) == 8 || cl.cs == 0 || pinned_res))
         rs.plan = resident_for(C, sizeof(Real) == 8 ? 0 : (p.field ? fs.G : tuned_grid()));
-      if (rs.plan.CR && resident_choice(ctx, rs, per_chunk, other_ms)) {
+      if (rs.plan.CR && resident_choice(ctx, rs, other_ms)) {
         // mid-size lattice: the whole sweep on chip, a region per SM (kite_resident.cu)
         rs.stall = ctx->debug_stall;
         ctx->debug_stall = 0;

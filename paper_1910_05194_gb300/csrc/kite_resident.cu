@@ -9,13 +9,14 @@
 // on-site terms beside them; r_0 as far as it fits, the rest of it is read from L2.  r_{n+1}
 // overwrites r_{n-1} in place.
 //
-// Per step the compute threads (one per column of a virtual CTA, sublattice and 16-byte
-// chunk) march down their rows with the next row's operands in flight, while 256 exchange
+// Per step the compute threads (one per column of a virtual CTA, sublattice and unit of a
+// sweep's vectors) march down their rows with the next row's operands in flight, while 256 exchange
 // threads (1) compute the region's edge sites once more, with their r_{n-1} in registers, and
 // send them at once, (2) add up the moment partials of the step before, (3) receive the
-// neighbours' edge sites into the frame.  The exchange's latency thus lies beside the march.  No grid-wide barrier and no fence: a
-// 16-byte chunk travels as four 8-byte words of 32 data bits and the 32-bit step number, so a
-// word that carries the step's number carries its data (8-byte accesses are single copies).
+// neighbours' edge sites into the frame.  The exchange's latency thus lies beside the march.
+// No grid-wide barrier and no fence: a unit travels as 8-byte words of 32 data bits and the
+// 32-bit step number, so a word that carries the step's number carries its data (8-byte
+// accesses are single copies).
 // The records are double-buffered by step parity: a region sends r_{n+1} only after it has
 // received all of its neighbours' r_n, which they sent after they had received r_{n-1}, so
 // the record that r_{n+1} overwrites has been read.  (A flag per region behind a release
@@ -32,8 +33,11 @@
 // poll) beside it.  Per recursion step of the batch, against the streaming kernels' launch,
 // ring fill and CTA reduction per step: honeycomb 257 x 510, R = 8 FP32 14.6 -> 5.0 us (two
 // sweeps of four vectors), 512 x 601 in a field, R = 4 17.4 -> 5.9 us, 300 x 300, R = 8
-// 11.4 -> 3.8 us; 64 x 64, R = 4 FP64 1.6-1.9 us against the cluster sweep's 2.2 us.  Which
-// runs is measured (resident_choice in kite_kpm1d.cu).
+// 11.4 -> 3.8 us; 64 x 64, R = 4 FP64 1.6-1.9 us against the cluster sweep's 2.2 us.  In units
+// of one complex FP32 vector, orbital updates per second: square 1024 x 1024, R = 4
+// 1.94e11 -> 4.65e11, R = 8 2.36e11 -> 3.77e11, 957 x 957, R = 4 1.78e11 -> 4.31e11, 1200 x 1200
+// 1.95e11 -> 2.55e11 (r_0 from L2), honeycomb 800 x 800 2.04e11 -> 2.45e11.  Which runs is
+// measured (resident_choice in kite_kpm1d.cu).
 #include <math.h>
 
 #include <algorithm>
@@ -49,48 +53,87 @@ namespace {
 
 constexpr int kRMax = 256;     // most compute threads of a CTA (512 threads: 128 registers each)
 constexpr int kRComm = 256;    // exchange threads
-constexpr int kRSites = 2;     // most edge sites, and most halo chunks, of one exchange thread
+constexpr int kRSites = 3;     // most edge sites, and most halo chunks, of one exchange thread
 constexpr int kRMaxV = 64;     // most virtual CTAs of a region
 constexpr int kRFlush = 32;    // rows of one FP32 moment sum (the streaming kernels' kFlushRows)
 constexpr int kResSmem = 227 * 1024 - 512;  // (the rest: static shared memory)
 
-// One record: 16 bytes of data as four 8-byte words of (data, step number), moved by one
-// 32-byte access.
-struct alignas(32) Rec {
-  unsigned long long w[4];
+// The unit of a sweep's vectors: a 16-byte chunk of the batch layout (two complex FP32 or one
+// complex FP64 vector), or half of one in FP32.  Half chunks let lattices of twice the size
+// stay on chip, one complex vector per sweep.
+struct alignas(8) HalfChunk {
+  static constexpr int kReals = 2;
+  static constexpr int kVecs = 1;
+  float v[2];
+  __device__ __forceinline__ static HalfChunk ldg(const void* base, size_t idx) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(base) + idx);
+    HalfChunk c;
+    c.v[0] = t.x;
+    c.v[1] = t.y;
+    return c;
+  }
+  __device__ __forceinline__ void st(void* base, size_t idx) const {
+    reinterpret_cast<float2*>(base)[idx] = make_float2(v[0], v[1]);
+  }
 };
-__device__ __forceinline__ void send_rec(Rec* p, const uint4& d, uint32_t step) {
+template <typename Real, int CBY>
+struct ResUnit {
+  using T = Chunk<Real>;
+};
+template <>
+struct ResUnit<float, 8> {
+  using T = HalfChunk;
+};
+
+// One record: a unit's data as 8-byte words of (32 data bits, step number), moved by one
+// 32-byte (half chunks: 16-byte) access.
+template <int W>
+struct alignas(8 * W) Rec {
+  unsigned long long w[W];
+};
+template <int W>
+__device__ __forceinline__ void send_rec(Rec<W>* p, const uint32_t (&d)[W], uint32_t step) {
   const unsigned long long h = (unsigned long long)step << 32;
-  asm volatile("st.relaxed.gpu.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(h | d.x), "l"(h | d.y),
-               "l"(h | d.z), "l"(h | d.w)
-               : "memory");
+  if constexpr (W == 4)
+    asm volatile("st.relaxed.gpu.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(h | d[0]), "l"(h | d[1]),
+                 "l"(h | d[2]), "l"(h | d[3])
+                 : "memory");
+  else
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(h | d[0]), "l"(h | d[1]) : "memory");
 }
-__device__ __forceinline__ Rec load_rec(const Rec* p) {
-  Rec r;
-  asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
-               : "=l"(r.w[0]), "=l"(r.w[1]), "=l"(r.w[2]), "=l"(r.w[3])
-               : "l"(p)
-               : "memory");
+template <int W>
+__device__ __forceinline__ Rec<W> load_rec(const Rec<W>* p) {
+  Rec<W> r;
+  if constexpr (W == 4)
+    asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(r.w[0]), "=l"(r.w[1]), "=l"(r.w[2]), "=l"(r.w[3])
+                 : "l"(p)
+                 : "memory");
+  else
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(r.w[0]), "=l"(r.w[1]) : "l"(p) : "memory");
   return r;
 }
-__device__ __forceinline__ bool rec_ready(const Rec& r, uint32_t step) {
-  return (uint32_t)(r.w[0] >> 32) == step && (uint32_t)(r.w[1] >> 32) == step && (uint32_t)(r.w[2] >> 32) == step &&
-         (uint32_t)(r.w[3] >> 32) == step;
+template <int W>
+__device__ __forceinline__ bool rec_ready(const Rec<W>& r, uint32_t step) {
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < W; ++i) ok = ok && (uint32_t)(r.w[i] >> 32) == step;
+  return ok;
 }
 
 template <typename Real>
 struct ResArgs {
-  const void* r0;     // batch layout [cell][sublattice][C chunks]
+  const void* r0;     // batch layout [cell][sublattice][C units]
   const Real* vt;     // 2 V~ per orbital, NaN on vacancies
   const Real* phase;  // [Ly][sublattice][2][2] (cos, sin), field only
   void* last[2];      // r_last: the last two iterates in the batch layout, r_n in last[n & 1]
   double* part;       // moment partials [slot n][CTA][exchange warps][32 >> levels]
-  Rec* rec;           // edge records [parity][cell][sublattice][CR chunks]
+  void* rec;          // edge records [parity][cell][sublattice][CR units]
   int* err;
   Real tt;
   int Lx, Ly, TX, G;  // strip width, virtual CTAs
   int rows_max, nv_max, nfl, r0_rows, levels;
-  int C, c0, CR;      // chunks per orbital of the batch, first chunk and chunks of this sweep
+  int C, c0, CR;      // units per orbital of the batch, first unit and units of this sweep
   int steps, open_x, open_y, stall;
   int write_last;
 };
@@ -99,10 +142,10 @@ struct ResArgs {
 struct ResSmem {
   int x0, x1, r0, vt, phase, sums, total;
 };
-__host__ __device__ inline ResSmem res_smem(int sorb, int CR, int TX, int rows, int nv, int nfl, int real_bytes,
+__host__ __device__ inline ResSmem res_smem(int cby, int sorb, int CR, int TX, int rows, int nv, int nfl, int real_bytes,
                                             int nsums, int dbl, int r0_rows, int field) {
   ResSmem s;
-  const int cellb = sorb * CR * 16, frame = (rows + 4) * (TX + 2);
+  const int cellb = sorb * CR * cby, frame = (rows + 4) * (TX + 2);
   int off = 0;
   auto take = [&](int bytes) {
     const int at = off;
@@ -120,9 +163,10 @@ __host__ __device__ inline ResSmem res_smem(int sorb, int CR, int TX, int rows, 
 }
 
 // VAR 0: complex vectors, 1: complex vectors in a magnetic field, 2: real vectors.
-template <typename Real, int LAT, bool DBL, int VAR>
+template <typename Real, int CBY, int LAT, bool DBL, int VAR>
 __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Real> a) {
-  using Ch = Chunk<Real>;
+  using Ch = typename ResUnit<Real, CBY>::T;
+  constexpr int W = CBY / 4;  // words of a record
   constexpr int SORB = LAT == KITE_HONEYCOMB ? 2 : 1;
   constexpr int NR = Ch::kReals, VPC = Ch::kVecs;
   constexpr bool IM = sizeof(Real) == 4 && VAR != 2;          // real and imaginary parts
@@ -133,11 +177,11 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
   const int T = (int)blockDim.x - kRComm;  // compute threads
   const int tid = threadIdx.x, cta = blockIdx.x;
   const int CR = a.CR, TPC = SORB * CR, TX = a.TX, colT = TX * TPC;
-  const ResSmem sm = res_smem(SORB, CR, TX, a.rows_max, a.nv_max, a.nfl, (int)sizeof(Real), NV, DBL, a.r0_rows,
+  const ResSmem sm = res_smem(CBY, SORB, CR, TX, a.rows_max, a.nv_max, a.nfl, (int)sizeof(Real), NV, DBL, a.r0_rows,
                               VAR == 1);
   // r_n and r_{n-1} are kept by sublattice, [sublattice][framed cell][chunk]: a warp's lanes
   // hold one sublattice of a row (where a row of TX * CR chunks fills whole warps)
-  const int P = TX + 2, CB = CR * 16, PB = P * CB;   // framed row; bytes of a cell, of a framed row
+  const int P = TX + 2, CB = CR * CBY, PB = P * CB;   // framed row; bytes of a cell, of a framed row
   const int PS = (a.rows_max + 4) * PB;              // bytes of a sublattice
   // the region: virtual CTAs v0 .. v1-1, units U0 .. U0+nrows-1, in one or two segments
   const long long units = (long long)((a.Lx + TX - 1) / TX) * a.Ly;
@@ -185,7 +229,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       const int f = i / TPC, k = i - f * TPC;
       const int ly = f / w - 1, lx = f - (ly + 1) * w - 1;
       const int s = k / CR, c = k - s * CR;
-      const int at = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+      const int at = s * PS + frame_cell(g, lx, ly) * CB + c * CBY;
       const int q = lattice_cell(g, lx, ly);
       Ch z, r;
 #pragma unroll
@@ -290,7 +334,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
           }
           e_on |= 1u << u;
           e_s |= (unsigned)s << u;
-          e_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+          e_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * CBY;
           e_row[u] = base + ly;
           e_v[u] = vts[(s * a.rows_max + base + ly) * TX + lx];
           e_rec[u] = (unsigned)((lattice_cell(g, lx, ly) * SORB + s) * CR + c);
@@ -319,7 +363,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
           const int q = lattice_cell(g, lx, ly);
           if (q < 0) continue;
           h_on |= 1u << u;
-          h_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * 16;
+          h_off[u] = s * PS + frame_cell(g, lx, ly) * CB + c * CBY;
           h_rec[u] = (unsigned)((q * SORB + s) * CR + c);
         }
         hoff += hlen;
@@ -329,7 +373,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
     const bool mute = a.stall && cta == 0;
     auto send_edges = [&](int n, auto first_tag) {
       const unsigned char* cur = xb + (n & 1) * xd;
-      Rec* dst = a.rec + ((n + 1) & 1) * half;
+      Rec<W>* dst = static_cast<Rec<W>*>(a.rec) + ((n + 1) & 1) * half;
 #pragma unroll
       for (int u = 0; u < kRSites; ++u) {
         if (!(e_on >> u & 1)) continue;
@@ -341,7 +385,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
         const Ch out = update(first_tag, ld(p + nb.o1), ld(p + nb.o2), ld(p + nb.o3), n4, me, e_prev[u], e_v[u],
                               phs + (e_row[u] * SORB + (int)(e_s >> u & 1)) * 4);
         e_prev[u] = me;
-        if (!mute) send_rec(dst + e_rec[u], *reinterpret_cast<const uint4*>(&out), (uint32_t)(n + 1));
+        if (!mute) send_rec<W>(dst + e_rec[u], *reinterpret_cast<const uint32_t(*)[W]>(&out), (uint32_t)(n + 1));
       }
     };
     // FP64 sums of step n's partials: each thread every kRComm-th entry (its own (chunk, sum)
@@ -370,19 +414,22 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       if (n + 1 < a.steps) {
         const uint32_t step = (uint32_t)(n + 1);
         unsigned char* nxt = xb + ((n + 1) & 1) * xd;
-        const Rec* src = a.rec + ((n + 1) & 1) * half;
+        const Rec<W>* src = static_cast<const Rec<W>*>(a.rec) + ((n + 1) & 1) * half;
         unsigned want = h_on;
         const long long t0 = clock64();
         while (want) {
-          Rec d[kRSites];
+          Rec<W> d[kRSites];
 #pragma unroll
           for (int u = 0; u < kRSites; ++u)
             if (want >> u & 1) d[u] = load_rec(src + h_rec[u]);
 #pragma unroll
           for (int u = 0; u < kRSites; ++u)
             if ((want >> u & 1) && rec_ready(d[u], step)) {
-              *reinterpret_cast<uint4*>(nxt + h_off[u]) =
-                  make_uint4((uint32_t)d[u].w[0], (uint32_t)d[u].w[1], (uint32_t)d[u].w[2], (uint32_t)d[u].w[3]);
+              Ch x;
+              uint32_t(&xw)[W] = *reinterpret_cast<uint32_t(*)[W]>(&x);
+#pragma unroll
+              for (int i = 0; i < W; ++i) xw[i] = (uint32_t)d[u].w[i];
+              *reinterpret_cast<Ch*>(nxt + h_off[u]) = x;
               want &= ~(1u << u);
             }
           if (want && clock64() - t0 > kWaitCycles) {
@@ -428,7 +475,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       };
       for (int r = s_vrow[j]; r < re; ++r) {
         if (!(r < nr0 ? tx_on0 : tx_on1)) continue;
-        const Ch me = ld(xb + s * PS + (frame_row(r) * P + xl + 1) * CB + c * 16);
+        const Ch me = ld(xb + s * PS + (frame_row(r) * P + xl + 1) * CB + c * CBY);
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
           const int v = IM ? q >> 1 : q;
@@ -460,7 +507,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
   auto march = [&](auto first_tag, auto s_tag, const unsigned char* cur, unsigned char* nxt, int g, int r, int rend) {
     constexpr bool FIRST = decltype(first_tag)::value;
     constexpr int S = decltype(s_tag)::value;
-    int at = s * PS + (frame_row(r) * P + xl + 1) * CB + c * 16;
+    int at = s * PS + (frame_row(r) * P + xl + 1) * CB + c * CBY;
     const Real* pv_v = vts + (s * a.rows_max + r) * TX + xl;
     const Ch* pr = reinterpret_cast<const Ch*>(smem + sm.r0) + ((s * a.r0_rows + r) * TX + xl) * CR + c;
     size_t gq = (((size_t)row_y(r) * a.Lx + (sx + g) * TX + xl) * SORB + s) * a.C + a.c0 + c;
@@ -587,7 +634,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       const int r = i / colT, kk = i - r * colT, ss = kk / (TX * CR), lx = (kk - ss * TX * CR) / CR, q = kk % CR;
       const int g = r < nr0 ? 0 : 1;
       if (lx >= seg_tx(g)) continue;
-      const int at = ss * PS + (frame_row(r) * P + lx + 1) * CB + q * 16;
+      const int at = ss * PS + (frame_row(r) * P + lx + 1) * CB + q * CBY;
       const size_t o = (((size_t)row_y(r) * a.Lx + (sx + g) * TX + lx) * SORB + ss) * a.C + a.c0 + q;
       for (int b = 0; b < 2; ++b) ld(xb + b * xd + at).st(a.last[b], o);
     }
@@ -621,29 +668,33 @@ __global__ void __launch_bounds__(256) k_resident_reduce(const double* __restric
   }
 }
 
-template <typename Real, int LAT, bool DBL>
+template <typename Real, int CBY, int LAT, bool DBL>
 const void* res_kernel_var(int var) {
-  return var == 0   ? reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 0>)
-         : var == 1 ? reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 1>)
-                    : reinterpret_cast<const void*>(&k_resident<Real, LAT, DBL, 2>);
+  return var == 0   ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 0>)
+         : var == 1 ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 1>)
+                    : reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 2>);
 }
-template <typename Real>
+template <typename Real, int CBY>
 const void* res_kernel(int lattice, int dbl, int var) {
   if (lattice == KITE_HONEYCOMB)
-    return dbl ? res_kernel_var<Real, KITE_HONEYCOMB, true>(var) : res_kernel_var<Real, KITE_HONEYCOMB, false>(var);
-  return dbl ? res_kernel_var<Real, KITE_SQUARE, true>(var) : res_kernel_var<Real, KITE_SQUARE, false>(var);
+    return dbl ? res_kernel_var<Real, CBY, KITE_HONEYCOMB, true>(var)
+               : res_kernel_var<Real, CBY, KITE_HONEYCOMB, false>(var);
+  return dbl ? res_kernel_var<Real, CBY, KITE_SQUARE, true>(var) : res_kernel_var<Real, CBY, KITE_SQUARE, false>(var);
 }
 
-int per_chunk_of(int fp64, int realv) { return fp64 ? (realv ? 2 : 1) : (realv ? 4 : 2); }  // vectors
-int sums_of(int fp64, int realv) { return fp64 ? (realv ? 2 : 1) : 4; }                      // moment sums
+// Vectors and moment sums (real and imaginary part in FP32) of a unit of cby bytes.
+int vectors_of(int fp64, int realv, int cby) { return (fp64 ? 1 : cby / 8) * (realv ? 2 : 1); }
+int sums_of(int fp64, int realv, int cby) { return fp64 ? (realv ? 2 : 1) : cby / 4; }
 
 }  // namespace
 
-// The regions for strips of TX cells and G virtual CTAs, and the chunks per sweep: as many as
-// fit on chip (fewer sweeps), with as many rows of r_0 as fit beside them.  CR = 0: no fit.
+// The regions for strips of TX cells and G virtual CTAs, and the units per sweep of a batch of
+// C 16-byte chunks: as many as fit on chip (fewer sweeps), with as many rows of r_0 as fit
+// beside them; half chunks only where no whole one fits.  CR = 0: no fit.
 ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, int realv, int field, int Lx, int Ly,
-                           int C, int M, int TX, long long G) {
+                           int C, int M, int TX, long long G, int cby) {
   ResidentPlan p{};
+  C *= 16 / cby;
   const int sorb = lattice == KITE_HONEYCOMB ? 2 : 1, real = fp64 ? 8 : 4;
   const int nstrips = (Lx + TX - 1) / TX;
   const long long units = (long long)nstrips * Ly;
@@ -665,13 +716,15 @@ ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, i
   for (int cr = C; cr >= 1; cr >>= 1) {
     const int colT = TX * sorb * cr;
     if (colT > kRMax || edge * cr > kRSites * kRComm) continue;
-    const int per = sums_of(fp64, realv);
+    const int per = sums_of(fp64, realv, cby);
     auto need = [&](int r0_rows) {
-      return res_smem(sorb, cr, TX, rows, nv, p.nfl, real, per, doubling, r0_rows, field).total;
+      return res_smem(cby, sorb, cr, TX, rows, nv, p.nfl, real, per, doubling, r0_rows, field).total;
     };
     if (need(0) > kResSmem) continue;
     int r0_rows = doubling ? 0 : rows;
     while (r0_rows > 0 && need(r0_rows) > kResSmem) --r0_rows;
+    p.cby = cby;
+    p.vecs = vectors_of(fp64, realv, cby);
     p.regions = regions;
     p.TX = TX;
     p.G = (int)G;
@@ -687,15 +740,7 @@ ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, i
     p.levels = lv;
     return p;
   }
-  return p;
-}
-
-// Whether any sweep of the lattice could fit, and the most chunks of one (for the work space).
-int resident_max_chunks(kite_ctx* ctx, int lattice, int Lx, int Ly, int C) {
-  const double orb = (double)Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1);
-  int cr = C;
-  while (cr >= 1 && orb * cr * 32.0 > (double)ctx->num_sms * kResSmem) cr >>= 1;
-  return cr;
+  return cby == 16 && !fp64 ? resident_plan(ctx, fp64, lattice, doubling, realv, field, Lx, Ly, C, M, TX, G, 8) : p;
 }
 
 // FP64 sums may be grouped freely: strips and virtual CTAs that give every SM a compact
@@ -714,7 +759,7 @@ ResidentPlan resident_plan_free(kite_ctx* ctx, int lattice, int doubling, int re
     const int colT = TX * sorb * C;
     const int nv = std::max(1, std::min(rows, kRMax / std::max(1, colT)));
     const ResidentPlan p = resident_plan(ctx, 1, lattice, doubling, realv, field, Lx, Ly, C, M, TX,
-                                         std::min<long long>((long long)regions * nv, units));
+                                         std::min<long long>((long long)regions * nv, units), 16);
     if (p.CR == 0) continue;
     // a step: the rows of the longest column in sites of the whole SM, plus the edge
     const long long sweeps = C / p.CR;
@@ -726,20 +771,31 @@ ResidentPlan resident_plan_free(kite_ctx* ctx, int lattice, int doubling, int re
   return best;
 }
 
-size_t resident_rec_bytes(int lattice, int Lx, int Ly, int CR) {
-  return (size_t)2 * Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1) * CR * 32;
+size_t rec_bytes_of(int lattice, int Lx, int Ly, int CR, int cby) {
+  return (size_t)2 * Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1) * CR * 2 * cby;
 }
 
-size_t resident_part_bytes(kite_ctx* ctx, int fp64, int realv, int C, int slots) {
-  const int lanes = C * sums_of(fp64, realv);
-  return (size_t)slots * ctx->num_sms * (kRComm / 32) * (fp64 ? std::max(8, lanes) : lanes) * sizeof(double);
+void resident_space(kite_ctx* ctx, int fp64, int lattice, int realv, int Lx, int Ly, int C, int slots, size_t* rec,
+                    size_t* part) {
+  *rec = *part = 0;
+  const double orb = (double)Lx * Ly * (lattice == KITE_HONEYCOMB ? 2 : 1);
+  for (int cby = 16; cby >= (fp64 ? 16 : 8); cby >>= 1) {
+    int cr = C * 16 / cby;  // two iterates of cr units must fit the SMs together
+    while (cr >= 1 && orb * cr * 2.0 * cby > (double)ctx->num_sms * kResSmem) cr >>= 1;
+    if (cr < 1) continue;
+    const int lanes = cr * sums_of(fp64, realv, cby);
+    *rec = std::max(*rec, rec_bytes_of(lattice, Lx, Ly, cr, cby));
+    *part = std::max(*part, (size_t)slots * ctx->num_sms * (kRComm / 32) * (fp64 ? std::max(8, lanes) : lanes) *
+                                sizeof(double));
+  }
 }
 
 int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
   const ResidentPlan& p = a->plan;
   const int var = a->phase ? 1 : (a->realv ? 2 : 0);
-  const void* fn = a->fp64 ? res_kernel<double>(a->lattice, a->doubling, var)
-                           : res_kernel<float>(a->lattice, a->doubling, var);
+  const void* fn = a->fp64        ? res_kernel<double, 16>(a->lattice, a->doubling, var)
+                   : p.cby == 16 ? res_kernel<float, 16>(a->lattice, a->doubling, var)
+                                 : res_kernel<float, 8>(a->lattice, a->doubling, var);
   {
     static std::mutex mu;
     static std::set<std::pair<const void*, int>> done;
@@ -750,8 +806,8 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
     }
   }
   const int steps = timing_steps > 0 ? timing_steps : (a->doubling ? (a->M + 1) / 2 : a->M - 1);
-  const int per_chunk = per_chunk_of(a->fp64, a->realv);
-  const size_t rec_bytes = resident_rec_bytes(a->lattice, a->Lx, a->Ly, p.CR);
+  const int per = p.vecs, C = a->C * (16 / p.cby);  // vectors per unit, units per orbital
+  const size_t rec_bytes = rec_bytes_of(a->lattice, a->Lx, a->Ly, p.CR, p.cby);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)p.regions);
   cfg.blockDim = dim3((unsigned)(p.T + kRComm));
@@ -763,7 +819,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   KITE_CUDA_TRY(ctx, cudaEventRecord(ctx->ev2, ctx->stream));
-  for (int c0 = 0; c0 < a->C && c0 * per_chunk < a->nvec; c0 += p.CR) {
+  for (int c0 = 0; c0 < C && c0 * per < a->nvec; c0 += p.CR) {
     // no record may carry a step number of an earlier sweep
     KITE_CUDA_TRY(ctx, cudaMemsetAsync(a->rec, 0, rec_bytes, ctx->stream));
     auto launch = [&](auto tag) -> cudaError_t {
@@ -775,7 +831,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
       r.last[1] = a->bA;  // odd iterates
       r.last[0] = a->bB;
       r.part = a->part;
-      r.rec = static_cast<Rec*>(a->rec);
+      r.rec = a->rec;
       r.err = ctx->d_status;
       r.tt = (Real)a->tt;
       r.Lx = a->Lx;
@@ -787,7 +843,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
       r.nfl = p.nfl;
       r.r0_rows = p.r0_rows;
       r.levels = p.levels;
-      r.C = a->C;
+      r.C = C;
       r.c0 = c0;
       r.CR = p.CR;
       r.steps = steps;
@@ -801,10 +857,10 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
     KITE_CUDA_TRY(ctx, a->fp64 ? launch(double()) : launch(float()));
     a->stall = 0;
     if (timing_steps > 0) break;
-    const int nvec = std::min(a->nvec - c0 * per_chunk, p.CR * per_chunk);
+    const int nvec = std::min(a->nvec - c0 * per, p.CR * per);
     k_resident_reduce<<<a->M, 256, 0, ctx->stream>>>(a->part, a->M, p.regions * (kRComm / 32) * (32 >> p.levels),
-                                                     p.CR * sums_of(a->fp64, a->realv), !a->fp64 && !a->realv, nvec,
-                                                     a->vec_base + c0 * per_chunk, a->n_eff,
+                                                     p.CR * sums_of(a->fp64, a->realv, p.cby),
+                                                     !a->fp64 && !a->realv, nvec, a->vec_base + c0 * per, a->n_eff,
                                                      a->mu_vec);
     KITE_CUDA_TRY(ctx, cudaGetLastError());
   }
@@ -821,7 +877,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
   const double n_orb = (double)a->Lx * a->Ly * sorb;
   const double off_chip = a->doubling ? 0.0 : 1.0 - (double)p.r0_rows / p.rows;
   a->bytes = n_orb * a->C * 16.0 * (1.0 + off_chip * steps) + n_orb * (a->fp64 ? 8.0 : 4.0) +
-             8.0 * a->M * p.regions * (kRComm / 32) * (32 >> p.levels) * ((a->C + p.CR - 1) / p.CR);
+             8.0 * a->M * p.regions * (kRComm / 32) * (32 >> p.levels) * ((C + p.CR - 1) / p.CR);
   return KITE_OK;
 }
 

@@ -109,18 +109,18 @@ __global__ void __launch_bounds__(kBlock, 3)  // <= 85 registers: three CTAs fit
         ok = step_body<float, LAT, C, true, MODE, NST, FIELD>(ring, rank, T.ncta, nullptr, S.r0, S.bA, S.r0,
                                                          S.vt, S.tt, S.Lx, S.Ly, S.units,
                                                          S.partial + (size_t)T.ncta * Q, S.partial, err, 0,
-                                                         nofam, 0, SeriesOut{}, S.phase);
+                                                         nofam, 0, SeriesOut{}, S.phase, Open{}, mcap > 0);
       else if (DBL)
         ok = step_body<float, LAT, C, false, MODE, NST, FIELD>(ring, rank, T.ncta, where(n - 1), where(n),
                                                           where(n + 1), S.r0, S.vt, S.tt, S.Lx, S.Ly, S.units,
                                                           S.partial + (size_t)(2 * n + 1) * T.ncta * Q,
                                                           S.partial + (size_t)(2 * n) * T.ncta * Q, err, 0,
-                                                          nofam, 0, SeriesOut{}, S.phase);
+                                                          nofam, 0, SeriesOut{}, S.phase, Open{}, mcap > 0);
       else
         ok = step_body<float, LAT, C, false, MODE, NST, FIELD>(ring, rank, T.ncta, where(n - 1), where(n),
                                                           where(n + 1), S.r0, S.vt, S.tt, S.Lx, S.Ly, S.units,
                                                           S.partial + (size_t)(n + 1) * T.ncta * Q, nullptr,
-                                                          err, 0, nofam, 0, SeriesOut{}, S.phase);
+                                                          err, 0, nofam, 0, SeriesOut{}, S.phase, Open{}, mcap > 0);
       if (!ok) return;
       // step_body reused the ring's shared memory for its reduction (generic-proxy
       // writes); order them before the next step's bulk copies into the same memory
@@ -200,10 +200,11 @@ __global__ void __launch_bounds__(kBlock2, KITE_BATCHED2_MIN_CTAS)
       const bool ok = DBL ? step2_body<float, LAT, C, NST, true>(ring, rank, T.ncta, w4(n - 1), w4(n), w4(n + 1),
                                                                  w4(n + 2), nullptr, S.vt, S.tt, S.Lx, S.Ly,
                                                                  S.units, slot(2 * n), slot(2 * n + 1), err, 0,
-                                                                 slot(2 * n + 2), slot(2 * n + 3))
+                                                                 slot(2 * n + 2), slot(2 * n + 3), nullptr, mcap > 0)
                           : step2_body<float, LAT, C, NST, false, true>(
                                 ring, rank, T.ncta, w4(n - 1), w4(n), w4(n + 1), w4(n + 2), S.r0, S.vt, S.tt,
-                                S.Lx, S.Ly, S.units, slot(n + 1), slot(n + 2), err, 0);
+                                S.Lx, S.Ly, S.units, slot(n + 1), slot(n + 2), err, 0, nullptr, nullptr, nullptr,
+                                mcap > 0);
       if (!ok) return;
       if (!sync_team()) return;
     }

@@ -145,19 +145,15 @@ __global__ void k_init_r0(int64_t ncell, const Real* __restrict__ vt, int vec_ba
 // Moment partial of one complex pair: (sr, si) += conj(a) b, as a chain of fused
 // multiply-adds (one rounding per product and sum); every kernel that accumulates the
 // moments <r_0|r_n> uses it, so the one-step and the two-step sweeps give the same bits.
-// The FP64 sweeps, bound by GB300's FP64 pipe, form the real part only: the imaginary
-// part of <r|T_n(H~)|r> (and of <r_n|r_n>, <r_n|r_{n+1}>) vanishes for a Hermitian H~, so
-// si stays 0 and two of the update's fourteen FP64 operations go.  The FP32 sweeps keep
-// it (their ALU work is free under the HBM bound) as a rounding diagnostic.
-template <typename Acc, typename Real>
-__device__ __forceinline__ void cacc(Acc& sr, Acc& si, Real ar_, Real ai_, Real br_, Real bi_) {
-  const Acc ar = ar_, ai = ai_, br = br_, bi = bi_;
+// The FP64 sweeps, bound by GB300's FP64 pipe, form the real part only (acc_reals below):
+// the imaginary part of <r|T_n(H~)|r> (and of <r_n|r_n>, <r_n|r_{n+1}>) vanishes for a
+// Hermitian H~, so it reads 0.  The FP32 sweeps keep it (their ALU work is free under the HBM
+// bound) as a rounding diagnostic.
+__device__ __forceinline__ void cacc(float& sr, float& si, float ar, float ai, float br, float bi) {
   sr = rfma(ar, br, sr);
   sr = rfma(ai, bi, sr);
-  if constexpr (sizeof(Real) == 4) {
-    si = rfma(ar, bi, si);
-    si = rfma(-ai, br, si);
-  }
+  si = rfma(ar, bi, si);
+  si = rfma(-ai, br, si);
 }
 
 template <typename Real>
@@ -265,27 +261,129 @@ __device__ __forceinline__ void cta_lane_sums(const double (&d)[QT], bool in_war
   }
 }
 
-// CTA reduction of the per-thread moment partials (the ring is drained, so its memory is
-// reused): lane (vector v = c*VPC + q, component) of `partial` for this CTA.
-template <int QT, int C, typename Acc>
-__device__ __forceinline__ void moment_partials(double (&dacc)[QT], Acc (&facc)[QT],
-                                                double (&dacc0)[QT], Acc (&facc0)[QT], bool first,
-                                                unsigned char* stages, double* partial,
-                                                double* partial0, int cta) {
+// The same sums, NS sets of them, in the same pairs and order (the same bits) with fewer adds,
+// which the FP64 pipe takes at two a cycle and SM: while a lane holds more than one component
+// it keeps half of them and hands its partner the other half, so that a thread adds 4 to 6
+// times a set instead of 12 to 20 (FP32), and the sets' last sums run side by side.  The
+// persistent batch of 24 square lattices, L up to 1024: 147.0 -> 139.4 ms.
+// `red` holds NS sets of kRedSet<QT, C> doubles; warp_lane_sums is called by the warps that
+// hold partials, then sets_lane_sums by every thread of the CTA.
+//
+// Where it runs: the FP64 sweeps and the persistent batch.  The FP32 sweeps of one system keep
+// cta_lane_sums, and so do the batch's probe launches: with the quicker sums the autotuner
+// took two steps a pass instead of one at 40 000 to 60 000 orbitals, and the shape it takes
+// sets the grouping of the FP32 sums (7e-10 of the moments there), while the sweep itself runs
+// on chip at these sizes (one of 16.8 million cells gains 0.8 %).
+template <int QT, int C>
+constexpr int kRedSet = kBlock / 32 * C * QT;
+
+template <int QT, int C>
+__device__ __forceinline__ void warp_lane_sums(const double (&d)[QT], double* red) {
+  static_assert((QT == 2 && C <= 16) || (QT == 4 && C <= 8), "a component per group of lanes");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double v[QT];
 #pragma unroll
-  for (int k = 0; k < QT; ++k) {
-    dacc[k] += (double)facc[k];
-    if (first) dacc0[k] += (double)facc0[k];
+  for (int k = 0; k < QT; ++k) v[k] = d[k];
+  int comp = 0;  // the component that v[0] ends as
+#pragma unroll
+  for (int off = 16, n = QT; off >= C; off >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & off;
+      if (up) comp += n;
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        const double keep = up ? v[k + n] : v[k], give = up ? v[k] : v[k + n];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    }
   }
-  double* red = reinterpret_cast<double*>(stages);
+  constexpr int held = 32 / QT - C;  // lane bits between the chunk and the component
+  if ((lane & held) == 0) red[(warp * C + (lane & (C - 1))) * QT + comp] = v[0];
+}
+
+template <int QT, int C, int NS>
+__device__ __forceinline__ void sets_lane_sums(const double* red, double* const (&out)[NS]) {
   constexpr int Q = C * QT;
-  cta_lane_sums<QT, C>(dacc, true, red, partial + (size_t)cta * Q);
-  if (first) {
-    __syncthreads();
-    cta_lane_sums<QT, C>(dacc0, true, red, partial0 + (size_t)cta * Q);
+  static_assert(NS * Q <= kBlock, "one thread per sum");
+  __syncthreads();
+  const int tid = threadIdx.x;
+  if (tid < NS * Q) {
+    const int set = tid / Q, i = tid - set * Q;
+    const double* r = red + set * kRedSet<QT, C> + i;
+    double sum = 0.0;
+#pragma unroll
+    for (int w = 0; w < kBlock / 32; ++w) sum += r[w * Q];
+    double* o = out[0];
+#pragma unroll
+    for (int k = 1; k < NS; ++k)
+      if (set == k) o = out[k];
+    o[i] = sum;
   }
 }
 
+// A thread's FP64 sum of one component: the rows promoted so far plus the FP32 rows since.
+// (The FP64 sweeps sum in `f` throughout: no promotion.)
+__device__ __forceinline__ double lane_total(double d, float f) { return d + (double)f; }
+__device__ __forceinline__ double lane_total(double, double f) { return f; }
+
+// FP64 products of a chunk's two reals, each in a chain of its own; fold_reals joins them
+// for complex vectors after the last row.  One form for real and complex vectors: a branch on
+// `realv` in the row loop is predicated, and the instructions it turns off still take the
+// FP64 pipe, the bound of the FP64 sweeps (20 of them a chunk and step instead of 14 with
+// moment doubling: 1000 x 1001 sites, four vectors 163 -> 124 us a step).
+template <int QT>
+__device__ __forceinline__ void acc_reals(double (&f)[QT], const double (&a)[QT], const double (&b)[QT]) {
+#pragma unroll
+  for (int k = 0; k < QT; ++k) f[k] = rfma(a[k], b[k], f[k]);
+}
+template <typename Acc, int QT>
+__device__ __forceinline__ void fold_reals(Acc (&f)[QT], int realv) {
+  if constexpr (sizeof(Acc) == 8) {
+    static_assert(QT == 2, "one complex vector");
+    if (!realv) {
+      f[0] += f[1];
+      f[1] = Acc(0);
+    }
+  }
+}
+
+// CTA reduction of the per-thread moment partials (the ring is drained, so its memory is
+// reused): lane (vector v = c*VPC + q, component) of `partial` for this CTA.
+template <int QT, int C, bool FIRST, typename Acc>
+__device__ __forceinline__ void moment_partials(double (&dacc)[QT], Acc (&facc)[QT], double (&dacc0)[QT],
+                                                Acc (&facc0)[QT], int realv, bool plain, unsigned char* stages,
+                                                double* partial, double* partial0, int cta) {
+  fold_reals(facc, realv);
+  if (FIRST) fold_reals(facc0, realv);
+#pragma unroll
+  for (int k = 0; k < QT; ++k) {
+    dacc[k] = lane_total(dacc[k], facc[k]);
+    if (FIRST) dacc0[k] = lane_total(dacc0[k], facc0[k]);
+  }
+  double* red = reinterpret_cast<double*>(stages);
+  constexpr int Q = C * QT;
+  double* const out = partial + (size_t)cta * Q;
+  if (plain) {
+    cta_lane_sums<QT, C>(dacc, true, red, out);
+    if (FIRST) {
+      __syncthreads();
+      cta_lane_sums<QT, C>(dacc0, true, red, partial0 + (size_t)cta * Q);
+    }
+    return;
+  }
+  warp_lane_sums<QT, C>(dacc, red);
+  if constexpr (FIRST) {
+    warp_lane_sums<QT, C>(dacc0, red + kRedSet<QT, C>);
+    double* const outs[2] = {out, partial0 + (size_t)cta * Q};
+    sets_lane_sums<QT, C, 2>(red, outs);
+  } else {
+    double* const outs[1] = {out};
+    sets_lane_sums<QT, C, 1>(red, outs);
+  }
+}
 
 // Open boundaries (the configuration's boundaries flag set to False): a bond whose cell
 // offset leaves the lattice along an open direction is absent.  The kernels stage the
@@ -355,7 +453,7 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
                                           int* __restrict__ err, int stall, const FamOut& fam,
                                           int realv = 0, const SeriesOut& ser = SeriesOut{},
                                           const Real* __restrict__ phase = nullptr,
-                                          const Open& open = Open{}) {
+                                          const Open& open = Open{}, bool plain = sizeof(Real) == 4) {
   static_assert(MODE == 0 || MODE == 3 || MODE == 4 || (sizeof(Real) == 4 && C * 2 <= kMaxFamVecs),
                 "family modes run on FP32 batches of at most two vectors");
   using Ch = Chunk<Real>;
@@ -541,7 +639,10 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
           a.st(ser.acc, qi);
         } else if constexpr (MODE == 3) {
           // moment doubling: <r_n|r_{n+1}> into facc, <r_n|r_n> into facc0
-          if (realv) {
+          if constexpr (sizeof(Real) == 8) {
+            acc_reals(facc, me.v, out.v);
+            acc_reals(facc0, me.v, me.v);
+          } else if (realv) {
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
               const Acc a = me.v[k], b = out.v[k];
@@ -556,7 +657,7 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
               facc0[2 * q] = rfma(ai, ai, rfma(ar, ar, facc0[2 * q]));
             }
           }
-          if (++rows == kFlushRows) {
+          if (sizeof(Real) == 4 && ++rows == kFlushRows) {
             rows = 0;
 #pragma unroll
             for (int k = 0; k < QT; ++k) {
@@ -600,7 +701,10 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
             }
           }
         } else {  // MODE 0: fused moment <r_0|r_{n+1}> (and <r_0|r_0> on the first step)
-          if (realv) {
+          if constexpr (sizeof(Real) == 8) {
+            acc_reals(facc, z0.v, out.v);
+            if (FIRST) acc_reals(facc0, z0.v, z0.v);
+          } else if (realv) {
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
               const Acc a = z0.v[k], b = out.v[k];
@@ -617,7 +721,7 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
               }
             }
           }
-          if (++rows == kFlushRows) {
+          if (sizeof(Real) == 4 && ++rows == kFlushRows) {
             rows = 0;
 #pragma unroll
             for (int k = 0; k < QT; ++k) {
@@ -653,9 +757,9 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
   }
   ring.gslot = gslot;
   if constexpr (MODE == 0)
-    moment_partials<QT, C>(dacc, facc, dacc0, facc0, FIRST, stages, partial, partial0, cta);
+    moment_partials<QT, C, FIRST>(dacc, facc, dacc0, facc0, realv, plain, stages, partial, partial0, cta);
   if constexpr (MODE == 3)
-    moment_partials<QT, C>(dacc, facc, dacc0, facc0, true, stages, partial, partial0, cta);
+    moment_partials<QT, C, true>(dacc, facc, dacc0, facc0, realv, plain, stages, partial, partial0, cta);
   return true;
 }
 

@@ -65,7 +65,8 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
                                            const Real* __restrict__ vt, Real tt, int Lx, int Ly, long long units,
                                            double* __restrict__ partial1, double* __restrict__ partial2,
                                            int* __restrict__ err, int realv, double* __restrict__ partial3 = nullptr,
-                                           double* __restrict__ partial4 = nullptr, const Series2* ser = nullptr) {
+                                           double* __restrict__ partial4 = nullptr, const Series2* ser = nullptr,
+                                           bool plain = sizeof(Real) == 4) {
   static_assert(SER < 0 || (!DBL && !SMACC && (SER == 0 || SER == 2 || SER == 4)), "series pass: 0, 2 or 4 terms");
   using Ch = Chunk<Real>;
   using Acc = typename AccT<Real>::T;
@@ -240,7 +241,9 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
       return out;
     };
     auto accumulate = [&](Acc(&facc)[QT], double(&dacc)[QT], int& rows, const Ch& z0, const Ch& out) {
-      if (realv) {
+      if constexpr (sizeof(Real) == 8) {
+        acc_reals(facc, z0.v, out.v);
+      } else if (realv) {
 #pragma unroll
         for (int k = 0; k < NR; ++k) facc[k] += (Acc)z0.v[k] * (Acc)out.v[k];
       } else {
@@ -248,7 +251,7 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
         for (int q = 0; q < VPC; ++q) cacc(facc[2 * q], facc[2 * q + 1], z0.v[2 * q], z0.v[2 * q + 1],
                                             out.v[2 * q], out.v[2 * q + 1]);
       }
-      if (++rows == kFlushRows) {
+      if (sizeof(Real) == 4 && ++rows == kFlushRows) {
         rows = 0;
 #pragma unroll
         for (int k = 0; k < QT; ++k) dacc[k] += (double)facc[k], facc[k] = Acc(0);
@@ -257,7 +260,9 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
 
     // the plain moment with its FP64 sum in this thread's shared-memory slot ks
     auto accumulate_sm = [&](Acc(&facc)[QT], int& rows, int ks, const Ch& z0, const Ch& out) {
-      if (realv) {
+      if constexpr (sizeof(Real) == 8) {
+        acc_reals(facc, z0.v, out.v);
+      } else if (realv) {
 #pragma unroll
         for (int k = 0; k < NR; ++k) facc[k] += (Acc)z0.v[k] * (Acc)out.v[k];
       } else {
@@ -265,7 +270,7 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
         for (int q = 0; q < VPC; ++q) cacc(facc[2 * q], facc[2 * q + 1], z0.v[2 * q], z0.v[2 * q + 1],
                                             out.v[2 * q], out.v[2 * q + 1]);
       }
-      if (++rows == kFlushRows) {
+      if (sizeof(Real) == 4 && ++rows == kFlushRows) {
         rows = 0;
 #pragma unroll
         for (int k = 0; k < QT; ++k) dsm[ks * QT + k] += (double)facc[k], facc[k] = Acc(0);
@@ -275,7 +280,10 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
     // (real part); every kFlushRows rows both go into this thread's FP64 slots ka, kb
     auto accumulate_dbl = [&](Acc(&fr)[QT], Acc(&fg)[QT], int& rows, int ka, int kb, const Ch& me,
                               const Ch& out) {
-      if (realv) {
+      if constexpr (sizeof(Real) == 8) {
+        acc_reals(fr, me.v, out.v);
+        acc_reals(fg, me.v, me.v);
+      } else if (realv) {
 #pragma unroll
         for (int k = 0; k < NR; ++k) {
           const Acc a = me.v[k], b = out.v[k];
@@ -290,7 +298,7 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
           fg[2 * q] = rfma(ai, ai, rfma(ar, ar, fg[2 * q]));
         }
       }
-      if (++rows == kFlushRows) {
+      if (sizeof(Real) == 4 && ++rows == kFlushRows) {
         rows = 0;
 #pragma unroll
         for (int k = 0; k < QT; ++k) {
@@ -493,18 +501,28 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
   constexpr int Q = C * QT;
   if constexpr (DBL) {
     // slot k's FP64 sum from shared memory plus the FP32 rows since the last flush
-    double* const outs[4] = {partial1, partial2, partial3, partial4};
+    fold_reals(facc1, realv);
+    fold_reals(facc2, realv);
+    fold_reals(gacc1, realv);
+    fold_reals(gacc2, realv);
+    double* const outs[4] = {partial1 + (size_t)cta * Q, partial2 + (size_t)cta * Q, partial3 + (size_t)cta * Q,
+                             partial4 + (size_t)cta * Q};
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       double d[QT];
 #pragma unroll
       for (int k = 0; k < QT; ++k) {
         const Acc f = kk == 0 ? gacc1[k] : kk == 1 ? facc1[k] : kk == 2 ? gacc2[k] : facc2[k];
-        d[k] = compute ? dsm[kk * QT + k] + (double)f : 0.0;
+        d[k] = compute ? lane_total(dsm[kk * QT + k], f) : 0.0;
       }
-      if (kk) __syncthreads();
-      cta_lane_sums<QT, C>(d, compute, red, outs[kk] + (size_t)cta * Q);
+      if (plain) {
+        if (kk) __syncthreads();
+        cta_lane_sums<QT, C>(d, compute, red, outs[kk]);
+      } else if (compute) {
+        warp_lane_sums<QT, C>(d, red + kk * kRedSet<QT, C>);
+      }
     }
+    if (!plain) sets_lane_sums<QT, C, 4>(red, outs);
     return true;
   }
   if constexpr (SMACC) {
@@ -514,11 +532,22 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
       dacc2[k] = compute ? dsm[QT + k] : 0.0;
     }
   }
+  fold_reals(facc1, realv);
+  fold_reals(facc2, realv);
 #pragma unroll
-  for (int k = 0; k < QT; ++k) dacc1[k] += (double)facc1[k], dacc2[k] += (double)facc2[k];
-  cta_lane_sums<QT, C>(dacc1, compute, red, partial1 + (size_t)cta * Q);
-  __syncthreads();
-  cta_lane_sums<QT, C>(dacc2, compute, red, partial2 + (size_t)cta * Q);
+  for (int k = 0; k < QT; ++k) dacc1[k] = lane_total(dacc1[k], facc1[k]), dacc2[k] = lane_total(dacc2[k], facc2[k]);
+  double* const outs[2] = {partial1 + (size_t)cta * Q, partial2 + (size_t)cta * Q};
+  if (plain) {
+    cta_lane_sums<QT, C>(dacc1, compute, red, outs[0]);
+    __syncthreads();
+    cta_lane_sums<QT, C>(dacc2, compute, red, outs[1]);
+    return true;
+  }
+  if (compute) {
+    warp_lane_sums<QT, C>(dacc1, red);
+    warp_lane_sums<QT, C>(dacc2, red + kRedSet<QT, C>);
+  }
+  sets_lane_sums<QT, C, 2>(red, outs);
   return true;
 }
 

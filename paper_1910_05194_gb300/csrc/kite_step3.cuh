@@ -138,7 +138,9 @@ __device__ __forceinline__ bool step3_body(Ring& ring, int cta, int ncta, const 
     return out;
   };
   auto accumulate = [&](Acc(&facc)[QT], double(&dacc)[QT], int& rows, const Ch& z0, const Ch& out) {
-    if (realv) {
+    if constexpr (sizeof(Real) == 8) {
+      acc_reals(facc, z0.v, out.v);
+    } else if (realv) {
 #pragma unroll
       for (int k = 0; k < NR; ++k) facc[k] += (Acc)z0.v[k] * (Acc)out.v[k];
     } else {
@@ -146,7 +148,7 @@ __device__ __forceinline__ bool step3_body(Ring& ring, int cta, int ncta, const 
       for (int q = 0; q < VPC; ++q)
         cacc(facc[2 * q], facc[2 * q + 1], z0.v[2 * q], z0.v[2 * q + 1], out.v[2 * q], out.v[2 * q + 1]);
     }
-    if (++rows == kFlushRows) {
+    if (sizeof(Real) == 4 && ++rows == kFlushRows) {
       rows = 0;
 #pragma unroll
       for (int k = 0; k < QT; ++k) dacc[k] += (double)facc[k], facc[k] = Acc(0);
@@ -335,9 +337,15 @@ __device__ __forceinline__ bool step3_body(Ring& ring, int cta, int ncta, const 
   ring.gslot = gslot;
   // partial1..3 <- <r_0|r_{n+1..n+3}>: fixed-order sums over the compute threads holding
   // each chunk (the ring is drained; its memory is reused)
+  fold_reals(facc1, realv);
+  fold_reals(facc2, realv);
+  fold_reals(facc3, realv);
 #pragma unroll
-  for (int k = 0; k < QT; ++k)
-    dacc1[k] += (double)facc1[k], dacc2[k] += (double)facc2[k], dacc3[k] += (double)facc3[k];
+  for (int k = 0; k < QT; ++k) {
+    dacc1[k] = lane_total(dacc1[k], facc1[k]);
+    dacc2[k] = lane_total(dacc2[k], facc2[k]);
+    dacc3[k] = lane_total(dacc3[k], facc3[k]);
+  }
   double* red = reinterpret_cast<double*>(stages);
   constexpr int Q = C * QT;
   cta_lane_sums<QT, C>(dacc1, compute, red, partial1 + (size_t)cta * Q);

@@ -420,6 +420,25 @@ inline bool autotune_enabled() {
   return !(e && e[0] == '0');
 }
 
+// Milliseconds of three launches of a candidate, the better of two timings after a warm-up:
+// the shape chosen sets the grouping of the FP32 moment sums, so one late launch should not
+// decide between two close candidates.
+template <typename Launch>
+float time_launches(kite_ctx* ctx, Launch launch) {
+  launch();  // warm-up
+  float best = 1e30f;
+  for (int rep = 0; rep < 2; ++rep) {
+    cudaEventRecord(ctx->ev2, ctx->stream);
+    for (int i = 0; i < 3; ++i) launch();
+    cudaEventRecord(ctx->ev3, ctx->stream);
+    float ms = 1e30f;
+    if (cudaEventSynchronize(ctx->ev3) != cudaSuccess || cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3) != cudaSuccess)
+      return 1e30f;
+    best = std::min(best, ms);
+  }
+  return best;
+}
+
 // KITE_PASS_STEPS=1, 2 or 3 pins the steps per pass of the plain moment sweep (the
 // autotuner then chooses only the ring depth and occupancy); unset, all are candidates.
 inline int pass_steps_pinned() {
@@ -449,14 +468,7 @@ float time_candidate2(kite_ctx* ctx, int k, long long units, const Plan& p, cons
         partial + (size_t)3 * G * Q, ctx->d_status, p.realv ? 1 : 0,
         DBL ? partial + (size_t)4 * G * Q : nullptr, DBL ? partial + (size_t)5 * G * Q : nullptr);
   };
-  launch();  // warm-up
-  cudaEventRecord(ctx->ev2, st);
-  for (int i = 0; i < 3; ++i) launch();
-  cudaEventRecord(ctx->ev3, st);
-  float ms = 1e30f;
-  if (cudaEventSynchronize(ctx->ev3) != cudaSuccess || cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3) != cudaSuccess)
-    return 1e30f;
-  return ms / 6.0f;
+  return time_launches(ctx, launch) / 6.0f;
 }
 
 template <typename Real, int LAT, int C, int NST>
@@ -479,14 +491,7 @@ float time_candidate3(kite_ctx* ctx, int k, long long units, const Plan& p, cons
         bA, bB, bC, bD, r0, vt, tt, p.Lx, p.Ly, units, partial + (size_t)2 * G * Q,
         partial + (size_t)3 * G * Q, partial + (size_t)4 * G * Q, ctx->d_status, p.realv ? 1 : 0);
   };
-  launch();  // warm-up
-  cudaEventRecord(ctx->ev2, st);
-  for (int i = 0; i < 3; ++i) launch();
-  cudaEventRecord(ctx->ev3, st);
-  float ms = 1e30f;
-  if (cudaEventSynchronize(ctx->ev3) != cudaSuccess || cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3) != cudaSuccess)
-    return 1e30f;
-  return ms / 9.0f;
+  return time_launches(ctx, launch) / 9.0f;
 }
 
 template <typename Real, int LAT, int C, int MODE, int NST>
@@ -502,14 +507,7 @@ float time_candidate(kite_ctx* ctx, int k, long long units, const Plan& p, const
         bA, bB, bA, MODE == 0 ? r0 : nullptr, vt, tt, p.Lx, p.Ly, units, partial + (size_t)2 * G * Q,
         MODE == 3 ? partial + (size_t)G * Q : nullptr, ctx->d_status, 0, FamOut{}, p.realv ? 1 : 0, SeriesOut{}, nullptr, p.open);
   };
-  launch();  // warm-up
-  cudaEventRecord(ctx->ev2, st);
-  for (int i = 0; i < 3; ++i) launch();
-  cudaEventRecord(ctx->ev3, st);
-  float ms = 1e30f;
-  if (cudaEventSynchronize(ctx->ev3) != cudaSuccess || cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3) != cudaSuccess)
-    return 1e30f;
-  return ms / 3.0f;  // per recursion step
+  return time_launches(ctx, launch) / 3.0f;  // per recursion step
 }
 
 // The two-step pass is a candidate of the plain moment sweep (MODE 0) and of the doubling

@@ -343,12 +343,13 @@ def secondary_legs(kite, ctx, peaks):
     s1 = kite.make_system(kite.HONEYCOMB, 64, 64, -2.7, 1.0, 0.0, 0.0, 1)
     mu1 = np.zeros(256)
     res = {}
-    # the autotuner's choice (the on-chip cluster sweep when it is measured faster), then
-    # the streaming step kernels alone (KITE_CLUSTER=0) for comparison
+    # the autotuner's choice (an on-chip sweep when it is measured faster), then the streaming
+    # step kernels alone (KITE_CLUSTER=0, KITE_RESIDENT=0) for comparison
+    on_chip = ("KITE_CLUSTER", "KITE_RESIDENT")
     for suffix, pin in (("", None), ("_streaming", "0")):
-        old = os.environ.pop("KITE_CLUSTER", None)
+        old = {k: os.environ.pop(k, None) for k in on_chip}
         if pin is not None:
-            os.environ["KITE_CLUSTER"] = pin
+            os.environ.update({k: pin for k in on_chip})
         try:
             for name, dbl in (("plain", False), ("doubling", True)):
                 kpm1 = kite.make_kpm(256, 4, 1, kite.FP64, -b, b, doubling=dbl)
@@ -362,9 +363,10 @@ def secondary_legs(kite, ctx, peaks):
                 if pin is None:
                     res[name + "_cluster_ctas"] = st.cluster_ctas
         finally:
-            os.environ.pop("KITE_CLUSTER", None)
-            if old is not None:
-                os.environ["KITE_CLUSTER"] = old
+            for k, v in old.items():
+                os.environ.pop(k, None)
+                if v is not None:
+                    os.environ[k] = v
     out["small_dos_honeycomb_64x64_M256_R4_fp64"] = res
     # batched: 256 square systems, L 64..1024, W 0..4, M in {512..4096}, R = 4, one launch
     specs = synth.batched_square_systems(256, seed=3)

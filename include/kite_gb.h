@@ -336,6 +336,16 @@ int kite_evolution_coeffs(int M, double dt, double e_min, double e_max, double* 
  * Errors: KITE_ERR_ARG. */
 int kite_debug_stall_once(kite_ctx* ctx, int enable);
 
+/* Test hook for the on-chip sweep of mid-size lattices (no counterpart in the paper): of the
+ * sweeps that kite_moments_1d starts from now on, timing runs included, `skip` run as usual
+ * and the next `count` fail.  KITE_FAIL_WAIT: one region sends nothing, so its neighbours'
+ * bounded waits give up (after about a second) and the sweep ends.  KITE_FAIL_LAUNCH: the
+ * launch is reported as refused and does not happen.  count = 0 disarms the hook.
+ * Errors: KITE_ERR_ARG. */
+#define KITE_FAIL_WAIT 1
+#define KITE_FAIL_LAUNCH 2
+int kite_debug_fail_resident(kite_ctx* ctx, int kind, int skip, int count);
+
 /* ---- 2D moments ----------------------------------------------------------------- */
 
 /* Velocity directions of the 2D moments. */

@@ -371,6 +371,16 @@ int kite_set_stream(kite_ctx* ctx, void* cuda_stream) {
   return KITE_OK;
 }
 
+int kite_debug_fail_resident(kite_ctx* ctx, int kind, int skip, int count) {
+  if (!ctx) return KITE_ERR_ARG;
+  if ((kind != KITE_FAIL_WAIT && kind != KITE_FAIL_LAUNCH) || skip < 0 || count < 0)
+    return fail(ctx, KITE_ERR_ARG, "need kind KITE_FAIL_WAIT or KITE_FAIL_LAUNCH, skip >= 0, count >= 0");
+  ctx->fail_kind = kind;
+  ctx->fail_skip = skip;
+  ctx->fail_count = count;
+  return KITE_OK;
+}
+
 int kite_debug_stall_once(kite_ctx* ctx, int enable) {
   if (!ctx) return KITE_ERR_ARG;
   ctx->debug_stall = enable ? 1 : 0;

@@ -49,6 +49,7 @@ struct kite_ctx {
   // Device status word: kernels set it (never trap) when a bounded wait gives up.
   int* d_status = nullptr;
   int debug_stall = 0;  // test hook, see kite_debug_stall_once
+  int fail_kind = 0, fail_skip = 0, fail_count = 0;  // test hook, see kite_debug_fail_resident
   // Autotuner cache: key (kernel family, precision, lattice, vectors per orbital, mode,
   // size bucket) -> (ring depth, CTAs per SM) measured fastest on this context's GPU.
   std::map<uint64_t, std::pair<int, int>> tune;

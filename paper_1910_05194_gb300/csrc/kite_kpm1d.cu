@@ -723,31 +723,52 @@ inline int resident_pinned() {  // 0 unset, 1 off, 2 on
 constexpr size_t kResidentPartMax = (size_t)2 << 30;
 
 // Whether to run the batch resident.  `other_ms` times the kernels chosen otherwise, per
-// recursion step of the batch.
-template <typename OtherMs>
-bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
-  if (resident_pinned() == 2) return true;
+// recursion step of the batch.  The verdict is kept with the tuned shapes: {1 or 0, 0}; {-1, n}
+// after n failed timings (a launch refused, or a short run that took as long as the long one),
+// which decide nothing: the next call times again, kResidentTries times at most.
+constexpr int kResidentTries = 3;
+
+inline uint64_t resident_key(const ResidentSweep& r) {
   uint64_t key = 0x6b697465726573ull;
   for (uint64_t f : {(uint64_t)r.fp64, (uint64_t)r.lattice, (uint64_t)r.doubling, (uint64_t)r.realv,
                      (uint64_t)r.nvec, (uint64_t)r.C, (uint64_t)r.Lx, (uint64_t)r.Ly, (uint64_t)r.open_x,
                      (uint64_t)r.open_y, (uint64_t)(r.phase != nullptr)})
     key = (key ^ f) * 0x100000001b3ull;
-  key = (key | 1ull << 63) & ~(1ull << 62);
+  return (key | 1ull << 63) & ~(1ull << 62);
+}
+
+template <typename OtherMs>
+bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
+  if (resident_pinned() == 2) return true;
+  const uint64_t key = resident_key(r);
+  int tries = 0;
   auto it = ctx->tune.find(key);
-  if (it != ctx->tune.end()) return it->second.first != 0;
+  if (it != ctx->tune.end()) {
+    if (it->second.first >= 0) return it->second.first != 0;
+    tries = it->second.second;
+    if (tries >= kResidentTries) return false;
+  }
   // two timing runs, so that the launch and load cost drops out; the best of two each
+  const std::string last_error = ctx->last_error;  // (a failed timing is no failed call)
+  bool ok = true;
   auto timed = [&](int steps) {
     double best = 1e30;
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 2 && ok; ++k) {
       ResidentSweep t = r;
-      if (resident_sweep(ctx, &t, steps) != KITE_OK) return 1e30;
+      ok = resident_sweep(ctx, &t, steps) == KITE_OK;
       best = std::min(best, t.seconds);
     }
     return best;
   };
   const double t8 = timed(8), t40 = timed(kClusterTimeSteps);
+  cudaGetLastError();
+  if (!ok || t40 <= t8) {
+    ctx->last_error = last_error;
+    ctx->tune[key] = {-1, tries + 1};
+    return false;
+  }
   const int per_sweep = r.plan.CR * r.plan.vecs, sweeps = (r.nvec + per_sweep - 1) / per_sweep;
-  const float ms = (float)(1e3 * std::max(0.0, t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
+  const float ms = (float)(1e3 * (t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
   const int pick = ms < 0.95f * other_ms() ? 1 : 0;  // it must win clearly
   cudaGetLastError();
   ctx->tune[key] = {pick, 0};

@@ -792,6 +792,16 @@ void resident_space(kite_ctx* ctx, int fp64, int lattice, int realv, int Lx, int
 
 int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
   const ResidentPlan& p = a->plan;
+  if (ctx->fail_count > 0) {  // test hook
+    if (ctx->fail_skip > 0) {
+      --ctx->fail_skip;
+    } else {
+      --ctx->fail_count;
+      if (ctx->fail_kind == KITE_FAIL_LAUNCH)
+        return cuda_fail(ctx, cudaErrorCooperativeLaunchTooLarge, "on-chip sweep");
+      a->stall = 1;
+    }
+  }
   const int var = a->phase ? 1 : (a->realv ? 2 : 0);
   const void* fn = a->fp64        ? res_kernel<double, 16>(a->lattice, a->doubling, var)
                    : p.cby == 16 ? res_kernel<float, 16>(a->lattice, a->doubling, var)

@@ -1,0 +1,65 @@
+"""What a call does when the on-chip sweep of a mid-size lattice cannot run: the streaming
+kernels take over, the moments are those of a call that never tried (the same tuned shape: the
+same bits), and nothing is decided from a failed timing.  The failures are made by the hook
+kite_debug_fail_resident: a launch reported as refused, or a bounded wait that runs out and
+returns a status."""
+import contextlib
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+kite = pytest.importorskip("paper_1910_05194_gb300")
+
+LATTICES = [dict(lattice=kite.HONEYCOMB, Lx=200, Ly=220, t=-2.7, W=1.0, seed=5),
+            dict(lattice=kite.SQUARE, Lx=200, Ly=201, t=-1.0, W=1.0, seed=5, flux=2.0 / 201)]
+
+
+@contextlib.contextmanager
+def env(**kw):
+    old = {k: os.environ.get(k) for k in kw}
+    os.environ.update(kw)
+    try:
+        yield
+    finally:
+        for k, v in old.items():
+            os.environ.pop(k, None) if v is None else os.environ.__setitem__(k, v)
+
+
+def call(ctx, d, precision, R=4, M=64):
+    mu, per = np.zeros(M), np.zeros((R, M, 2))
+    st = kite.moments_1d(ctx, kite.make_system(**d), kite.make_kpm(M, R, 1, precision), mu, per)
+    return per, st.block
+
+
+@contextlib.contextmanager
+def fresh(d, precision, R=4):
+    """A context of its own, with the streaming sweep's moments and the two paths' block sizes."""
+    with kite.Context(0) as ctx:
+        with env(KITE_RESIDENT="0"):
+            ref, stream = call(ctx, d, precision, R)
+        with env(KITE_RESIDENT="1"):
+            chip = call(ctx, d, precision, R)[1]
+        assert chip != stream
+        yield ctx, ref, stream, chip
+
+
+@pytest.mark.parametrize("precision", [kite.FP32, kite.FP64])
+@pytest.mark.parametrize("d", LATTICES)
+@pytest.mark.parametrize("count", [1, 100])
+def test_a_failed_timing_decides_nothing(d, precision, count):
+    with fresh(d, precision) as (ctx, ref, stream, chip):
+        kite.debug_fail_resident(ctx, kite.FAIL_LAUNCH, 0, count)
+        per, block = call(ctx, d, precision)
+        assert block == stream and np.array_equal(per, ref)
+        kite.debug_fail_resident(ctx, kite.FAIL_LAUNCH, 0, 0)
+        assert call(ctx, d, precision)[1] == chip  # timed again: faster at these sizes
+
+
+@pytest.mark.parametrize("kind,skip,count", [(0, 0, 1), (3, 0, 1), (1, -1, 1), (2, 0, -1)])
+def test_the_hook_refuses_what_it_does_not_know(kind, skip, count):
+    with kite.Context(0) as ctx, pytest.raises(kite.KiteError) as e:
+        kite.debug_fail_resident(ctx, kind, skip, count)
+    assert e.value.status == kite.ERR_ARG

@@ -351,6 +351,7 @@ void kite_destroy(kite_ctx* ctx) {
   if (ctx->ev2) cudaEventDestroy(ctx->ev2);
   if (ctx->ev3) cudaEventDestroy(ctx->ev3);
   if (ctx->d_status) cudaFree(ctx->d_status);
+  if (ctx->sweep_status) cudaFreeHost(const_cast<int*>(ctx->sweep_status));
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }

@@ -48,6 +48,10 @@ struct kite_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // Device status word: kernels set it (never trap) when a bounded wait gives up.
   int* d_status = nullptr;
+  // The on-chip sweep's own status word, page-locked host memory that its kernel writes when a
+  // wait gives up: the host reads it after each sweep without a copy, and a timing run that
+  // gave up leaves the call's d_status alone.
+  volatile int* sweep_status = nullptr;
   int debug_stall = 0;  // test hook, see kite_debug_stall_once
   int fail_kind = 0, fail_skip = 0, fail_count = 0;  // test hook, see kite_debug_fail_resident
   // Autotuner cache: key (kernel family, precision, lattice, vectors per orbital, mode,
@@ -188,7 +192,8 @@ struct ResidentSweep {
   int grid, block;
 };
 // timing_steps > 0: a timing run of that many steps of the first chunks; 0: the whole sweep,
-// then the moments into mu_vec (with doubling, before the undoubling).
+// then the moments into mu_vec (with doubling, before the undoubling).  KITE_ERR_TIMEOUT: a
+// wait gave up; the start vectors are as they were.
 int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps);
 
 // AdamW step coefficients of the learned reconstructor's training (kite_mlp.cu).

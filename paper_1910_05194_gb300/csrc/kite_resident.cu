@@ -129,7 +129,7 @@ struct ResArgs {
   void* last[2];      // r_last: the last two iterates in the batch layout, r_n in last[n & 1]
   double* part;       // moment partials [slot n][CTA][exchange warps][32 >> levels]
   void* rec;          // edge records [parity][cell][sublattice][CR units]
-  int* err;
+  volatile int* err;  // host memory: 1 when a wait gave up
   Real tt;
   int Lx, Ly, TX, G;  // strip width, virtual CTAs
   int rows_max, nv_max, nfl, r0_rows, levels;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       if (!ok) s_abort = 1;
       __syncthreads();  // r_{n+1} complete in the region and its frame
       if (s_abort) {
-        if (ct == 0) atomicExch(a.err, 1);
+        if (ct == 0) *a.err = 1;
         return;
       }
     }
@@ -815,6 +815,12 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
       done.insert({fn, ctx->device});
     }
   }
+  if (!ctx->sweep_status) {
+    void* word = nullptr;
+    KITE_CUDA_TRY(ctx, cudaHostAlloc(&word, 64, cudaHostAllocMapped));  // (unified addressing: one address)
+    ctx->sweep_status = static_cast<volatile int*>(word);
+  }
+  *ctx->sweep_status = 0;  // (no sweep of this context is in flight: each one is waited for)
   const int steps = timing_steps > 0 ? timing_steps : (a->doubling ? (a->M + 1) / 2 : a->M - 1);
   const int per = p.vecs, C = a->C * (16 / p.cby);  // vectors per unit, units per orbital
   const size_t rec_bytes = rec_bytes_of(a->lattice, a->Lx, a->Ly, p.CR, p.cby);
@@ -842,7 +848,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
       r.last[0] = a->bB;
       r.part = a->part;
       r.rec = a->rec;
-      r.err = ctx->d_status;
+      r.err = ctx->sweep_status;
       r.tt = (Real)a->tt;
       r.Lx = a->Lx;
       r.Ly = a->Ly;
@@ -878,6 +884,7 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
   float ms = 0.f;
   KITE_CUDA_TRY(ctx, cudaEventSynchronize(ctx->ev3));
   KITE_CUDA_TRY(ctx, cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3));
+  if (*ctx->sweep_status) return fail(ctx, KITE_ERR_TIMEOUT, "a bounded wait of the on-chip sweep gave up");
   a->seconds = 1e-3 * ms;
   a->grid = p.regions;
   a->block = p.T + kRComm;

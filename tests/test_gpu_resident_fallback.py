@@ -58,6 +58,18 @@ def test_a_failed_timing_decides_nothing(d, precision, count):
         assert call(ctx, d, precision)[1] == chip  # timed again: faster at these sizes
 
 
+@pytest.mark.parametrize("precision", [kite.FP32, kite.FP64])
+@pytest.mark.parametrize("d", LATTICES)
+@pytest.mark.parametrize("skip,count", [(0, 1), (2, 1), (0, 2), (2, 2)])
+def test_a_wait_that_runs_out_in_a_timing_run_does_not_fail_the_call(d, precision, skip, count):
+    with fresh(d, precision) as (ctx, ref, stream, chip):
+        kite.debug_fail_resident(ctx, kite.FAIL_WAIT, skip, count)
+        per, block = call(ctx, d, precision)
+        assert block == stream and np.array_equal(per, ref)
+        kite.debug_fail_resident(ctx, kite.FAIL_WAIT, 0, 0)
+        assert call(ctx, d, precision)[1] == chip
+
+
 @pytest.mark.parametrize("kind,skip,count", [(0, 0, 1), (3, 0, 1), (1, -1, 1), (2, 0, -1)])
 def test_the_hook_refuses_what_it_does_not_know(kind, skip, count):
     with kite.Context(0) as ctx, pytest.raises(kite.KiteError) as e:

@@ -259,8 +259,10 @@ int kite_flux_nearest(const kite_system* sys, double flux, double* out);
  * to about 1.5 million orbitals in FP32) may run the sweep on chip as well, one region of the
  * lattice per SM in one cooperative launch whose CTAs wait on their neighbours within a
  * bound; it keeps the streaming launch's grouping of the FP32 moment sums.  Chosen where
- * measured faster; KITE_RESIDENT=0 / 1 forbids / forces it.  If a wait runs out (its SMs held
- * by another long kernel), the call runs the streaming kernels instead.
+ * measured faster; KITE_RESIDENT=0 / 1 forbids / forces it.  Where it cannot run (its launch
+ * is refused, or a wait runs out because another long kernel holds its SMs), the kernels
+ * chosen otherwise take that batch of vectors and the rest of the call; after three such
+ * failures of a size the context no longer tries it there, unless KITE_RESIDENT=1.
  *   mu          [M] FP64, real part of the average, host or device (required)
  *   mu_per_vec  [S*R][M] complex FP64 interleaved (re, im) per vector, or NULL
  *   st          statistics, or NULL

@@ -723,9 +723,10 @@ inline int resident_pinned() {  // 0 unset, 1 off, 2 on
 constexpr size_t kResidentPartMax = (size_t)2 << 30;
 
 // Whether to run the batch resident.  `other_ms` times the kernels chosen otherwise, per
-// recursion step of the batch.  The verdict is kept with the tuned shapes: {1 or 0, 0}; {-1, n}
-// after n failed timings (a launch refused, or a short run that took as long as the long one),
-// which decide nothing: the next call times again, kResidentTries times at most.
+// recursion step of the batch.  The verdict is kept with the tuned shapes: {1 or 0, n}; {-1, n}
+// after a failure (a launch refused, a wait that ran out, or a short timing run that took as long
+// as the long one), n failures so far.  A failure decides nothing: the next call times again,
+// until kResidentTries of them have shown that this GPU's SMs are not to be had.
 constexpr int kResidentTries = 3;
 
 inline uint64_t resident_key(const ResidentSweep& r) {
@@ -737,16 +738,22 @@ inline uint64_t resident_key(const ResidentSweep& r) {
   return (key | 1ull << 63) & ~(1ull << 62);
 }
 
+inline void resident_failed(kite_ctx* ctx, const ResidentSweep& r) {
+  std::pair<int, int>& verdict = ctx->tune[resident_key(r)];
+  verdict = {-1, verdict.second + 1};
+}
+
+// 1: resident, 0: not, -1: not, and a timing run failed.
 template <typename OtherMs>
-bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
-  if (resident_pinned() == 2) return true;
+int resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
+  if (resident_pinned() == 2) return 1;
   const uint64_t key = resident_key(r);
-  int tries = 0;
+  int failures = 0;
   auto it = ctx->tune.find(key);
   if (it != ctx->tune.end()) {
-    if (it->second.first >= 0) return it->second.first != 0;
-    tries = it->second.second;
-    if (tries >= kResidentTries) return false;
+    if (it->second.first >= 0) return it->second.first;
+    failures = it->second.second;
+    if (failures >= kResidentTries) return 0;
   }
   // two timing runs, so that the launch and load cost drops out; the best of two each
   const std::string last_error = ctx->last_error;  // (a failed timing is no failed call)
@@ -764,21 +771,21 @@ bool resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
   cudaGetLastError();
   if (!ok || t40 <= t8) {
     ctx->last_error = last_error;
-    ctx->tune[key] = {-1, tries + 1};
-    return false;
+    resident_failed(ctx, r);
+    return -1;
   }
   const int per_sweep = r.plan.CR * r.plan.vecs, sweeps = (r.nvec + per_sweep - 1) / per_sweep;
   const float ms = (float)(1e3 * (t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
   const int pick = ms < 0.95f * other_ms() ? 1 : 0;  // it must win clearly
   cudaGetLastError();
-  ctx->tune[key] = {pick, 0};
-  return pick != 0;
+  ctx->tune[key] = {pick, failures};
+  return pick;
 }
 
 template <typename Real, int LAT>
 int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const Scale& sc,
               double* mu_dev, double* imag_dev, double* mu_vec_dev_ext, kite_stats* stats,
-              const double* r0_dev_all, bool* resident_used, bool allow_resident) {
+              const double* r0_dev_all) {
   constexpr int SORB = (LAT == KITE_HONEYCOMB) ? 2 : 1;
   constexpr int VPC = Chunk<Real>::kVecs;
   constexpr int kMaxC = 4;
@@ -834,7 +841,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
           : cluster_part_doubles(p.realv ? p.max_batch : 2 * p.max_batch, 16, p.M, p.doubling, kClusterTimeSteps);
   // the resident sweep's moment partials and edge records, where the lattice may fit on chip
   size_t resident_part = 0, resident_rec = 0;
-  if (allow_resident && resident_pinned() != 1 && p.M >= 4)
+  if (resident_pinned() != 1 && p.M >= 4)
     resident_space(ctx, sizeof(Real) == 8, LAT, p.realv, p.Lx, p.Ly, Cmax, std::max(p.M + 1, 2 * kClusterTimeSteps + 2),
                    &resident_rec, &resident_part);
   if (resident_part > kResidentPartMax) resident_part = resident_rec = 0;
@@ -894,6 +901,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
   int grid_used = 0;
   Tune tune_used{kStages, 0};
   int cluster_used = 0, steps_used = 0, block_used = kBlock;
+  bool resident_off = false;  // an on-chip sweep of this call failed
   double step_s = 0.0, step_bytes = 0.0;
   int64_t step_n = 0;
   KITE_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
@@ -1123,18 +1131,37 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       // (an FP32 batch that runs on chip in clusters stays there: its moment sums are grouped
       // by the clusters' threads)
       const bool pinned_res = resident_pinned() == 2;
-      const bool may_reside = resident_rec != 0 && (pinned_res || (!ctx->debug_stall && autotune_enabled() &&
-                                                                   !pass_steps_pinned() && !getenv("KITE_TUNE") &&
-                                                                   cluster_pinned() != 2));
+      const bool may_reside =
+          resident_rec != 0 && !resident_off &&
+          (pinned_res || (!ctx->debug_stall && autotune_enabled() && !pass_steps_pinned() && !getenv("KITE_TUNE") &&
+                          cluster_pinned() != 2));
       if (may_reside && (sizeof(Real) == 8 || cl.cs == 0 || pinned_res))
         rs.plan = resident_for(C, sizeof(Real) == 8 ? 0 : (p.field ? fs.G : tuned_grid()));
-      if (rs.plan.CR && resident_choice(ctx, rs, other_ms)) {
-        // mid-size lattice: the whole sweep on chip, a region per SM (kite_resident.cu)
-        rs.stall = ctx->debug_stall;
+      const int choice = rs.plan.CR ? resident_choice(ctx, rs, other_ms) : 0;
+      if (choice < 0) resident_off = true;
+      bool resident = choice > 0;
+      if (resident) {
+        // mid-size lattice: the whole sweep on chip, a region per SM (kite_resident.cu).  Where
+        // it cannot run (its launch refused, or a neighbour that did not come up within the
+        // bounded wait because another long kernel holds its SM), the other kernels, whose CTAs
+        // do not wait on one another, take this batch from the same start vectors and the rest
+        // of the call.
+        const std::string last_error = ctx->last_error;
+        const bool stalled = ctx->debug_stall != 0;
+        rs.stall = stalled;
         ctx->debug_stall = 0;
-        *resident_used = true;
         rc = resident_sweep(ctx, &rs, 0);
-        if (rc != KITE_OK) return rc;
+        if (rc != KITE_OK && stalled) return rc;  // the hook asks for the status
+        if (rc != KITE_OK) {
+          cudaGetLastError();
+          ctx->last_error = last_error;
+          resident_failed(ctx, rs);
+          resident_off = true;
+          resident = false;
+          block_used = kBlock;
+        }
+      }
+      if (resident) {
         if (p.doubling) {
           k_undouble<<<(nvec * p.M + 255) / 256, 256, 0, st>>>(mu_vec, p.M, nvec, vec_base);
           KITE_CUDA_TRY(ctx, cudaGetLastError());
@@ -1268,24 +1295,11 @@ int moments_1d_impl(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
                     double* mu_dev, double* imag_dev, double* mu_vec_dev, kite_stats* st,
                     const double* r0_dev_all) {
   const bool fp64 = kpm->precision == KITE_FP64;
-  bool resident = false;
-  const bool stalled = ctx->debug_stall != 0;
-  auto run = [&](bool allow_resident) {
-    if (sys->lattice == KITE_HONEYCOMB)
-      return fp64 ? run_typed<double, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
-                                                      &resident, allow_resident)
-                  : run_typed<float, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
-                                                     &resident, allow_resident);
-    return fp64 ? run_typed<double, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
-                                                 &resident, allow_resident)
-                : run_typed<float, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all,
-                                                &resident, allow_resident);
-  };
-  int rc = run(true);
-  // A neighbour that never came up within the bounded wait (another long kernel holding its
-  // SM): the streaming kernels, whose CTAs do not wait on one another, take the call.
-  if (rc == KITE_ERR_TIMEOUT && resident && !stalled) rc = run(false);
-  return rc;
+  if (sys->lattice == KITE_HONEYCOMB)
+    return fp64 ? run_typed<double, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all)
+                : run_typed<float, KITE_HONEYCOMB>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all);
+  return fp64 ? run_typed<double, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all)
+              : run_typed<float, KITE_SQUARE>(ctx, sys, kpm, sc, mu_dev, imag_dev, mu_vec_dev, st, r0_dev_all);
 }
 
 }  // namespace kite

@@ -70,6 +70,34 @@ def test_a_wait_that_runs_out_in_a_timing_run_does_not_fail_the_call(d, precisio
         assert call(ctx, d, precision)[1] == chip
 
 
+@pytest.mark.parametrize("kind", [kite.FAIL_LAUNCH, kite.FAIL_WAIT])
+@pytest.mark.parametrize("precision", [kite.FP32, kite.FP64])
+@pytest.mark.parametrize("d", LATTICES)
+@pytest.mark.parametrize("pinned", [False, True])
+def test_a_failed_sweep_goes_to_the_streaming_kernels(d, precision, kind, pinned):
+    with fresh(d, precision, 16) as (ctx, ref, stream, chip):  # two or four batches
+        assert call(ctx, d, precision, 16)[1] == chip
+        with env(**({"KITE_RESIDENT": "1"} if pinned else {})):
+            kite.debug_fail_resident(ctx, kind, 0, 1)
+            per, block = call(ctx, d, precision, 16)
+            assert block == stream and np.array_equal(per, ref)
+            assert kite.lib().kite_last_error(ctx.handle) == b""
+            assert call(ctx, d, precision, 16)[1] == chip
+
+
+@pytest.mark.parametrize("d", LATTICES)
+def test_a_sweep_that_keeps_failing_is_tried_once_a_call_and_three_times_in_all(d):
+    with fresh(d, kite.FP32, 16) as (ctx, ref, stream, chip):
+        assert call(ctx, d, kite.FP32, 16)[1] == chip
+        for n, left in ((2, "one is left after the first batch"), (1, "the third failure")):
+            kite.debug_fail_resident(ctx, kite.FAIL_WAIT, 0, n)
+            for _ in range(n):
+                per, block = call(ctx, d, kite.FP32, 16)
+                assert block == stream and np.array_equal(per, ref), left
+        per, block = call(ctx, d, kite.FP32, 16)
+        assert block == stream and np.array_equal(per, ref)
+
+
 @pytest.mark.parametrize("kind,skip,count", [(0, 0, 1), (3, 0, 1), (1, -1, 1), (2, 0, -1)])
 def test_the_hook_refuses_what_it_does_not_know(kind, skip, count):
     with kite.Context(0) as ctx, pytest.raises(kite.KiteError) as e:

@@ -1,0 +1,69 @@
+"""Calls on a device that is nearly full: where the faster path's work space does not fit, the
+path that needs less runs, with the same results, and the call is refused only when that one
+does not fit either."""
+import contextlib
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+kite = pytest.importorskip("paper_1910_05194_gb300")
+
+MiB = 1 << 20
+
+
+@contextlib.contextmanager
+def env(**kw):
+    old = {k: os.environ.get(k) for k in kw}
+    os.environ.update(kw)
+    try:
+        yield
+    finally:
+        for k, v in old.items():
+            os.environ.pop(k, None) if v is None else os.environ.__setitem__(k, v)
+
+
+@contextlib.contextmanager
+def free_memory(mib):
+    """All but `mib` MiB of the device's free memory taken."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    block = torch.empty(torch.cuda.mem_get_info()[0] - mib * MiB, dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del block
+        torch.cuda.empty_cache()
+
+
+def moments(ctx, M, R=8):
+    s = kite.make_system(kite.HONEYCOMB, 257, 510, t=-2.7, W=2.0, seed=3)
+    mu, per = np.zeros(M), np.zeros((R, M, 2))
+    st = kite.moments_1d(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), mu, per)
+    return per, st.block
+
+
+def test_moments_without_room_for_the_on_chip_sweeps_partials():
+    """262140 orbitals, eight vectors, M = 8192: five vector buffers of 17 MB and partials of 152
+    CTAs times the streaming grid's CTAs per SM (3 to 5), 16 sums and 8 bytes a step: 0.5 to
+    0.9 GB; on chip 152 x 8 instead: 1.3 GB and 0.03 GB of records."""
+    M = 8192
+    with kite.Context(0) as ctx:
+        with env(KITE_RESIDENT="0"):
+            ref, stream = moments(ctx, M)
+        short = moments(ctx, 64)[1]
+    assert short != stream  # on chip where there is room
+    with kite.Context(0) as ctx:
+        with env(KITE_RESIDENT="0"):
+            moments(ctx, 64)  # the same tuned shape
+        with free_memory(1240):
+            per, block = moments(ctx, M)
+            assert kite.lib().kite_last_error(ctx.handle) == b""
+        assert block == stream and np.max(np.abs(per - ref)) <= 1e-6
+    with kite.Context(0) as ctx, free_memory(64):
+        with pytest.raises(kite.KiteError) as e:
+            moments(ctx, M)
+        assert e.value.status == kite.ERR_OOM

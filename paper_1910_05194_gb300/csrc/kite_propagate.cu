@@ -198,7 +198,7 @@ int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
   // two steps per pass (its outputs never alias its inputs: two more buffers)
   constexpr bool kPass = sizeof(Real) == 4 && !FIELD;
   const char* pin = getenv("KITE_PASS_STEPS");
-  const bool pass = kPass && !sys->open_x && !sys->open_y && M >= 4 && !(pin && pin[0] == '1' && pin[1] == 0);
+  bool pass = kPass && !sys->open_x && !sys->open_y && M >= 4 && !(pin && pin[0] == '1' && pin[1] == 0);
   void *bC = nullptr, *bD = nullptr;
   Carver probe(nullptr);
   auto lay = [&](Carver& k, Real** vt, void** r0, void** bA, void** bB, void** acc, double** part,
@@ -220,7 +220,15 @@ int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
   unsigned long long* ne;
   Real* ph;
   lay(probe, &vt, &r0, &bA, &bB, &acc, &part, &ne, &ph);
+  const std::string last_error = ctx->last_error;
   int rc = ensure_ws(ctx, probe.used());
+  if (rc == KITE_ERR_OOM && pass) {  // single steps need four vector buffers instead of six
+    pass = false;
+    probe = Carver(nullptr);
+    lay(probe, &vt, &r0, &bA, &bB, &acc, &part, &ne, &ph);
+    rc = ensure_ws(ctx, probe.used());
+    if (rc == KITE_OK) ctx->last_error = last_error;
+  }
   if (rc != KITE_OK) return rc;
   Carver w(ctx->ws);
   lay(w, &vt, &r0, &bA, &bB, &acc, &part, &ne, &ph);

@@ -67,3 +67,24 @@ def test_moments_without_room_for_the_on_chip_sweeps_partials():
         with pytest.raises(kite.KiteError) as e:
             moments(ctx, M)
         assert e.value.status == kite.ERR_OOM
+
+
+def test_time_evolution_without_room_for_two_steps_a_pass():
+    """3.2 million cells, eight packets: a vector buffer has 205 MB; single steps take four of
+    them and 13 MB (0.83 GB), two steps a pass two more (1.24 GB).  The bits are the same."""
+    L, R, M = 1789, 8, 12
+    s = kite.make_system(kite.SQUARE, L, L, t=-1.0, W=1.0, seed=4)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    psi0 = torch.randn(R, L * L, 2, dtype=torch.float64, device="cuda", generator=g) / L
+    ref, psi = psi0.clone(), psi0.clone()
+    norms = np.zeros((2, 1, R))
+    with kite.Context(0) as ctx:
+        kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, ref, norms[0])
+    with kite.Context(0) as ctx, free_memory(1050):
+        st = kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, psi, norms[1])
+        assert st.step_launches == M - 1 and kite.lib().kite_last_error(ctx.handle) == b""
+    assert torch.equal(ref, psi) and np.array_equal(norms[0], norms[1])
+    with kite.Context(0) as ctx, free_memory(700):
+        with pytest.raises(kite.KiteError) as e:
+            kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, psi)
+        assert e.value.status == kite.ERR_OOM

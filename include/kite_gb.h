@@ -196,8 +196,8 @@ typedef struct kite_ctx kite_ctx;
  *   KITE_AUTOTUNE=0       no timing of launch shapes: 8-stage rings at full occupancy, one
  *                         recursion step per launch, no on-chip sweep
  *   KITE_TUNE=SxK[x2|x3]  pins the 1D sweep's ring depth S, CTAs per SM K and steps per pass
- *   KITE_PASS_STEPS=1|2|3 pins the steps per pass (1D and batched sweeps; 3: 1D only; 1 also
- *                         the FP32 time evolution's)
+ *   KITE_PASS_STEPS=1|2|3 pins the steps per pass (1D and batched sweeps; 3: 1D only; 1 and
+ *                         2 also the FP32 time evolution's)
  *   KITE_CLUSTER=0|1      forbids / forces the on-chip cluster sweep of small lattices
  *                         (KITE_CLUSTER_CTAS=2..16 pins its CTAs per cluster)
  *   KITE_RESIDENT=0|1     forbids / forces the on-chip sweep of mid-size lattices

@@ -197,8 +197,12 @@ int propagate_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, 
   const int nb = (int)std::min<int64_t>((nchunk + 255) / 256, (int64_t)ctx->num_sms * 8);
   // two steps per pass (its outputs never alias its inputs: two more buffers)
   constexpr bool kPass = sizeof(Real) == 4 && !FIELD;
-  const char* pin = getenv("KITE_PASS_STEPS");
-  bool pass = kPass && !sys->open_x && !sys->open_y && M >= 4 && !(pin && pin[0] == '1' && pin[1] == 0);
+  // (KITE_AUTOTUNE=0 keeps one step per launch unless KITE_PASS_STEPS asks for two, as in the
+  // moment sweeps)
+  const char *pin = getenv("KITE_PASS_STEPS"), *tuner = getenv("KITE_AUTOTUNE");
+  const int pinned = (pin && pin[0] && !pin[1]) ? pin[0] - '0' : 0;
+  bool pass = kPass && !sys->open_x && !sys->open_y && M >= 4 && pinned != 1 &&
+              (pinned == 2 || !(tuner && tuner[0] == '0'));
   void *bC = nullptr, *bD = nullptr;
   Carver probe(nullptr);
   auto lay = [&](Carver& k, Real** vt, void** r0, void** bA, void** bB, void** acc, double** part,

@@ -303,8 +303,8 @@ inline int batched_pass_steps_pinned() {
 
 template <int LAT, int C, int NST, bool DBL = false>
 int batched2_occupancy() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     constexpr int SMEM = Batched2Shape<LAT, C, NST, DBL>::SMEM;
     int o = 0;
     if (SMEM > 227 * 1024 ||
@@ -314,24 +314,22 @@ int batched2_occupancy() {
             cudaSuccess)
       o = 0;
     cudaGetLastError();
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 template <int LAT, int C, bool DBL, int NST, bool FIELD>
 int batched_occupancy() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     constexpr int SMEM = StepShape<LAT, C, NST>::template smem_bytes<DBL ? 3 : 0>();
     cudaFuncSetAttribute(k_batched<LAT, C, DBL, NST, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     int o = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_batched<LAT, C, DBL, NST, FIELD>, kBlock, SMEM) !=
         cudaSuccess)
       o = 0;
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 // smallest target share whose schedule fits `gmax` resident CTAs

@@ -56,8 +56,8 @@ constexpr int kFieldStages = 8;
 
 template <typename Real, int LAT, int C, int MODE>
 int field_occupancy_t() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     constexpr int SM = StepShape<LAT, C, kFieldStages>::template smem_bytes<MODE>();
     cudaFuncSetAttribute(k_step<Real, LAT, C, true, MODE, kFieldStages, true>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
@@ -67,9 +67,8 @@ int field_occupancy_t() {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_step<Real, LAT, C, false, MODE, kFieldStages, true>,
                                                       kBlock, SM) != cudaSuccess || o < 1)
       o = 1;
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 // The step launches of one vector batch (the plain sweep's schedule, one step per launch):

@@ -459,12 +459,13 @@ int gemm_split_bf16(kite_ctx* ctx, const void* Ahi, const void* Alo, const void*
   a.Nrows = Nrows;
   a.part = part;
   a.err = ctx->d_status;
-  static bool attr = false;
-  if (!attr) {
-    KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_gemm_split_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            kGemmSmem));
-    attr = true;
-  }
+  static PerDevice attr;
+  cudaError_t ae = cudaSuccess;
+  attr.get(ctx->device, [&] {
+    ae = cudaFuncSetAttribute(k_gemm_split_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+    return ae == cudaSuccess ? 1 : -1;
+  });
+  KITE_CUDA_TRY(ctx, ae);
   CUtensorMap mAh, mAl, mBh, mBl;
   int rc;
   if ((rc = make_map(ctx, &mAh, Ahi, Kp, Mrows, kBM)) != KITE_OK) return rc;

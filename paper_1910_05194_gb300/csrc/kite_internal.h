@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "kite_gb.h"
+#include "kite_once.h"
 
 namespace kite {
 // How the resident sweep cuts a lattice over the SMs (kite_resident.cu).
@@ -66,6 +67,12 @@ namespace kite {
 // Records a message on the context and returns `status`.
 int fail(kite_ctx* ctx, int status, const std::string& msg);
 int cuda_fail(kite_ctx* ctx, cudaError_t e, const char* what);
+
+// The calling thread's device (the entry points set it to their context's).
+inline int current_device() {
+  int d = 0;
+  return cudaGetDevice(&d) == cudaSuccess ? d : 0;
+}
 
 // Ensures at least `bytes` of device work space; returns KITE_OK / KITE_ERR_OOM.
 int ensure_ws(kite_ctx* ctx, size_t bytes);

@@ -533,11 +533,13 @@ int operand_map(kite_ctx* ctx, const __nv_bfloat16* p, int rows, int cols, int l
 int gemm(kite_ctx* ctx, cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
          int N, int K, GemmEpi ep) {
   if (M < 1 || N < 1 || K < 1) return KITE_OK;
-  static bool attr = false;
-  if (!attr) {
-    KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTSmem));
-    attr = true;
-  }
+  static PerDevice attr;
+  cudaError_t ae = cudaSuccess;
+  attr.get(ctx->device, [&] {
+    ae = cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTSmem);
+    return ae == cudaSuccess ? 1 : -1;
+  });
+  KITE_CUDA_TRY(ctx, ae);
   CUtensorMap mA, mB;
   int rc = operand_map(ctx, A, M, K, lda, &mA);
   if (rc == KITE_OK) rc = operand_map(ctx, B, N, K, ldb, &mB);

@@ -169,16 +169,15 @@ __global__ void __launch_bounds__(kBlock2, 3)
 
 template <typename Real, int LAT, int C, int TERMS>
 int series2_occupancy() {
-  static int occ = -1;  // per template instance
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     int o = 0;
     constexpr int SM = Step2Shape<LAT, C, kSeriesStages, false, false, TERMS>::SMEM;
     cudaFuncSetAttribute(k_series2<Real, LAT, C, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_series2<Real, LAT, C, TERMS>, kBlock2, SM) != cudaSuccess)
       o = 1;
-    occ = std::max(1, o);
-  }
-  return occ;
+    return std::max(1, o);
+  });
 }
 
 template <typename Real, int LAT, int C, bool FIELD>

@@ -832,8 +832,8 @@ __global__ void k_extract(int64_t ncell, const void* __restrict__ buf, int nvec,
 // kernels' dynamic shared-memory limit).
 template <typename Real, int LAT, int C, int MODE = 0, int NST = kStages, bool FIELD = false>
 int step_occupancy() {
-  static int occ = -1;  // per template instance; device-independent enough for one GPU type
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     int o = 0;
     const int smem = StepShape<LAT, C, NST>::template smem_bytes<MODE>();
     cudaFuncSetAttribute(k_step<Real, LAT, C, true, MODE, NST, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -844,9 +844,8 @@ int step_occupancy() {
                                                       smem) != cudaSuccess ||
         o < 1)
       o = 1;
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 // Persistent grid of the step kernel: min(ctas_per_sm, occupancy) CTAs per SM (0 = the

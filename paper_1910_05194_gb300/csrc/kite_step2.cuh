@@ -574,17 +574,16 @@ __global__ void __launch_bounds__(kBlock2, 3 * Step2Shape<LAT, C, NST, DBL>::SME
 
 template <typename Real, int LAT, int C, int NST, bool DBL = false>
 int step2_occupancy() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     int o = 0;
     const int smem = Step2Shape<LAT, C, NST, DBL>::SMEM;
     cudaFuncSetAttribute(k_step2<Real, LAT, C, NST, DBL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_step2<Real, LAT, C, NST, DBL>, kBlock2, smem) !=
         cudaSuccess)
       o = 0;
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 }  // namespace

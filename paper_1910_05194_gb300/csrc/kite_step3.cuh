@@ -379,8 +379,8 @@ __global__ void __launch_bounds__(kBlock3, 2)
 
 template <typename Real, int LAT, int C, int NST>
 int step3_occupancy() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ;  // per template instance
+  return occ.get(current_device(), [] {
     int o = 0;
     const int smem = Step3Shape<LAT, C, NST>::SMEM;
     if (smem > 227 * 1024 ||
@@ -389,9 +389,8 @@ int step3_occupancy() {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_step3<Real, LAT, C, NST>, kBlock3, smem) != cudaSuccess)
       o = 0;
     cudaGetLastError();
-    occ = o;
-  }
-  return occ;
+    return o;
+  });
 }
 
 }  // namespace

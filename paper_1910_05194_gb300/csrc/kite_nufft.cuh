@@ -26,6 +26,15 @@ constexpr double kPi = 3.141592653589793;
 // to 1.8 of it at M = 32 .. 48, 0.9 at 64, 0.2 at 256, 0.1 at 512, against extended precision)
 // and there is little to gain; above, a row no longer fits an SM's shared memory.
 constexpr int kNufftMinM = 64, kNufftMaxM = 2048;
+// Nodes the transform is used for.  It costs an FFT per row whatever the number of nodes, the
+// dense product M multiply-adds per row and node.  GB300, us per call, dense / transform:
+// optical sums (two products) at 64 nodes 164 / 195 (M = 64), 339 / 407 (256), 1245 / 1560
+// (1024), 3439 / 4909 (2048), at 96 nodes 685 / 647 (M = 512), 1510 / 1569 (1024); Bastin's
+// (one product) at 128 nodes of one energy 138 / 251 (M = 64), 424 / 1170 (512), 1013 / 2419
+// (1024), at 32 nodes of eight energies 137 / 270, 568 / 1253, 1427 / 2699.  The dense side wins
+// further at small M, but its errors are the larger ones there: the line stays below the
+// default rule's 2 M + 64 nodes.
+constexpr int kNufftMinNodes = 65, kNufftMinNodesBastin = 129, kNufftMinNodesBastinAll = 257;
 
 // Coefficients ((2j-1)/j, (j-1)/j) of the Legendre recurrence
 // P_j = (2j-1)/j z P_{j-1} - (j-1)/j P_{j-2}, j = 1..K.

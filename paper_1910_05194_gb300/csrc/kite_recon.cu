@@ -156,7 +156,7 @@ int reconstruct_dos_impl(kite_ctx* ctx, const double* mu_dev, int M_use, int ker
 // (Eq. conductivity_1st_order in rescaled units).  With e = cos(theta), Delta_m(e) de =
 // (2/pi) cos(m theta) d theta, integrated by Gauss-Legendre quadrature in theta.  Then
 // U[n][k] = sum_m Gamma_nm D[m][k] and W[m][k] = sum_n Gamma_nm D[n][k] (cosine sums at the
-// nodes, kite_nufft.cuh; dense FP64 products outside its range of orders), and per frequency
+// nodes, kite_nufft.cuh; dense FP64 products outside its range of orders and nodes), and per frequency
 // S = sum_k sum_n (g^R_n(e_k + w) U[n][k] + g^A_n(e_k - w) W[n][k]).
 // The CPGF coefficients (Eq. green_function_cheb_expansionb) are geometric in n:
 // g^{s}_n(z) = -2 s i q^n / sqrt(1 - z^2) with q = exp(-s i arccos z) = z - s i sqrt(1 - z^2)
@@ -389,7 +389,7 @@ double theta_fermi(double E_F, const Scale& sc) {
 struct Nufft {
   int M, Nf, L, logN;
   double *inv, *tw, *grid;
-  static bool fits(int M) { return M >= kNufftMinM && M <= kNufftMaxM; }
+  static bool fits(int M) { return M >= kNufftMinM && M <= kNufftMaxM; }  // (and enough nodes)
   explicit Nufft(int M_) : M(M_), Nf(nufft_grid(M_)), L(nufft_row(Nf)), logN(0) {
     while ((1 << logN) < Nf) ++logN;
   }
@@ -421,7 +421,7 @@ int reconstruct_sigma_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, int
                            int kernel, const Scale& sc, double E_F, double kT, double eta,
                            const double* omega_host, int K_w, int n_quad, double* sigma_dev) {
   const int K = n_quad > 0 ? n_quad : 2 * M + 64;
-  const bool fast = Nufft::fits(M);
+  const bool fast = Nufft::fits(M) && K >= kNufftMinNodes;
   Nufft nf(M);
   std::vector<double> in((size_t)K_w + 2);  // rescaled frequencies, then the Fermi energy in E and theta
   for (int i = 0; i < K_w; ++i) in[i] = omega_host[i] / sc.de_minus;
@@ -531,7 +531,7 @@ int reconstruct_sigma_dc_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, 
 // the second term folds into the first: with the Hermitian B_nm = A_nm + conj(A_mn),
 //   Im F_k = Im sum_m dG^R_m(e_k) V[m][k],  V[m][k] = sum_n B_nm D[n][k],
 // D[n][k] = (2/pi) cos(n theta_k) w_k: half the products, and V by the non-uniform transform
-// (kite_nufft.cuh; a dense FP64 product outside its range of orders).  The CPGF terms are
+// (kite_nufft.cuh; a dense FP64 product outside its range of orders and nodes).  The CPGF terms are
 // geometric, g_m = g_0 q^m with q = z - i sqrt(1 - z^2): S0 = sum_m q^m V_m and S1 = sum_m m
 // q^m V_m by Horner's rule and its derivative, sum_m dg_m V_m = g_0 (i S1 / r + z S0 / r^2),
 // r = sqrt(1 - z^2).  sigma = -ucf Im(sum_k F_k), each energy's node sum in a fixed order.
@@ -628,7 +628,8 @@ int reconstruct_sigma_bastin_impl(kite_ctx* ctx, const double* mu_dev, int M_ava
                                   int kernel, double param, const Scale& sc, double eta, double kT,
                                   const double* E_host, int K_E, int n_quad, double* sigma_dev) {
   const int K = n_quad > 0 ? n_quad : 2 * M + 64;
-  const bool fast = Nufft::fits(M);
+  const bool fast =
+      Nufft::fits(M) && (K >= kNufftMinNodesBastin || (long long)K * K_E >= kNufftMinNodesBastinAll);
   Nufft nf(M);
   // nodes per batch of energies: theta, weight, F and the taps, or D and V (dense)
   const size_t per_energy = (size_t)K * (fast ? 3 + kTaps + 1 : 3 + 3 * (size_t)M);

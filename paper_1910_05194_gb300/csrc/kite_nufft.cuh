@@ -110,6 +110,19 @@ __global__ void __launch_bounds__(kGaussBlock) k_gauss_legendre(int K, const dou
 // (E - E_F)/kT = de_minus (cos t - cos theta_F)/kT as a product of sines, whose relative error
 // stays at the rounding for nodes next to the Fermi energy (a difference of cosines divided by
 // a small kT does not); Fermi energies outside the band take the difference.
+__host__ __device__ inline void fermi_node(double u, double w, double E_F, double theta_F, double de_plus,
+                                           double de_minus, double kT, double* theta, double* wq) {
+  const double thF = kT > 0.0 ? 0.0 : theta_F;
+  const double t = thF + (kPi - thF) * 0.5 * u;
+  double v = w * 0.5 * (kPi - thF);
+  if (kT > 0.0) {
+    const double eF = (E_F - de_plus) / de_minus;
+    const double d = fabs(eF) < 1.0 ? -2.0 * sin(0.5 * (t + theta_F)) * sin(0.5 * (t - theta_F)) : cos(t) - eF;
+    v /= (1.0 + exp(d * de_minus / kT));
+  }
+  *theta = t;
+  *wq = v;
+}
 __global__ void k_fermi_nodes(const double* __restrict__ u, const double* __restrict__ w, int K,
                               const double* __restrict__ E_F, const double* __restrict__ theta_F, int K_E,
                               double de_plus, double de_minus, double kT,
@@ -117,16 +130,7 @@ __global__ void k_fermi_nodes(const double* __restrict__ u, const double* __rest
   const int64_t n = (int64_t)K * K_E;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / K), k = (int)(e - (int64_t)i * K);
-    const double thF = kT > 0.0 ? 0.0 : theta_F[i];
-    const double t = thF + (kPi - thF) * 0.5 * u[k];
-    double v = w[k] * 0.5 * (kPi - thF);
-    if (kT > 0.0) {
-      const double eF = (E_F[i] - de_plus) / de_minus;
-      const double d = fabs(eF) < 1.0 ? -2.0 * sin(0.5 * (t + theta_F[i])) * sin(0.5 * (t - theta_F[i])) : cos(t) - eF;
-      v /= (1.0 + exp(d * de_minus / kT));
-    }
-    theta[e] = t;
-    wq[e] = v;
+    fermi_node(u[k], w[k], E_F[i], theta_F[i], de_plus, de_minus, kT, &theta[e], &wq[e]);
   }
 }
 

@@ -380,6 +380,46 @@ void gauss_rule(cudaStream_t st, int K, double* ab, double* u, double* w) {
       K, reinterpret_cast<const double2*>(ab), u, w);
 }
 
+// The rule of few nodes on the host, in the kernel's form (four roots side by side), where the
+// kernel's two launches and its serial chain cost more: Bastin's sum of eight nodes at M = 8
+// takes 87 us so, 107 us with the kernel; of 64 nodes 88 and 107.
+constexpr int kHostRule = 64;
+void gauss_rule_host(int K, double* u, double* w) {
+  double ca[kHostRule], cb[kHostRule];
+  for (int j = 1; j <= K; ++j) ca[j - 1] = (2.0 * j - 1.0) / j, cb[j - 1] = (j - 1.0) / j;
+  const int half = (K + 1) / 2;
+  const double dK = (double)K;
+  for (int i0 = 0; i0 < half; i0 += 4) {
+    double d[4], wt[4];
+    for (int q = 0; q < 4; ++q) {
+      const double sh = sin(0.5 * kPi * (std::min(i0 + q, half - 1) + 0.75) / (dK + 0.5)), c0 = -2.0 * sh * sh;
+      d[q] = c0 - (0.125 / (dK * dK) - 0.125 / (dK * dK * dK)) * (1.0 + c0);
+    }
+    bool done = false;
+    for (int it = 0; it < 9 && !done; ++it) {
+      double p[4] = {1.0, 1.0, 1.0, 1.0}, D[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int j = 0; j < K; ++j)
+        for (int q = 0; q < 4; ++q) {
+          D[q] = cb[j] * D[q] + (ca[j] * d[q]) * p[q];
+          p[q] += D[q];
+        }
+      done = true;
+      for (int q = 0; q < 4; ++q) {
+        const double om = -d[q] * (2.0 + d[q]), dp = -dK * (d[q] * p[q] + D[q]) / om, dz = p[q] / dp;
+        wt[q] = 2.0 / (om * dp * dp) * (1.0 + 2.0 * (1.0 + d[q]) * dz / om);
+        d[q] -= dz;
+        done = done && !(fabs(dz) > 4e-9 * om);
+      }
+    }
+    for (int q = 0; q < 4 && i0 + q < half; ++q) {
+      const int i = i0 + q;
+      u[K - 1 - i] = 2.0 + d[q];
+      u[i] = -d[q];
+      w[i] = w[K - 1 - i] = wt[q];
+    }
+  }
+}
+
 // The Fermi energy in theta (the lower end of the sea at T = 0).
 double theta_fermi(double E_F, const Scale& sc) {
   return acos(fmin(1.0, fmax(-1.0, (E_F - sc.de_plus) / sc.de_minus)));
@@ -423,13 +463,21 @@ int reconstruct_sigma_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, int
   const int K = n_quad > 0 ? n_quad : 2 * M + 64;
   const bool fast = Nufft::fits(M) && K >= kNufftMinNodes;
   Nufft nf(M);
-  std::vector<double> in((size_t)K_w + 2);  // rescaled frequencies, then the Fermi energy in E and theta
+  // rescaled frequencies, then the Fermi energy in E and theta, then few nodes and their weights
+  const size_t Kp = ((size_t)K + 1) / 2 * 2, Wp = ((size_t)K_w + 3) / 2 * 2;
+  std::vector<double> in(Wp + (K <= kHostRule ? 2 * Kp : 0));
   for (int i = 0; i < K_w; ++i) in[i] = omega_host[i] / sc.de_minus;
   in[K_w] = E_F;
   in[K_w + 1] = theta_fermi(E_F, sc);
+  const bool on_host = K <= kHostRule;
+  if (on_host) {
+    double *th = in.data() + Wp, *wq = th + Kp;
+    gauss_rule_host(K, th, wq);
+    for (int k = 0; k < K; ++k)
+      fermi_node(th[k], wq[k], E_F, in[K_w + 1], sc.de_plus, sc.de_minus, kT, &th[k], &wq[k]);
+  }
   // all offsets even: 16-byte aligned complex values
-  const size_t nU = 2 * (size_t)M * K, Kp = ((size_t)K + 1) / 2 * 2, Wp = ((size_t)K_w + 3) / 2 * 2,
-               Mp = ((size_t)M + 1) / 2 * 2;
+  const size_t nU = 2 * (size_t)M * K, Mp = ((size_t)M + 1) / 2 * 2;
   const int blocks = (K + 127) / 128;
   const size_t nPart = 4 * (size_t)K_w * blocks;
   const size_t nDense = 2 * (size_t)M * M + (size_t)M * Kp;       // Gamma, D
@@ -439,21 +487,24 @@ int reconstruct_sigma_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, int
   KITE_CUDA_TRY(ctx, cudaMallocAsync((void**)&buf, total * sizeof(double), ctx->stream));
   double* U = buf;
   double* W = U + nU;
-  double* th_d = W + nU;
-  double* wq_d = th_d + Kp;
-  double* gx = wq_d + Kp;
+  double* gab = W + nU;
+  double* gx = gab + 2 * Kp;
   double* gw = gx + Kp;
-  double* gab = gw + Kp;
-  double* in_d = gab + 2 * Kp;
-  double* wk = in_d + Wp;
+  double* in_d = gw + Kp;
+  double* th_d = in_d + Wp;
+  double* wq_d = th_d + Kp;
+  double* wk = wq_d + Kp;
   double* part = wk + Mp;
   double* rest = part + nPart;
   cudaStream_t st = ctx->stream;
   cudaError_t e = cudaMemcpyAsync(in_d, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice, st);
   int rc = e == cudaSuccess ? KITE_OK : cuda_fail(ctx, e, "sigma set-up");
   if (rc == KITE_OK) {
-    gauss_rule(st, K, gab, gx, gw);
-    k_fermi_nodes<<<(K + 255) / 256, 256, 0, st>>>(gx, gw, K, in_d + K_w, in_d + K_w + 1, 1, sc.de_plus, sc.de_minus, kT, th_d, wq_d);
+    if (!on_host) {
+      gauss_rule(st, K, gab, gx, gw);
+      k_fermi_nodes<<<(K + 255) / 256, 256, 0, st>>>(gx, gw, K, in_d + K_w, in_d + K_w + 1, 1, sc.de_plus, sc.de_minus,
+                                                     kT, th_d, wq_d);
+    }
     if (fast) {
       nf.carve(rest);
       double* taps = rest + (nf.doubles(2 * M) + 2) / 2 * 2;
@@ -655,12 +706,17 @@ int reconstruct_sigma_bastin_impl(kite_ctx* ctx, const double* mu_dev, int M_ava
   cudaStream_t st = ctx->stream;
   const double ucf = lattice == KITE_HONEYCOMB ? 4.0 / sqrt(3.0) : 1.0;
   k_dc_weights<<<(M + 63) / 64, 64, 0, st>>>(M, kernel, param, wk);
-  gauss_rule(st, K, gab, gx, gw);
-  std::vector<double> thF((size_t)K_E);
-  for (int i = 0; i < K_E; ++i) thF[i] = theta_fermi(E_host[i], sc);
-  cudaError_t e = cudaMemcpyAsync(E_d, E_host, (size_t)K_E * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(thF_d, thF.data(), (size_t)K_E * sizeof(double), cudaMemcpyHostToDevice, st);
+  // the Fermi energies in E and theta, then the rule of few nodes
+  std::vector<double> in(2 * Ep + (K <= kHostRule ? 2 * Kp : 0));
+  for (int i = 0; i < K_E; ++i) {
+    in[i] = E_host[i];
+    in[Ep + i] = theta_fermi(E_host[i], sc);
+  }
+  if (K <= kHostRule)
+    gauss_rule_host(K, in.data() + 2 * Ep, in.data() + 2 * Ep + Kp);
+  else
+    gauss_rule(st, K, gab, gx, gw);
+  cudaError_t e = cudaMemcpyAsync(E_d, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice, st);
   int rc = KITE_OK;
   if (fast) {
     nf.carve(mid);

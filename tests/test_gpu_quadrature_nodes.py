@@ -1,6 +1,7 @@
 """The conductivity reconstructions on both sides of the number of quadrature nodes where their
 cosine sums change path (dense products below 65 nodes in the optical sums, below 129 nodes of
-one energy and 257 of all in Bastin's), against the oracle's direct sums at the bars of
+one energy and 257 of all in Bastin's) and the rule moves from the host to the device (65
+nodes), against the oracle's direct sums at the bars of
 test_gpu_sigma.py and test_gpu_hall.py (1e-9 and 1e-10 of the largest value)."""
 import numpy as np
 import pytest
@@ -29,7 +30,7 @@ def moments(M, seed, hermitian):
 
 
 @pytest.mark.parametrize("M", [64, 100, 321])
-@pytest.mark.parametrize("n_quad,kT", [(1, 0.0), (2, 0.05), (17, 0.0), (64, 0.0), (64, 0.05), (65, 0.0), (66, 0.05)])
+@pytest.mark.parametrize("n_quad,kT", [(1, 0.0), (2, 0.05), (17, 0.0), (63, 0.0), (64, 0.0), (64, 0.05), (65, 0.0), (66, 0.05)])
 def test_optical_conductivity_with_few_nodes(ctx, M, n_quad, kT):
     mu, om = moments(M, M, True), np.linspace(0.3, 9.0, 5)
     out = np.zeros(5, np.complex128)

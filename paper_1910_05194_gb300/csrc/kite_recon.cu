@@ -553,8 +553,11 @@ int reconstruct_sigma_dc_impl(kite_ctx* ctx, const double* mu_dev, int M_avail, 
                               double* w) {
   cudaStream_t st = ctx->stream;
   k_dc_weights<<<(M + 63) / 64, 64, 0, st>>>(M, kernel, param, w);
-  // few energies: wide blocks, so that each one's SM has enough warps in flight
-  const int block = K < 2 * ctx->num_sms ? 1024 : 256;
+  // Few energies and long rows: wide blocks, so that each one's SM has enough warps in flight.
+  // us per call with 256 / 512 / 1024 threads: M = 4096, 48 energies 6880 / 4413 / 4421, M = 2048
+  // 1273 / 1207 / 1212, M = 1024 371 / 369 / 379, M = 64 50 / 53 / 60; more energies than SMs, M =
+  // 2048 2365 / 2369 / 2383.
+  const int block = K <= ctx->num_sms && M >= 1536 ? 512 : 256;
   const size_t smem = sizeof(double) * ((size_t)M + block / 32);
   if (smem > 48 * 1024)
     KITE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_sigma_dc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

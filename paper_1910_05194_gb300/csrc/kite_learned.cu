@@ -47,8 +47,11 @@ namespace {
 constexpr int IN = KITE_MLP_IN, OUT = KITE_MLP_OUT;
 constexpr double kSdFloor = 1e-4;
 // Largest fallback order that takes every flagged row in one launch (its table of Chebyshev
-// polynomials is 4 KiB per order); above, row by row.
-constexpr int kBatchPlainMax = 8192;
+// polynomials is 4 KiB per order); above, row by row.  A single flagged row takes the table only
+// up to kTablePlainMax: us per call of one row, table / row by row: 218 / 228 at order 128,
+// 275 / 260 at 512, 492 / 383 at 2048, 1344 / 847 at 8192; of two rows 283 / 338 at 512, 491 / 570
+// at 2048, 1330 / 1497 at 8192.
+constexpr int kBatchPlainMax = 8192, kTablePlainMax = 256;
 
 // A model's device buffers (params, shift, scale) in one allocation.
 int new_model(kite_ctx* ctx, double e_min, double e_max, kite_model** out) {
@@ -206,7 +209,7 @@ int kite_learned_dos(kite_ctx* ctx, const kite_model* model, const double* mu, i
   // 3. the plain path for every flagged row, on the model's grid
   int flagged = 0;
   for (int i = 0; i < n; ++i) flagged += flags[i] != 0;
-  if (rc == KITE_OK && flagged > 0 && !systems && M_plain <= kBatchPlainMax) {
+  if (rc == KITE_OK && flagged > 0 && !systems && M_plain <= (flagged == 1 ? kTablePlainMax : kBatchPlainMax)) {
     std::vector<int> rows;
     for (int i = 0; i < n; ++i)
       if (flags[i]) rows.push_back(i);

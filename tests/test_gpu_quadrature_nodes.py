@@ -49,3 +49,24 @@ def test_bastin_conductivity_with_few_nodes(ctx, M, n_quad, K, kT):
                                      n_quad)
     ref = oracle.sigma_dc_bastin(mu, E, LO, HI, 0.3, 1, kernel="lorentz", lam=3.0, kT=kT, n_quad=n_quad)
     assert np.max(np.abs(out - ref)) <= 1e-10 * max(1.0, np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("M,n_quad", [(2047, 70), (2048, 65), (2048, 64), (2049, 70), (256, 333), (257, 333)])
+def test_optical_conductivity_at_the_transforms_edges(ctx, M, n_quad):
+    """The largest order of the transform (8192 grid points, 128 KB of shared memory a row), the
+    dense products above it, and the orders between which the grid gets coarser (256, 257)."""
+    mu, om = moments(M, M, True), np.linspace(0.3, 9.0, 2)
+    out = np.zeros(2, np.complex128)
+    kite.reconstruct_sigma(ctx, mu, M, M, kite.HONEYCOMB, kite.KERNEL_JACKSON, LO, HI, 0.4, 0.0, 0.2, om, 2, out, n_quad)
+    ref = oracle.sigma_xx(mu, om, LO, HI, 0.4, 0.2, 0, kernel="jackson", n_quad=n_quad)
+    assert np.max(np.abs(out - ref)) <= 1e-9 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("M,n_quad", [(2047, 140), (2048, 129), (2048, 128), (2049, 140), (256, 333), (257, 333)])
+def test_bastin_conductivity_at_the_transforms_edges(ctx, M, n_quad):
+    mu, E = moments(M, M + 1, False), np.array([1.3])
+    out = np.zeros(1)
+    kite.reconstruct_sigma_dc_bastin(ctx, mu, M, M, kite.SQUARE, kite.KERNEL_LORENTZ, 3.0, LO, HI, 0.3, 0.0, E, 1, out,
+                                     n_quad)
+    ref = oracle.sigma_dc_bastin(mu, E, LO, HI, 0.3, 1, kernel="lorentz", lam=3.0, n_quad=n_quad)
+    assert np.max(np.abs(out - ref)) <= 1e-10 * max(1.0, np.max(np.abs(ref)))

@@ -420,11 +420,13 @@ inline bool autotune_enabled() {
   return !(e && e[0] == '0');
 }
 
-// Milliseconds of three launches of a candidate, the better of two timings after a warm-up:
-// the shape chosen sets the grouping of the FP32 moment sums, so one late launch should not
-// decide between two close candidates.
+// Milliseconds per recursion step of a candidate, from three launches after a warm-up.  The shape
+// chosen sets the grouping of the FP32 moment sums, so one late launch should not decide between
+// two close candidates: a first timing below `again` is taken a second time and the better one
+// counts.  (All candidates twice: a new size's first call took up to 1.4 times as long as with
+// one timing, 20.3 against 14.9 ms at 1300^2 square cells, M = 128, R = 8.)
 template <typename Launch>
-float time_launches(kite_ctx* ctx, Launch launch) {
+float time_launches(kite_ctx* ctx, Launch launch, int steps_per_launch, float again) {
   launch();  // warm-up
   float best = 1e30f;
   for (int rep = 0; rep < 2; ++rep) {
@@ -434,9 +436,16 @@ float time_launches(kite_ctx* ctx, Launch launch) {
     float ms = 1e30f;
     if (cudaEventSynchronize(ctx->ev3) != cudaSuccess || cudaEventElapsedTime(&ms, ctx->ev2, ctx->ev3) != cudaSuccess)
       return 1e30f;
-    best = std::min(best, ms);
+    best = std::min(best, ms / (3.0f * (float)steps_per_launch));
+    if (!(best < again)) break;
   }
   return best;
+}
+// `again` for a candidate of the sweep while the best one so far takes `best` ms: FP64 sums may be
+// grouped freely, one timing does.
+template <typename Real>
+constexpr float time_again(float best = 1e30f) {
+  return sizeof(Real) == 4 ? 1.25f * best : 0.0f;
 }
 
 // KITE_PASS_STEPS=1, 2 or 3 pins the steps per pass of the plain moment sweep (the
@@ -453,11 +462,11 @@ int step2_grid(kite_ctx* ctx, long long units, int ctas_per_sm = 0) {
   return (int)std::max(1LL, std::min((long long)ctx->num_sms * k, units));
 }
 
-// Seconds per recursion step of the two-step pass (DBL: its doubling form): three launches
-// = six steps.
+// Milliseconds per recursion step of the two-step pass (DBL: its doubling form).
 template <typename Real, int LAT, int C, int NST, bool DBL = false>
 float time_candidate2(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt,
-                      void* r0, void* bA, void* bB, void* bC, void* bD, double* partial) {
+                      void* r0, void* bA, void* bB, void* bC, void* bD, double* partial,
+                      float again = time_again<Real>()) {
   constexpr int SMEM = Step2Shape<LAT, C, NST, DBL>::SMEM;
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = step2_grid<Real, LAT, C, NST, DBL>(ctx, units, k);
@@ -468,7 +477,7 @@ float time_candidate2(kite_ctx* ctx, int k, long long units, const Plan& p, cons
         partial + (size_t)3 * G * Q, ctx->d_status, p.realv ? 1 : 0,
         DBL ? partial + (size_t)4 * G * Q : nullptr, DBL ? partial + (size_t)5 * G * Q : nullptr);
   };
-  return time_launches(ctx, launch) / 6.0f;
+  return time_launches(ctx, launch, 2, again);
 }
 
 template <typename Real, int LAT, int C, int NST>
@@ -478,10 +487,11 @@ int step3_grid(kite_ctx* ctx, long long units, int ctas_per_sm = 0) {
   return (int)std::max(1LL, std::min((long long)ctx->num_sms * k, units));
 }
 
-// Seconds per recursion step of the three-step pass: three launches = nine steps.
+// Milliseconds per recursion step of the three-step pass.
 template <typename Real, int LAT, int C, int NST>
 float time_candidate3(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt,
-                      void* r0, void* bA, void* bB, void* bC, void* bD, double* partial) {
+                      void* r0, void* bA, void* bB, void* bC, void* bD, double* partial,
+                      float again = time_again<Real>()) {
   constexpr int SMEM = Step3Shape<LAT, C, NST>::SMEM;
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = step3_grid<Real, LAT, C, NST>(ctx, units, k);
@@ -491,12 +501,12 @@ float time_candidate3(kite_ctx* ctx, int k, long long units, const Plan& p, cons
         bA, bB, bC, bD, r0, vt, tt, p.Lx, p.Ly, units, partial + (size_t)2 * G * Q,
         partial + (size_t)3 * G * Q, partial + (size_t)4 * G * Q, ctx->d_status, p.realv ? 1 : 0);
   };
-  return time_launches(ctx, launch) / 9.0f;
+  return time_launches(ctx, launch, 3, again);
 }
 
 template <typename Real, int LAT, int C, int MODE, int NST>
 float time_candidate(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt, void* r0,
-                     void* bA, void* bB, double* partial) {
+                     void* bA, void* bB, double* partial, float again = time_again<Real>()) {
   constexpr int SMEM = StepShape<LAT, C, NST>::template smem_bytes<MODE>();
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = grid_for<Real, LAT, C, false, MODE, NST>(ctx, units, k);
@@ -507,7 +517,7 @@ float time_candidate(kite_ctx* ctx, int k, long long units, const Plan& p, const
         bA, bB, bA, MODE == 0 ? r0 : nullptr, vt, tt, p.Lx, p.Ly, units, partial + (size_t)2 * G * Q,
         MODE == 3 ? partial + (size_t)G * Q : nullptr, ctx->d_status, 0, FamOut{}, p.realv ? 1 : 0, SeriesOut{}, nullptr, p.open);
   };
-  return time_launches(ctx, launch) / 3.0f;  // per recursion step
+  return time_launches(ctx, launch, 1, again);
 }
 
 // The two-step pass is a candidate of the plain moment sweep (MODE 0) and of the doubling
@@ -569,11 +579,13 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
   if (!two_only && !three_only) {
     const int o8 = step_occupancy<Real, LAT, C, MODE, 8>(), o4 = step_occupancy<Real, LAT, C, MODE, 4>();
     for (int k = 1; k <= o8; ++k) {
-      const float ms = time_candidate<Real, LAT, C, MODE, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, partial);
+      const float ms = time_candidate<Real, LAT, C, MODE, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, partial,
+                                                             time_again<Real>(best_ms));
       if (ms < best_ms) best_ms = ms, best = Tune{8, k, 0};
     }
     for (int k = 1; k <= o4; ++k) {
-      const float ms = time_candidate<Real, LAT, C, MODE, 4>(ctx, k, units, p, vt, tt, r0, bA, bB, partial);
+      const float ms = time_candidate<Real, LAT, C, MODE, 4>(ctx, k, units, p, vt, tt, r0, bA, bB, partial,
+                                                             time_again<Real>(best_ms));
       if (ms < best_ms * 0.98f) best_ms = ms, best = Tune{4, k, 0};  // prefer the deeper ring on a tie
     }
   }
@@ -585,15 +597,18 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
     const int o8 = step2_occupancy<Real, LAT, C, 8, DB>(), o6 = step2_occupancy<Real, LAT, C, 6, DB>(),
               o5 = step2_occupancy<Real, LAT, C, 5, DB>();
     for (int k = 1; k <= o8; ++k) {
-      const float ms = time_candidate2<Real, LAT, C, 8, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial);
+      const float ms = time_candidate2<Real, LAT, C, 8, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
+                                                            time_again<Real>(best2));
       if (ms < best2) best2 = ms, best = Tune{8, k, 1};
     }
     for (int k = 1; k <= o6; ++k) {
-      const float ms = time_candidate2<Real, LAT, C, 6, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial);
+      const float ms = time_candidate2<Real, LAT, C, 6, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
+                                                            time_again<Real>(best2));
       if (ms < best2 * 0.98f) best2 = ms, best = Tune{6, k, 1};
     }
     for (int k = 1; k <= o5; ++k) {
-      const float ms = time_candidate2<Real, LAT, C, 5, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial);
+      const float ms = time_candidate2<Real, LAT, C, 5, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
+                                                            time_again<Real>(best2));
       if (ms < best2 * 0.98f) best2 = ms, best = Tune{5, k, 1};
     }
   }
@@ -601,11 +616,13 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
     float best3 = 1e30f;
     const int o8 = step3_occupancy<Real, LAT, C, 8>(), o7 = step3_occupancy<Real, LAT, C, 7>();
     for (int k = 1; k <= o8; ++k) {
-      const float ms = time_candidate3<Real, LAT, C, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial);
+      const float ms = time_candidate3<Real, LAT, C, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
+                                                          time_again<Real>(best3));
       if (ms < best3) best3 = ms, best = Tune{8, k, 2};
     }
     for (int k = 1; k <= o7; ++k) {
-      const float ms = time_candidate3<Real, LAT, C, 7>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial);
+      const float ms = time_candidate3<Real, LAT, C, 7>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
+                                                          time_again<Real>(best3));
       if (ms < best3 * 0.98f) best3 = ms, best = Tune{7, k, 2};
     }
   }
@@ -1109,7 +1126,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
         if (cl.cs > 0) return cluster_step_ms(ctx, cl);
         if (p.field) {
           FieldSweep f = fs;
-          f.M = std::min(p.M, 33);
+          f.M = std::min(p.M, 9);
           if (field_sweep(ctx, &f) != KITE_OK || field_sweep(ctx, &f) != KITE_OK || f.launches < 1) return 1e30f;
           return (float)(1e3 * f.seconds / (double)f.launches);
         }

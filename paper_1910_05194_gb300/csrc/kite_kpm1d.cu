@@ -664,14 +664,21 @@ inline int cluster_ctas_pinned() {
 }
 constexpr int kClusterTimeSteps = 40;  // longest timing run of the autotuner
 
-// Per-step seconds of the cluster sweep: two timing runs, 8 and 40 steps, so that the
-// launch and load cost drops out.
-inline float cluster_step_ms(kite_ctx* ctx, ClusterSweep c) {
-  if (cluster_sweep(ctx, &c, 8) != KITE_OK) return 1e30f;
-  if (cluster_sweep(ctx, &c, 8) != KITE_OK) return 1e30f;
+// Milliseconds of a batch's sweep: per recursion step, and what a sweep costs besides (launch and
+// load; 0 where it hides behind the steps).
+struct SweepCost {
+  float step, fixed;
+};
+
+// Cost of the cluster sweep: two timing runs, 8 and 40 steps, so that the launch and load cost
+// drops out of the step's.
+inline SweepCost cluster_cost(kite_ctx* ctx, ClusterSweep c) {
+  if (cluster_sweep(ctx, &c, 8) != KITE_OK) return {1e30f, 0.0f};
+  if (cluster_sweep(ctx, &c, 8) != KITE_OK) return {1e30f, 0.0f};
   const double t8 = c.seconds;
-  if (cluster_sweep(ctx, &c, kClusterTimeSteps) != KITE_OK) return 1e30f;
-  return (float)(1e3 * std::max(0.0, c.seconds - t8) / (kClusterTimeSteps - 8));
+  if (cluster_sweep(ctx, &c, kClusterTimeSteps) != KITE_OK) return {1e30f, 0.0f};
+  const float step = (float)(1e3 * std::max(0.0, c.seconds - t8) / (kClusterTimeSteps - 8));
+  return {step, std::max(0.0f, (float)(1e3 * t8) - 8.0f * step)};
 }
 
 // Cluster size to run the batch with, 0 for the streaming kernels.  `stream_ms` times the
@@ -719,7 +726,7 @@ int cluster_choice(kite_ctx* ctx, const Plan& p, const ClusterSweep& c, long lon
   for (int k = 0; k < nc; ++k) {
     ClusterSweep t = c;
     t.cs = cand[k];
-    const float ms = cluster_step_ms(ctx, t);
+    const float ms = cluster_cost(ctx, t).step;
     if (ms < best) best = ms, pick = cand[k];
   }
   cudaGetLastError();
@@ -739,11 +746,20 @@ inline int resident_pinned() {  // 0 unset, 1 off, 2 on
 // kernels run.
 constexpr size_t kResidentPartMax = (size_t)2 << 30;
 
-// Whether to run the batch resident.  `other_ms` times the kernels chosen otherwise, per
-// recursion step of the batch.  The verdict is kept with the tuned shapes: {1 or 0, n}; {-1, n}
-// after a failure (a launch refused, a wait that ran out, or a short timing run that took as long
-// as the long one), n failures so far.  A failure decides nothing: the next call times again,
-// until kResidentTries of them have shown that this GPU's SMs are not to be had.
+// Whether to run the batch resident.  `other_cost` times the kernels chosen otherwise.  The
+// verdict is kept with the tuned shapes: {fewest recursion steps from which the sweep is taken,
+// n}; {-1, n} after a failure (a launch refused, a wait that ran out, or a short timing run that
+// took as long as the long one), n failures so far.  A failure decides nothing: the next call
+// times again, until kResidentTries of them have shown that this GPU's SMs are not to be had.
+//
+// A sweep's launch, record memset and load cost 8 to 20 us and its host part and reduction about
+// 10 us more than the other kernels' (the timing runs do not see those), which a few faster steps
+// do not bring in: at 64 x 64 honeycomb cells, FP64, R = 4 a step takes 1.86 us on chip and 2.26 us
+// in clusters, and calls of M = 4 .. 16 took 5 to 7 % longer with it; 300 x 300 square cells, FP32,
+// R = 4, M = 4 149 -> 169 us.  Fewer than kResidentMinSteps steps hardly gain at any size (at best
+// 9 us a step) and are neither taken nor timed (the timing runs take 56 to 104 steps).
+constexpr float kResidentExtraMs = 0.010f;
+constexpr int kResidentMinSteps = 8;
 constexpr int kResidentTries = 3;
 
 inline uint64_t resident_key(const ResidentSweep& r) {
@@ -761,42 +777,49 @@ inline void resident_failed(kite_ctx* ctx, const ResidentSweep& r) {
 }
 
 // 1: resident, 0: not, -1: not, and a timing run failed.
-template <typename OtherMs>
-int resident_choice(kite_ctx* ctx, const ResidentSweep& r, OtherMs other_ms) {
+template <typename OtherCost>
+int resident_choice(kite_ctx* ctx, const ResidentSweep& r, int steps, OtherCost other_cost) {
   if (resident_pinned() == 2) return 1;
   const uint64_t key = resident_key(r);
   int failures = 0;
   auto it = ctx->tune.find(key);
   if (it != ctx->tune.end()) {
-    if (it->second.first >= 0) return it->second.first;
+    if (it->second.first >= 0) return steps >= it->second.first;
     failures = it->second.second;
     if (failures >= kResidentTries) return 0;
   }
-  // two timing runs, so that the launch and load cost drops out; the best of two each
+  // two timing runs, so that the launch and load cost drops out: the better of two short ones,
+  // and a second long one only where the first did not win (a late launch makes it look slower)
   const std::string last_error = ctx->last_error;  // (a failed timing is no failed call)
   bool ok = true;
+  const int per_sweep = r.plan.CR * r.plan.vecs, sweeps = (r.nvec + per_sweep - 1) / per_sweep;
   auto timed = [&](int steps) {
-    double best = 1e30;
-    for (int k = 0; k < 2 && ok; ++k) {
-      ResidentSweep t = r;
-      ok = resident_sweep(ctx, &t, steps) == KITE_OK;
-      best = std::min(best, t.seconds);
-    }
-    return best;
+    ResidentSweep t = r;
+    ok = ok && resident_sweep(ctx, &t, steps) == KITE_OK;
+    return t.seconds;
   };
-  const double t8 = timed(8), t40 = timed(kClusterTimeSteps);
+  constexpr int kNever = 1 << 30;
+  int from = kNever;
+  SweepCost other{0.0f, 0.0f};
+  timed(8);  // warm-up
+  for (int rep = 0; rep < 2 && ok && from == kNever; ++rep) {
+    const double t8 = timed(8), t40 = timed(kClusterTimeSteps);
+    ok = ok && t40 > t8;
+    if (ok && rep == 0) other = other_cost();
+    const float step = (float)(1e3 * (t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
+    if (ok && step < 0.95f * other.step) {  // it must win clearly
+      const float more = (float)(1e3 * t8 * sweeps) - 8.0f * step - other.fixed + kResidentExtraMs;
+      from = (int)std::min(1e6f, std::max(0.0f, more / (other.step - step)));
+    }
+  }
   cudaGetLastError();
-  if (!ok || t40 <= t8) {
+  if (!ok) {
     ctx->last_error = last_error;
     resident_failed(ctx, r);
     return -1;
   }
-  const int per_sweep = r.plan.CR * r.plan.vecs, sweeps = (r.nvec + per_sweep - 1) / per_sweep;
-  const float ms = (float)(1e3 * (t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
-  const int pick = ms < 0.95f * other_ms() ? 1 : 0;  // it must win clearly
-  cudaGetLastError();
-  ctx->tune[key] = {pick, failures};
-  return pick;
+  ctx->tune[key] = {from, failures};
+  return steps >= from;
 }
 
 template <typename Real, int LAT>
@@ -1120,15 +1143,16 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
         return C == 1 ? one(std::integral_constant<int, 1>{})
                       : (C == 2 ? one(std::integral_constant<int, 2>{}) : one(std::integral_constant<int, 4>{}));
       };
-      // the kernels that run otherwise, per recursion step: the cluster sweep, the field
-      // sweep, or the streaming kernel of the tuned shape
-      auto other_ms = [&]() -> float {
-        if (cl.cs > 0) return cluster_step_ms(ctx, cl);
+      // the kernels that run otherwise: the cluster sweep, the field sweep, or the streaming
+      // kernel of the tuned shape
+      auto other_cost = [&]() -> SweepCost {
+        if (cl.cs > 0) return cluster_cost(ctx, cl);
         if (p.field) {
           FieldSweep f = fs;
           f.M = std::min(p.M, 9);
-          if (field_sweep(ctx, &f) != KITE_OK || field_sweep(ctx, &f) != KITE_OK || f.launches < 1) return 1e30f;
-          return (float)(1e3 * f.seconds / (double)f.launches);
+          if (field_sweep(ctx, &f) != KITE_OK || field_sweep(ctx, &f) != KITE_OK || f.launches < 1)
+            return {1e30f, 0.0f};
+          return {(float)(1e3 * f.seconds / (double)f.launches), 0.0f};
         }
         auto one = [&](auto cc) -> float {
           constexpr int CC = decltype(cc)::value;
@@ -1147,8 +1171,10 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
           };
           return p.doubling ? mode(std::integral_constant<int, 3>{}) : mode(std::integral_constant<int, 0>{});
         };
-        return C == 1 ? one(std::integral_constant<int, 1>{})
-                      : (C == 2 ? one(std::integral_constant<int, 2>{}) : one(std::integral_constant<int, 4>{}));
+        const float ms = C == 1   ? one(std::integral_constant<int, 1>{})
+                         : C == 2 ? one(std::integral_constant<int, 2>{})
+                                  : one(std::integral_constant<int, 4>{});
+        return {ms, 0.0f};
       };
       const bool want_last = kpm->r_last && !p.doubling;
       rs.want_last = want_last;
@@ -1160,11 +1186,11 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       const bool pinned_res = resident_pinned() == 2;
       const bool may_reside =
           resident_rec != 0 && !resident_off &&
-          (pinned_res || (!ctx->debug_stall && autotune_enabled() && !pass_steps_pinned() && !getenv("KITE_TUNE") &&
-                          cluster_pinned() != 2));
+          (pinned_res || (steps_for(p) >= kResidentMinSteps && !ctx->debug_stall && autotune_enabled() &&
+                          !pass_steps_pinned() && !getenv("KITE_TUNE") && cluster_pinned() != 2));
       if (may_reside && (sizeof(Real) == 8 || cl.cs == 0 || pinned_res))
         rs.plan = resident_for(C, sizeof(Real) == 8 ? 0 : (p.field ? fs.G : tuned_grid()));
-      const int choice = rs.plan.CR ? resident_choice(ctx, rs, other_ms) : 0;
+      const int choice = rs.plan.CR ? resident_choice(ctx, rs, steps_for(p), other_cost) : 0;
       if (choice < 0) resident_off = true;
       bool resident = choice > 0;
       if (resident) {

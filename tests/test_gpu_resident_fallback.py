@@ -98,6 +98,20 @@ def test_a_sweep_that_keeps_failing_is_tried_once_a_call_and_three_times_in_all(
         assert block == stream and np.array_equal(per, ref)
 
 
+@pytest.mark.parametrize("precision", [kite.FP32, kite.FP64])
+@pytest.mark.parametrize("d", LATTICES)
+@pytest.mark.parametrize("M", [4, 8])
+def test_a_short_sweep_is_not_taken_on_chip(d, precision, M):
+    """Fewer than eight steps: the sweep's launch and load cost more than the steps gain."""
+    with fresh(d, precision) as (ctx, _, stream, chip):
+        with env(KITE_RESIDENT="0"):
+            ref, block = call(ctx, d, precision, 4, M)
+        for _ in range(2):
+            per, short = call(ctx, d, precision, 4, M)
+            assert block == short == stream and np.array_equal(per, ref)
+            assert call(ctx, d, precision)[1] == chip  # 63 steps
+
+
 @pytest.mark.parametrize("kind,skip,count", [(0, 0, 1), (3, 0, 1), (1, -1, 1), (2, 0, -1)])
 def test_the_hook_refuses_what_it_does_not_know(kind, skip, count):
     with kite.Context(0) as ctx, pytest.raises(kite.KiteError) as e:

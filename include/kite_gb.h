@@ -168,7 +168,9 @@ typedef struct {
                            imaginary part, which vanishes for a Hermitian H~, and read 0) */
   double e_min, e_max;  /* bounds used (eV)                                          */
   int64_t n_eff;        /* non-vacant orbitals of the last realisation               */
-  int32_t grid, block;  /* launch shape of the sweep kernel                           */
+  int32_t grid, block;  /* launch shape of the sweep kernel: block is 256 for the streaming
+                           and the cluster sweep, more where the on-chip sweep of mid-size
+                           lattices ran (its compute and exchange threads)               */
   double step_seconds;  /* device time of the recursion-step launches alone          */
   int64_t step_launches;/* number of recursion-step launches timed in step_seconds (the
                            on-chip sweep of mid-size lattices counts its recursion steps)  */
@@ -259,7 +261,9 @@ int kite_flux_nearest(const kite_system* sys, double flux, double* out);
  * to about 1.5 million orbitals in FP32) may run the sweep on chip as well, one region of the
  * lattice per SM in one cooperative launch whose CTAs wait on their neighbours within a
  * bound; it keeps the streaming launch's grouping of the FP32 moment sums.  Chosen where
- * measured faster; KITE_RESIDENT=0 / 1 forbids / forces it.  Where it cannot run (its launch
+ * measured faster for the call's number of steps; KITE_RESIDENT=0 / 1 forbids / forces it.
+ * Its moment partials may take 2 GiB of work space (about M = 13800 for eight FP32 vectors);
+ * longer sweeps stream, as calls do that find no room for them.  Where it cannot run (its launch
  * is refused, or a wait runs out because another long kernel holds its SMs), the kernels
  * chosen otherwise take that batch of vectors and the rest of the call; after three such
  * failures of a size the context no longer tries it there, unless KITE_RESIDENT=1.

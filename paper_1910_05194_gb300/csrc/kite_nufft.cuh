@@ -91,8 +91,11 @@ __global__ void __launch_bounds__(kGaussBlock) k_gauss_legendre(int K, const dou
     // (P_K, D_K): the image of (P_0, D_0) = (1, 0); (1 - z^2) P'_K = K (P_{K-1} - z P_K)
     const double om = -d * (2.0 + d);  // 1 - z^2
     const double dp = -dK * fma(d, a1, a0) / om, dz = a1 / dp;
-    // the weight 2 / ((1 - z^2) P'^2) at the root, from its logarithmic derivative there
-    wt = 2.0 / (om * dp * dp) * (1.0 + 2.0 * (1.0 + d) * dz / om);
+    // the weight 2 / ((1 - z^2) P'^2) at the root, from its logarithmic derivative at z,
+    // (-2 z + 2 K (K + 1) dz) / (1 - z^2) (Legendre's equation): without the second term the
+    // last step, up to 4e-9, left every weight too large, by 6e-14 at most and 1 to 3e-15 in the
+    // sum at K = 66 .. 192
+    wt = 2.0 / (om * dp * dp) * (1.0 + dz * fma(-dK * (dK + 1.0), dz, 2.0 * (1.0 + d)) / om);
     d -= dz;
     // the next step would be below z / om * dz^2
     if (__all_sync(0xffffffffu, !(fabs(dz) > 4e-9 * om))) break;

@@ -406,7 +406,7 @@ void gauss_rule_host(int K, double* u, double* w) {
       done = true;
       for (int q = 0; q < 4; ++q) {
         const double om = -d[q] * (2.0 + d[q]), dp = -dK * (d[q] * p[q] + D[q]) / om, dz = p[q] / dp;
-        wt[q] = 2.0 / (om * dp * dp) * (1.0 + 2.0 * (1.0 + d[q]) * dz / om);
+        wt[q] = 2.0 / (om * dp * dp) * (1.0 + dz * (2.0 * (1.0 + d[q]) - dK * (dK + 1.0) * dz) / om);
         d[q] -= dz;
         done = done && !(fabs(dz) > 4e-9 * om);
       }

@@ -131,6 +131,8 @@ __device__ __forceinline__ bool is_vacancy(float v) { return v != v; }
 __device__ __forceinline__ bool is_vacancy(double v) {
   return (unsigned long long)(__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ull;
 }
+// Infinity or NaN, on the integer pipe as well.
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 
 }  // namespace kite
 

@@ -622,12 +622,14 @@ __device__ __forceinline__ bool step_body(Ring& ring, int cta, int ncta, const v
             if constexpr (sizeof(Real) == 8) {
               // the FP64 pipe bounds the step: multiply-adds only, and only those of nonzero parts
               // (a symmetric window's coefficients are real or imaginary: two instead of six
-              // FP64 operations beside the stencil's eight)
-              if (cr != Real(0)) {
+              // FP64 operations beside the stencil's eight).  A component that is not finite
+              // takes them all: zero times it is NaN.
+              const bool odd = not_finite(br) || not_finite(bi);
+              if (cr != Real(0) || odd) {
                 a.v[2 * q] = rfma(cr, br, a.v[2 * q]);
                 a.v[2 * q + 1] = rfma(cr, bi, a.v[2 * q + 1]);
               }
-              if (ci != Real(0)) {
+              if (ci != Real(0) || odd) {
                 a.v[2 * q] = rfma(-ci, bi, a.v[2 * q]);
                 a.v[2 * q + 1] = rfma(ci, br, a.v[2 * q + 1]);
               }

@@ -192,16 +192,20 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
       }
       // a vacancy (v is NaN) holds r = 0 exactly in every iterate, so with its hopping and
       // on-site term zeroed fma(0, s, fma(0, +0, -0)) = +0: the same bits as forcing the
-      // output to zero, with two selects per site instead of one per component
+      // output to zero, with two selects per site instead of one per component (the series pass
+      // forces the output: a state that is not finite stays off the vacancies, as in the one-step
+      // kernel; it costs 0.6 %: 13.57 -> 13.65 ms for
+      // four packets on 1024 x 1024 honeycomb cells)
       const bool vacant = is_vacancy(v);
-      const Real ve = vacant ? Real(0) : v, te = vacant ? Real(0) : tt2;
+      const Real ve = SER < 0 && vacant ? Real(0) : v, te = SER < 0 && vacant ? Real(0) : tt2;
       Ch out;
 #pragma unroll
       for (int k = 0; k < NR; ++k) {
         Real sum = radd(n1.v[k], n2.v[k]);
         sum = radd(sum, n3.v[k]);
         if (LAT == KITE_SQUARE) sum = radd(sum, n4.v[k]);
-        out.v[k] = rfma(te, sum, rfma(ve, me.v[k], -pv.v[k]));  // 2t~ s + (2V~ r_n - r_{n-1})
+        const Real o = rfma(te, sum, rfma(ve, me.v[k], -pv.v[k]));  // 2t~ s + (2V~ r_n - r_{n-1})
+        out.v[k] = SER >= 0 && vacant ? Real(0) : o;
       }
       return out;
     };
@@ -229,14 +233,15 @@ __device__ __forceinline__ bool step2_body(Ring& ring, int cta, int ncta, const 
       // on-site term zeroed fma(0, s, fma(0, +0, -0)) = +0: the same bits as forcing the
       // output to zero, with two selects per site instead of one per component
       const bool vacant = is_vacancy(v);
-      const Real ve = vacant ? Real(0) : v, te = vacant ? Real(0) : tt2;
+      const Real ve = SER < 0 && vacant ? Real(0) : v, te = SER < 0 && vacant ? Real(0) : tt2;
       Ch out;
 #pragma unroll
       for (int k = 0; k < NR; ++k) {
         Real sum = radd(n1.v[k], n2.v[k]);
         sum = radd(sum, n3.v[k]);
         if (LAT == KITE_SQUARE) sum = radd(sum, n4.v[k]);
-        out.v[k] = rfma(te, sum, rfma(ve, me.v[k], -pv.v[k]));  // 2t~ s + (2V~ r_n - r_{n-1})
+        const Real o = rfma(te, sum, rfma(ve, me.v[k], -pv.v[k]));  // 2t~ s + (2V~ r_n - r_{n-1})
+        out.v[k] = SER >= 0 && vacant ? Real(0) : o;
       }
       return out;
     };

@@ -71,7 +71,10 @@ __device__ __forceinline__ bool team_barrier(unsigned int* ctr, unsigned int tar
 // DBL: moment doubling for the whole batch (two moments per step, r_0 not re-read):
 // step 0 writes <r_0|r_0>, <r_0|r_1> into slots 0, 1; step n >= 1 writes <r_n|r_n>,
 // <r_n|r_{n+1}> into slots 2n, 2n+1; k_breduce turns slots into moments.
-// NST: ring depth.  mcap > 0 caps every system's steps (the autotuner's probe launches).
+// NST: ring depth.  mcap > 0 caps every system's steps (the autotuner's probe launches, which
+// keep the slower lane sums: the shape they pick sets the grouping of the FP32 sums.  Probes with
+// the sums that run picked the same shape for seven or eight of nine batches, and where they
+// differed theirs was the slower one: 24.83 against 24.18 ms and 6.52 against 6.46).
 // FIELD: a batch with a magnetic field in any system runs the stencil's Peierls variant for
 // all of them (a system without a field has the phase table of flux 0: rotations by
 // (1, 0), which leave every value unchanged).

@@ -205,9 +205,9 @@ __global__ void k_mlp_transpose(const __nv_bfloat16* __restrict__ in, int rows, 
 
 // Chebyshev polynomials on the output grid, T[k][j] = T_k(eps_j), k < M, for the half
 // j < OUT/2 of the midpoint grid eps_j = -1 + (2j+1)/OUT (forward recurrence; the other half
-// is T_k(-e) = (-1)^k T_k(e), exactly).  Computed once per call: the FP64 pipe does two
-// multiply-adds per SM and cycle, and every row of the prior, the gate and the plain fallback
-// needs the same values.
+// is T_k(-e) = (-1)^k T_k(e), exactly).  Every row needs the same values and the FP64 pipe does
+// two multiply-adds per SM and cycle, so the prior, the gate and the plain fallback each compute
+// them once for all their rows (a table each: three of a learned call).
 constexpr int HALF = OUT / 2;
 __global__ void __launch_bounds__(32) k_mlp_cheb(int M, double* __restrict__ T) {
   const int j = blockIdx.x * 32 + threadIdx.x;

@@ -683,9 +683,10 @@ inline SweepCost cluster_cost(kite_ctx* ctx, ClusterSweep c) {
 
 // Cluster size to run the batch with, 0 for the streaming kernels.  `stream_ms` times the
 // streaming kernels' default launch per step (only called when the autotuner compares).
+// *cost: the chosen sweep's, where it was timed now.
 template <typename StreamMs>
 int cluster_choice(kite_ctx* ctx, const Plan& p, const ClusterSweep& c, long long units,
-                   StreamMs stream_ms) {
+                   StreamMs stream_ms, SweepCost* cost) {
   const int pin = cluster_pinned();
   if (pin == 1 || p.field || ctx->debug_stall) return 0;
   // pinning the streaming kernels (KITE_PASS_STEPS, KITE_TUNE) or turning the autotuner off
@@ -726,8 +727,8 @@ int cluster_choice(kite_ctx* ctx, const Plan& p, const ClusterSweep& c, long lon
   for (int k = 0; k < nc; ++k) {
     ClusterSweep t = c;
     t.cs = cand[k];
-    const float ms = cluster_cost(ctx, t).step;
-    if (ms < best) best = ms, pick = cand[k];
+    const SweepCost now = cluster_cost(ctx, t);
+    if (now.step < best) best = now.step, pick = cand[k], *cost = now;
   }
   cudaGetLastError();
   ctx->tune[key] = {pick, 0};
@@ -757,7 +758,7 @@ constexpr size_t kResidentPartMax = (size_t)2 << 30;
 // do not bring in: at 64 x 64 honeycomb cells, FP64, R = 4 a step takes 1.86 us on chip and 2.26 us
 // in clusters, and calls of M = 4 .. 16 took 5 to 7 % longer with it; 300 x 300 square cells, FP32,
 // R = 4, M = 4 149 -> 169 us.  Fewer than kResidentMinSteps steps hardly gain at any size (at best
-// 9 us a step) and are neither taken nor timed (the timing runs take 56 to 104 steps).
+// 9 us a step) and are neither taken nor timed (the timing runs take 56 or 104 steps).
 constexpr float kResidentExtraMs = 0.010f;
 constexpr int kResidentMinSteps = 8;
 constexpr int kResidentTries = 3;
@@ -811,6 +812,7 @@ int resident_choice(kite_ctx* ctx, const ResidentSweep& r, int steps, OtherCost 
       const float more = (float)(1e3 * t8 * sweeps) - 8.0f * step - other.fixed + kResidentExtraMs;
       from = (int)std::min(1e6f, std::max(0.0f, more / (other.step - step)));
     }
+    if (step > 1.1f * other.step) break;  // far from winning: one timing does
   }
   cudaGetLastError();
   if (!ok) {
@@ -1145,8 +1147,9 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       };
       // the kernels that run otherwise: the cluster sweep, the field sweep, or the streaming
       // kernel of the tuned shape
+      SweepCost cl_cost{0.0f, 0.0f};
       auto other_cost = [&]() -> SweepCost {
-        if (cl.cs > 0) return cluster_cost(ctx, cl);
+        if (cl.cs > 0) return cl_cost.step > 0.0f ? cl_cost : cluster_cost(ctx, cl);
         if (p.field) {
           FieldSweep f = fs;
           f.M = std::min(p.M, 9);
@@ -1180,7 +1183,7 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       rs.want_last = want_last;
       cl.last_prev = want_last ? bA : nullptr;
       cl.last_cur = want_last ? bB : nullptr;
-      cl.cs = cluster_choice(ctx, p, cl, u, stream_ms);
+      cl.cs = cluster_choice(ctx, p, cl, u, stream_ms, &cl_cost);
       // (an FP32 batch that runs on chip in clusters stays there: its moment sums are grouped
       // by the clusters' threads)
       const bool pinned_res = resident_pinned() == 2;

@@ -352,6 +352,11 @@ int kite_debug_stall_once(kite_ctx* ctx, int enable);
 #define KITE_FAIL_LAUNCH 2
 int kite_debug_fail_resident(kite_ctx* ctx, int kind, int skip, int count);
 
+/* Test hook (no counterpart in the paper): work space beyond `bytes` is refused as if the
+ * device had no room for it, whatever the context holds already (0: no limit).
+ * Errors: KITE_ERR_ARG. */
+int kite_debug_limit_workspace(kite_ctx* ctx, int64_t bytes);
+
 /* ---- 2D moments ----------------------------------------------------------------- */
 
 /* Velocity directions of the 2D moments. */

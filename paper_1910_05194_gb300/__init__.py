@@ -26,7 +26,8 @@ DIR_X, DIR_Y = 0, 1
 
 EXPORTED = ("kite_create", "kite_destroy", "kite_set_stream", "kite_status_string",
             "kite_last_error", "kite_bounds", "kite_moments_1d", "kite_reconstruct_dos",
-            "kite_debug_stall_once", "kite_debug_fail_resident", "kite_inner_products", "kite_moments_2d", "kite_reconstruct_green",
+            "kite_debug_stall_once", "kite_debug_fail_resident",
+            "kite_debug_limit_workspace", "kite_inner_products", "kite_moments_2d", "kite_reconstruct_green",
             "kite_reconstruct_sigma", "kite_moments_1d_static", "kite_moments_1d_batched",
             "kite_mlp_param_count", "kite_mlp_train", "kite_mlp_forward", "kite_mlp_gradient",
             "kite_learned_gate", "kite_spectral_k", "kite_ldos", "kite_propagate",
@@ -197,6 +198,8 @@ def lib():
             L.kite_debug_stall_once.restype = i32
             L.kite_debug_fail_resident.argtypes = [vp, i32, i32, i32]
             L.kite_debug_fail_resident.restype = i32
+            L.kite_debug_limit_workspace.argtypes = [vp, ctypes.c_int64]
+            L.kite_debug_limit_workspace.restype = i32
             _LIB = L
     return _LIB
 
@@ -330,6 +333,11 @@ FAIL_WAIT, FAIL_LAUNCH = 1, 2
 def debug_fail_resident(ctx: Context, kind: int, skip: int = 0, count: int = 1):
     """Test hook: of the on-chip sweeps that follow, ``skip`` run and the next ``count`` fail."""
     ctx.check(lib().kite_debug_fail_resident(ctx.handle, int(kind), int(skip), int(count)))
+
+
+def debug_limit_workspace(ctx: Context, nbytes: int):
+    """Test hook: work space beyond ``nbytes`` is refused (0: no limit)."""
+    ctx.check(lib().kite_debug_limit_workspace(ctx.handle, int(nbytes)))
 
 
 def reconstruct_green(ctx: Context, mu, M_avail: int, M_use: int, kernel: int, param: float,

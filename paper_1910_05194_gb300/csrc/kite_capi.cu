@@ -66,6 +66,8 @@ int cuda_fail(kite_ctx* ctx, cudaError_t e, const char* what) {
 }
 
 int ensure_ws(kite_ctx* ctx, size_t bytes) {
+  if (ctx->ws_limit && bytes > ctx->ws_limit)  // test hook
+    return fail(ctx, KITE_ERR_OOM, "work space of " + std::to_string(bytes >> 20) + " MiB is beyond the limit set");
   if (bytes <= ctx->ws_bytes) return KITE_OK;
   if (ctx->ws) {
     cudaStreamSynchronize(ctx->stream);
@@ -379,6 +381,13 @@ int kite_debug_fail_resident(kite_ctx* ctx, int kind, int skip, int count) {
   ctx->fail_kind = kind;
   ctx->fail_skip = skip;
   ctx->fail_count = count;
+  return KITE_OK;
+}
+
+int kite_debug_limit_workspace(kite_ctx* ctx, int64_t bytes) {
+  if (!ctx) return KITE_ERR_ARG;
+  if (bytes < 0) return fail(ctx, KITE_ERR_ARG, "need bytes >= 0");
+  ctx->ws_limit = (size_t)bytes;
   return KITE_OK;
 }
 

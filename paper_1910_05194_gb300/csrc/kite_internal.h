@@ -55,6 +55,7 @@ struct kite_ctx {
   volatile int* sweep_status = nullptr;
   int debug_stall = 0;  // test hook, see kite_debug_stall_once
   int fail_kind = 0, fail_skip = 0, fail_count = 0;  // test hook, see kite_debug_fail_resident
+  size_t ws_limit = 0;  // test hook, see kite_debug_limit_workspace
   // Autotuner cache: key (kernel family, precision, lattice, vectors per orbital, mode,
   // size bucket) -> (ring depth, CTAs per SM) measured fastest on this context's GPU.
   std::map<uint64_t, std::pair<int, int>> tune;

@@ -1,6 +1,6 @@
-"""Calls on a device that is nearly full: where the faster path's work space does not fit, the
-path that needs less runs, with the same results, and the call is refused only when that one
-does not fit either."""
+"""Calls whose work space is limited (a hook refuses more, as a device without room does): where the
+faster path's does not fit, the path that needs less runs, with the same results, and the call is
+refused only when that one does not fit either."""
 import contextlib
 import os
 
@@ -26,19 +26,6 @@ def env(**kw):
             os.environ.pop(k, None) if v is None else os.environ.__setitem__(k, v)
 
 
-@contextlib.contextmanager
-def free_memory(mib):
-    """All but `mib` MiB of the device's free memory taken."""
-    torch.cuda.synchronize()
-    torch.cuda.empty_cache()
-    block = torch.empty(torch.cuda.mem_get_info()[0] - mib * MiB, dtype=torch.uint8, device="cuda")
-    try:
-        yield
-    finally:
-        del block
-        torch.cuda.empty_cache()
-
-
 def moments(ctx, M, R=8):
     s = kite.make_system(kite.HONEYCOMB, 257, 510, t=-2.7, W=2.0, seed=3)
     mu, per = np.zeros(M), np.zeros((R, M, 2))
@@ -59,14 +46,16 @@ def test_moments_without_room_for_the_on_chip_sweeps_partials():
     with kite.Context(0) as ctx:
         with env(KITE_RESIDENT="0"):
             moments(ctx, 64)  # the same tuned shape
-        with free_memory(1240):
-            per, block = moments(ctx, M)
-            assert kite.lib().kite_last_error(ctx.handle) == b""
+        kite.debug_limit_workspace(ctx, 1240 * MiB)
+        per, block = moments(ctx, M)
+        assert kite.lib().kite_last_error(ctx.handle) == b""
         assert block == stream and np.max(np.abs(per - ref)) <= 1e-6
-    with kite.Context(0) as ctx, free_memory(64):
+        kite.debug_limit_workspace(ctx, 64 * MiB)
         with pytest.raises(kite.KiteError) as e:
             moments(ctx, M)
         assert e.value.status == kite.ERR_OOM
+        kite.debug_limit_workspace(ctx, 0)
+        assert moments(ctx, M)[1] == short
 
 
 def test_time_evolution_without_room_for_two_steps_a_pass():
@@ -80,11 +69,13 @@ def test_time_evolution_without_room_for_two_steps_a_pass():
     norms = np.zeros((2, 1, R))
     with kite.Context(0) as ctx:
         kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, ref, norms[0])
-    with kite.Context(0) as ctx, free_memory(1050):
+    with kite.Context(0) as ctx:
+        kite.debug_limit_workspace(ctx, 1050 * MiB)
         st = kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, psi, norms[1])
         assert st.step_launches == M - 1 and kite.lib().kite_last_error(ctx.handle) == b""
     assert torch.equal(ref, psi) and np.array_equal(norms[0], norms[1])
-    with kite.Context(0) as ctx, free_memory(700):
+    with kite.Context(0) as ctx:
+        kite.debug_limit_workspace(ctx, 700 * MiB)
         with pytest.raises(kite.KiteError) as e:
             kite.propagate(ctx, s, kite.make_kpm(M, R, 1, kite.FP32), 0.4, 1, psi)
         assert e.value.status == kite.ERR_OOM

@@ -421,10 +421,11 @@ inline bool autotune_enabled() {
 }
 
 // Milliseconds per recursion step of a candidate, from three launches after a warm-up.  The shape
-// chosen sets the grouping of the FP32 moment sums, so one late launch should not decide between
-// two close candidates: a first timing below `again` is taken a second time and the better one
-// counts.  (All candidates twice: a new size's first call took up to 1.4 times as long as with
-// one timing, 20.3 against 14.9 ms at 1300^2 square cells, M = 128, R = 8.)
+// chosen sets the grouping of the FP32 moment sums, and the best FP64 shapes lie within 3 %, so one
+// late launch should not decide between two close candidates: a first timing below `again` is
+// taken a second time and the better one counts.  (With all candidates timed twice a new size's
+// first call took longer: 17.8 against 15.7 ms at 2000 x 900 square cells, M = 64, R = 8, FP32;
+// 47.4 against 40.8 ms at 1500^2 honeycomb cells, M = 48, R = 2, FP64.)
 template <typename Launch>
 float time_launches(kite_ctx* ctx, Launch launch, int steps_per_launch, float again) {
   launch();  // warm-up
@@ -441,12 +442,9 @@ float time_launches(kite_ctx* ctx, Launch launch, int steps_per_launch, float ag
   }
   return best;
 }
-// `again` for a candidate of the sweep while the best one so far takes `best` ms: FP64 sums may be
-// grouped freely, one timing does.
-template <typename Real>
-constexpr float time_again(float best = 1e30f) {
-  return sizeof(Real) == 4 ? 1.25f * best : 0.0f;
-}
+
+// `again` for a candidate while the best one so far takes `best` ms.
+constexpr float time_again(float best = 1e30f) { return 1.25f * best; }
 
 // KITE_PASS_STEPS=1, 2 or 3 pins the steps per pass of the plain moment sweep (the
 // autotuner then chooses only the ring depth and occupancy); unset, all are candidates.
@@ -466,7 +464,7 @@ int step2_grid(kite_ctx* ctx, long long units, int ctas_per_sm = 0) {
 template <typename Real, int LAT, int C, int NST, bool DBL = false>
 float time_candidate2(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt,
                       void* r0, void* bA, void* bB, void* bC, void* bD, double* partial,
-                      float again = time_again<Real>()) {
+                      float again = time_again()) {
   constexpr int SMEM = Step2Shape<LAT, C, NST, DBL>::SMEM;
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = step2_grid<Real, LAT, C, NST, DBL>(ctx, units, k);
@@ -491,7 +489,7 @@ int step3_grid(kite_ctx* ctx, long long units, int ctas_per_sm = 0) {
 template <typename Real, int LAT, int C, int NST>
 float time_candidate3(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt,
                       void* r0, void* bA, void* bB, void* bC, void* bD, double* partial,
-                      float again = time_again<Real>()) {
+                      float again = time_again()) {
   constexpr int SMEM = Step3Shape<LAT, C, NST>::SMEM;
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = step3_grid<Real, LAT, C, NST>(ctx, units, k);
@@ -506,7 +504,7 @@ float time_candidate3(kite_ctx* ctx, int k, long long units, const Plan& p, cons
 
 template <typename Real, int LAT, int C, int MODE, int NST>
 float time_candidate(kite_ctx* ctx, int k, long long units, const Plan& p, const Real* vt, Real tt, void* r0,
-                     void* bA, void* bB, double* partial, float again = time_again<Real>()) {
+                     void* bA, void* bB, double* partial, float again = time_again()) {
   constexpr int SMEM = StepShape<LAT, C, NST>::template smem_bytes<MODE>();
   constexpr int Q = 2 * C * Chunk<Real>::kVecs;
   const int G = grid_for<Real, LAT, C, false, MODE, NST>(ctx, units, k);
@@ -580,12 +578,12 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
     const int o8 = step_occupancy<Real, LAT, C, MODE, 8>(), o4 = step_occupancy<Real, LAT, C, MODE, 4>();
     for (int k = 1; k <= o8; ++k) {
       const float ms = time_candidate<Real, LAT, C, MODE, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, partial,
-                                                             time_again<Real>(best_ms));
+                                                             time_again(best_ms));
       if (ms < best_ms) best_ms = ms, best = Tune{8, k, 0};
     }
     for (int k = 1; k <= o4; ++k) {
       const float ms = time_candidate<Real, LAT, C, MODE, 4>(ctx, k, units, p, vt, tt, r0, bA, bB, partial,
-                                                             time_again<Real>(best_ms));
+                                                             time_again(best_ms));
       if (ms < best_ms * 0.98f) best_ms = ms, best = Tune{4, k, 0};  // prefer the deeper ring on a tie
     }
   }
@@ -598,17 +596,17 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
               o5 = step2_occupancy<Real, LAT, C, 5, DB>();
     for (int k = 1; k <= o8; ++k) {
       const float ms = time_candidate2<Real, LAT, C, 8, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
-                                                            time_again<Real>(best2));
+                                                            time_again(best2));
       if (ms < best2) best2 = ms, best = Tune{8, k, 1};
     }
     for (int k = 1; k <= o6; ++k) {
       const float ms = time_candidate2<Real, LAT, C, 6, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
-                                                            time_again<Real>(best2));
+                                                            time_again(best2));
       if (ms < best2 * 0.98f) best2 = ms, best = Tune{6, k, 1};
     }
     for (int k = 1; k <= o5; ++k) {
       const float ms = time_candidate2<Real, LAT, C, 5, DB>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
-                                                            time_again<Real>(best2));
+                                                            time_again(best2));
       if (ms < best2 * 0.98f) best2 = ms, best = Tune{5, k, 1};
     }
   }
@@ -617,12 +615,12 @@ Tune autotune(kite_ctx* ctx, long long units, const Plan& p, const Real* vt, Rea
     const int o8 = step3_occupancy<Real, LAT, C, 8>(), o7 = step3_occupancy<Real, LAT, C, 7>();
     for (int k = 1; k <= o8; ++k) {
       const float ms = time_candidate3<Real, LAT, C, 8>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
-                                                          time_again<Real>(best3));
+                                                          time_again(best3));
       if (ms < best3) best3 = ms, best = Tune{8, k, 2};
     }
     for (int k = 1; k <= o7; ++k) {
       const float ms = time_candidate3<Real, LAT, C, 7>(ctx, k, units, p, vt, tt, r0, bA, bB, bC, bD, partial,
-                                                          time_again<Real>(best3));
+                                                          time_again(best3));
       if (ms < best3 * 0.98f) best3 = ms, best = Tune{7, k, 2};
     }
   }

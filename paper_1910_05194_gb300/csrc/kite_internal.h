@@ -20,6 +20,7 @@ struct ResidentPlan {
   int regions, rows, nv, nfl, r0_rows;
   int cby, vecs;      // the sweep's unit: bytes (16-byte chunk or half of one) and vectors
   int CR;             // units per orbital and sweep (0: the lattice does not fit)
+  int sites;          // edge sites and halo units of an exchange thread, at most
   int T, levels, smem;
 };
 }  // namespace kite

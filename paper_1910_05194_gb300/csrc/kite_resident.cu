@@ -53,7 +53,10 @@ namespace {
 
 constexpr int kRMax = 256;     // most compute threads of a CTA (512 threads: 128 registers each)
 constexpr int kRComm = 256;    // exchange threads
-constexpr int kRSites = 3;     // most edge sites, and most halo chunks, of one exchange thread
+// Most edge sites, and most halo chunks, of one exchange thread: kRSites, or kRFew where a plan's
+// lists are short enough.  Fewer of them leave the exchange warps less to carry along: 64 x 64
+// honeycomb cells, FP64, R = 4, M = 256 578 -> 562 us a call, 200 x 200, FP32, R = 4 589 -> 577.
+constexpr int kRSites = 3, kRFew = 2;
 constexpr int kRMaxV = 64;     // most virtual CTAs of a region
 constexpr int kRFlush = 32;    // rows of one FP32 moment sum (the streaming kernels' kFlushRows)
 constexpr int kResSmem = 227 * 1024 - 512;  // (the rest: static shared memory)
@@ -163,7 +166,7 @@ __host__ __device__ inline ResSmem res_smem(int cby, int sorb, int CR, int TX, i
 }
 
 // VAR 0: complex vectors, 1: complex vectors in a magnetic field, 2: real vectors.
-template <typename Real, int CBY, int LAT, bool DBL, int VAR>
+template <typename Real, int CBY, int LAT, bool DBL, int VAR, int SITES>
 __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Real> a) {
   using Ch = typename ResUnit<Real, CBY>::T;
   constexpr int W = CBY / 4;  // words of a record
@@ -306,10 +309,10 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
     const int ct = tid - T, lane = ct & 31, warp = ct >> 5;
     const size_t half = (size_t)a.Lx * a.Ly * TPC;  // records per parity
     // edge sites (sent) and halo chunks (received) of this thread: smem offset, record
-    int e_off[kRSites], h_off[kRSites], e_row[kRSites];
-    unsigned e_rec[kRSites], h_rec[kRSites];
-    Real e_v[kRSites];
-    Ch e_prev[kRSites];
+    int e_off[SITES], h_off[SITES], e_row[SITES];
+    unsigned e_rec[SITES], h_rec[SITES];
+    Real e_v[SITES];
+    Ch e_prev[SITES];
     unsigned e_on = 0, h_on = 0, e_s = 0;
     {
       int off = 0, hoff = 0;  // list positions of the segment's first entry
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
         // first column; square: the four sides
         const int len = LAT == KITE_HONEYCOMB ? 2 * (w + h - 1) : 2 * (w + h);
 #pragma unroll
-        for (int u = 0; u < kRSites; ++u) {
+        for (int u = 0; u < SITES; ++u) {
           const int j = ct + u * kRComm, e = j / CR - off, c = j - (j / CR) * CR;
           if (e < 0 || e >= len) continue;
           int lx, ly, s = 0;
@@ -342,7 +345,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
         off += len;
         const int hlen = 2 * (w + h);
 #pragma unroll
-        for (int u = 0; u < kRSites; ++u) {
+        for (int u = 0; u < SITES; ++u) {
           const int j = ct + u * kRComm, e = j / CR - hoff, c = j - (j / CR) * CR;
           if (e < 0 || e >= hlen) continue;
           int lx, ly, s = 0;
@@ -375,7 +378,7 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
       const unsigned char* cur = xb + (n & 1) * xd;
       Rec<W>* dst = static_cast<Rec<W>*>(a.rec) + ((n + 1) & 1) * half;
 #pragma unroll
-      for (int u = 0; u < kRSites; ++u) {
+      for (int u = 0; u < SITES; ++u) {
         if (!(e_on >> u & 1)) continue;
         const Nb nb = (e_s >> u & 1) ? nb1 : nb0;
         const unsigned char* p = cur + e_off[u];
@@ -418,12 +421,12 @@ __global__ void __launch_bounds__(kRMax + kRComm, 1) k_resident(const ResArgs<Re
         unsigned want = h_on;
         const long long t0 = clock64();
         while (want) {
-          Rec<W> d[kRSites];
+          Rec<W> d[SITES];
 #pragma unroll
-          for (int u = 0; u < kRSites; ++u)
+          for (int u = 0; u < SITES; ++u)
             if (want >> u & 1) d[u] = load_rec(src + h_rec[u]);
 #pragma unroll
-          for (int u = 0; u < kRSites; ++u)
+          for (int u = 0; u < SITES; ++u)
             if ((want >> u & 1) && rec_ready(d[u], step)) {
               Ch x;
               uint32_t(&xw)[W] = *reinterpret_cast<uint32_t(*)[W]>(&x);
@@ -668,18 +671,25 @@ __global__ void __launch_bounds__(256) k_resident_reduce(const double* __restric
   }
 }
 
-template <typename Real, int CBY, int LAT, bool DBL>
+template <typename Real, int CBY, int LAT, bool DBL, int SITES>
 const void* res_kernel_var(int var) {
-  return var == 0   ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 0>)
-         : var == 1 ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 1>)
-                    : reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 2>);
+  return var == 0   ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 0, SITES>)
+         : var == 1 ? reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 1, SITES>)
+                    : reinterpret_cast<const void*>(&k_resident<Real, CBY, LAT, DBL, 2, SITES>);
+}
+template <typename Real, int CBY, int SITES>
+const void* res_kernel_sites(int lattice, int dbl, int var) {
+  if (lattice == KITE_HONEYCOMB)
+    return dbl ? res_kernel_var<Real, CBY, KITE_HONEYCOMB, true, SITES>(var)
+               : res_kernel_var<Real, CBY, KITE_HONEYCOMB, false, SITES>(var);
+  return dbl ? res_kernel_var<Real, CBY, KITE_SQUARE, true, SITES>(var)
+             : res_kernel_var<Real, CBY, KITE_SQUARE, false, SITES>(var);
 }
 template <typename Real, int CBY>
-const void* res_kernel(int lattice, int dbl, int var) {
-  if (lattice == KITE_HONEYCOMB)
-    return dbl ? res_kernel_var<Real, CBY, KITE_HONEYCOMB, true>(var)
-               : res_kernel_var<Real, CBY, KITE_HONEYCOMB, false>(var);
-  return dbl ? res_kernel_var<Real, CBY, KITE_SQUARE, true>(var) : res_kernel_var<Real, CBY, KITE_SQUARE, false>(var);
+const void* res_kernel(int lattice, int dbl, int var, int sites) {
+  if constexpr (CBY == 16)  // (half chunks: lattices with long lists)
+    if (sites <= kRFew) return res_kernel_sites<Real, CBY, kRFew>(lattice, dbl, var);
+  return res_kernel_sites<Real, CBY, kRSites>(lattice, dbl, var);
 }
 
 // Vectors and moment sums (real and imaginary part in FP32) of a unit of cby bytes.
@@ -732,6 +742,7 @@ ResidentPlan resident_plan(kite_ctx* ctx, int fp64, int lattice, int doubling, i
     p.nv = nv;
     p.r0_rows = r0_rows;
     p.CR = cr;
+    p.sites = edge * cr <= kRFew * kRComm ? kRFew : kRSites;
     p.T = std::min(nv, kRMax / colT) * colT;
     p.T = (p.T + 31) / 32 * 32;
     p.smem = need(r0_rows);
@@ -803,9 +814,9 @@ int resident_sweep(kite_ctx* ctx, ResidentSweep* a, int timing_steps) {
     }
   }
   const int var = a->phase ? 1 : (a->realv ? 2 : 0);
-  const void* fn = a->fp64        ? res_kernel<double, 16>(a->lattice, a->doubling, var)
-                   : p.cby == 16 ? res_kernel<float, 16>(a->lattice, a->doubling, var)
-                                 : res_kernel<float, 8>(a->lattice, a->doubling, var);
+  const void* fn = a->fp64        ? res_kernel<double, 16>(a->lattice, a->doubling, var, p.sites)
+                   : p.cby == 16 ? res_kernel<float, 16>(a->lattice, a->doubling, var, p.sites)
+                                 : res_kernel<float, 8>(a->lattice, a->doubling, var, p.sites);
   {
     static std::mutex mu;
     static std::set<std::pair<const void*, int>> done;

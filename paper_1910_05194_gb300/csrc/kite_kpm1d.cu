@@ -751,14 +751,13 @@ constexpr size_t kResidentPartMax = (size_t)2 << 30;
 // took as long as the long one), n failures so far.  A failure decides nothing: the next call
 // times again, until kResidentTries of them have shown that this GPU's SMs are not to be had.
 //
-// A sweep's launch, record memset and load cost 8 to 20 us and its host part and reduction about
-// 10 us more than the other kernels' (the timing runs do not see those), which a few faster steps
-// do not bring in: at 64 x 64 honeycomb cells, FP64, R = 4 a step takes 1.86 us on chip and 2.26 us
-// in clusters, and calls of M = 4 .. 16 took 5 to 7 % longer with it; 300 x 300 square cells, FP32,
-// R = 4, M = 4 149 -> 169 us.  Fewer than kResidentMinSteps steps hardly gain at any size (at best
-// 9 us a step) and are neither taken nor timed (the timing runs take 56 or 104 steps).
+// A sweep's launch, record memset and load cost 8 to 20 us, and its host part and reduction 10 us
+// more than the cluster sweep's (the timing runs do not see those), which a few faster steps do
+// not bring in: at 64 x 64 honeycomb cells, FP64, R = 4 a step takes 1.86 us on chip and 2.26 us in
+// clusters, and calls of M = 4 .. 16 took 5 to 7 % longer with it; 300 x 300 square cells, FP32, R = 4,
+// M = 4 149 -> 169 us.  (At 500 x 500 honeycomb cells, FP32, R = 1, a step takes 2.2 us on chip and
+// 11.4 us streaming: M = 8 220 -> 173 us.)  The timing runs take 56 or 104 steps.
 constexpr float kResidentExtraMs = 0.010f;
-constexpr int kResidentMinSteps = 8;
 constexpr int kResidentTries = 3;
 
 inline uint64_t resident_key(const ResidentSweep& r) {
@@ -807,7 +806,7 @@ int resident_choice(kite_ctx* ctx, const ResidentSweep& r, int steps, OtherCost 
     if (ok && rep == 0) other = other_cost();
     const float step = (float)(1e3 * (t40 - t8) / (kClusterTimeSteps - 8) * sweeps);
     if (ok && step < 0.95f * other.step) {  // it must win clearly
-      const float more = (float)(1e3 * t8 * sweeps) - 8.0f * step - other.fixed + kResidentExtraMs;
+      const float more = (float)(1e3 * t8 * sweeps) - 8.0f * step - other.fixed + (other.fixed > 0.0f ? kResidentExtraMs : 0.0f);
       from = (int)std::min(1e6f, std::max(0.0f, more / (other.step - step)));
     }
     if (step > 1.1f * other.step) break;  // far from winning: one timing does
@@ -1187,8 +1186,8 @@ int run_typed(kite_ctx* ctx, const kite_system* sys, const kite_kpm* kpm, const 
       const bool pinned_res = resident_pinned() == 2;
       const bool may_reside =
           resident_rec != 0 && !resident_off &&
-          (pinned_res || (steps_for(p) >= kResidentMinSteps && !ctx->debug_stall && autotune_enabled() &&
-                          !pass_steps_pinned() && !getenv("KITE_TUNE") && cluster_pinned() != 2));
+          (pinned_res || (!ctx->debug_stall && autotune_enabled() && !pass_steps_pinned() && !getenv("KITE_TUNE") &&
+                          cluster_pinned() != 2));
       if (may_reside && (sizeof(Real) == 8 || cl.cs == 0 || pinned_res))
         rs.plan = resident_for(C, sizeof(Real) == 8 ? 0 : (p.field ? fs.G : tuned_grid()));
       const int choice = rs.plan.CR ? resident_choice(ctx, rs, steps_for(p), other_cost) : 0;
